@@ -646,6 +646,7 @@ struct StepQueue {
     int warps;               // warps per block of Ln
     const InstanceDev *one;  // single instance: its parameters by value; else NULL
     int wx;                  // some instance uses an interpolated wall rule
+    bool to_and_fro;         // every other step takes the tiles from the last to the first
     const TmaLaunch *tma;    // non-reducing steps on the TMA brick kernel; else NULL
     int collision, layout;
     unsigned *status;
@@ -670,17 +671,18 @@ static cudaError_t queue_steps(const StepQueue &q, cudaStream_t s, long long n, 
             if (e != cudaSuccess) return e;
         }
         const int kind = q.layout == LBM_LAYOUT_AB ? KIND_AB : (aa == 0 ? KIND_AA_PULL : KIND_AA_LOCAL);
+        const int order = q.to_and_fro && ((q.layout == LBM_LAYOUT_AB ? flip : aa) & 1) ? kStepBackwards : 0;
         cudaError_t e;
         if (!red && q.tma) {  // the reducing step always runs the tile kernel
             TmaLaunch T = *q.tma;
             T.stream = s;
             e = q.ops->step_tma(q.collision, q.wx, T, *q.one, flip);
         } else if (red || q.wx) {  // the reducing and interpolated-wall steps: kStepWarps tiles
-            e = q.ops->step(q.collision, kind, L, flip, red ? 1 : 0, q.status, q.one, q.wx, kStepWarps);
+            e = q.ops->step(q.collision, kind, L, flip | order, red ? 1 : 0, q.status, q.one, q.wx, kStepWarps);
         } else {
             Launch Ls = q.Ln[kind == KIND_AA_LOCAL ? 1 : 0];
             Ls.stream = s;
-            e = q.ops->step(q.collision, kind, Ls, flip, 0, q.status, q.one, 0, q.warps);
+            e = q.ops->step(q.collision, kind, Ls, flip | order, 0, q.status, q.one, 0, q.warps);
         }
         if (e != cudaSuccess) return e;
         ++launches;
@@ -703,6 +705,21 @@ Launch Batch::shaped_launch(const StepShape &sh, int kind) const
     (void)kind;
     const int nt = nwtiles_[w];
     return Launch{d_table_, d_wtiles_[w], nt, sh.warps, std::max(1, nt), sh.warps * 32, stream_, &maps_[w]};
+}
+
+// Every other step takes its tiles from the last to the first, so that it begins with the
+// cells the previous step ended with, whose populations are still in L2.  A state larger
+// than L2, swept in one direction, finds none of its lines there (each is evicted just before
+// its turn); swept to and fro it finds about an L2's worth.  Per step, one direction -> to and
+// fro: FP32 AA 112^3 19.7 -> 18.4 us, 128^3 36.1 -> 29.0, 160^3 68.3 -> 60.2, 256^3 270.7 ->
+// 259.3, 384^3 869 -> 860; FP32 A-B 96^3 19.9 -> 16.2, 128^3 44.5 -> 42.7; BF16 AA 160^3
+// 56.8 -> 52.1.  Below 32 MiB of fluid populations (FP32 AA 80^3 and 96^3, BF16 AA 112^3) both
+// orders take the same time, and a cell of one tile per multiprocessor is 3 % slower to and
+// fro (FP64 20^3 17.1 -> 17.7 us), so those keep one direction.
+bool Batch::to_and_fro() const
+{
+    const long long bytes = fluid_cells() * Q * (long long)storage_bytes(storage_);
+    return bytes * (layout_ == LBM_LAYOUT_AB ? 2 : 1) >= (32ll << 20);
 }
 
 // The graph of m steps (+ the reduction when red) from (flip_, aa_phase_) in shape sh,
@@ -730,6 +747,7 @@ lbm_status Batch::graph_for(long long m, bool red, const StepShape &sh, int wx, 
                 sh.warps,
                 size() == 1 ? &h_table_[0] : nullptr,
                 wx,
+                to_and_fro(),
                 tma_ ? &tma_launch_ : nullptr,
                 collision_,
                 layout_,

@@ -112,6 +112,7 @@ private:
         long long used;
     };
     static constexpr size_t kGraphCache = 16;  // instantiated step graphs kept per batch
+    bool to_and_fro() const;            // the order of the step tiles alternates
     Launch shaped_launch(const StepShape &sh, int kind) const;
     lbm_status graph_for(long long m, bool red, const StepShape &sh, int wx, cudaGraphExec_t *out);
     void lookup_shape();                // the cached shape of this batch, or tuning pending

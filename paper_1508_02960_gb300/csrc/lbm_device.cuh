@@ -344,6 +344,8 @@ struct TileDev {
 };
 
 enum { KIND_AB = 0, KIND_AA_PULL = 1, KIND_AA_LOCAL = 2 };
+// Bit of the step kernel's flip argument: this step takes its tiles from the last to the first.
+constexpr int kStepBackwards = 2;
 
 // The tiles of a batched step launch, as a kernel parameter (constant bank) for batches of up
 // to kBatchMapMax instances: instance i owns tiles tile_start[i] .. tile_start[i + 1] - 1 of

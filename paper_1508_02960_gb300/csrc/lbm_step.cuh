@@ -731,11 +731,12 @@ __device__ __forceinline__ const InstanceDev &instance_of(const InstanceDev *tab
 // each), one item per warp.  Each cell's arithmetic does not depend on WARPS, so every block
 // shape gives the same state bit for bit; the reducing step always runs kStepWarps-warp
 // tiles.  A single instance's parameters travel by value (constant bank); a batch's come
-// from the device table.  flip selects the A-B buffer pair (src = f[phase ^ flip]).  The RED
-// variant (the step that ends a chunk) also makes every tile write its FP64 partial sums
-// (the kRedSlots slots: drho, u_x, u_y, u_z and the momentum exchanged with the solid) and
-// flags diverged cells in status[instance]; the other steps carry none of that code.  The WX
-// variant (A-B only) also runs the interpolated wall rules LIBB, QIBB, IEBB and MR.
+// from the device table.  flip selects the A-B buffer pair (src = f[phase ^ flip], bit 0)
+// and the order of the tiles (bit kStepBackwards).  The RED variant (the step that ends a
+// chunk) also makes every tile write its FP64 partial sums (the kRedSlots slots: drho, u_x,
+// u_y, u_z and the momentum exchanged with the solid) and flags diverged cells in
+// status[instance]; the other steps carry none of that code.  The WX variant (A-B only)
+// also runs the interpolated wall rules LIBB, QIBB, IEBB and MR.
 template <int COLL, int STORE, int KIND, bool BATCH, bool RED, bool WX, int WARPS = kStepWarps>
 __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, WX, WARPS, KIND, BATCH>())
     step_kernel(const InstanceDev *__restrict__ table, const __grid_constant__ InstanceDev one,
@@ -748,8 +749,8 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
     using R = typename S::R;
     allow_next_step();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t = blockIdx.x;
-    if (t >= ntiles) return;
+    if ((int)blockIdx.x >= ntiles) return;
+    const int t = (flip & kStepBackwards) ? ntiles - 1 - (int)blockIdx.x : (int)blockIdx.x;
     // a single instance's tiles are consecutive: tile t holds work items WARPS t ... (its
     // table entry holds the same, so that no load precedes the work list's)
     TileDev tile;
@@ -776,7 +777,7 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
     const T *fs;  // state read this step
     T *fd;        // state written this step
     if constexpr (KIND == KIND_AB) {
-        const int cur = I.phase ^ flip;
+        const int cur = I.phase ^ (flip & 1);
         fs = reinterpret_cast<const T *>(cur ? I.f1 : I.f0);
         fd = reinterpret_cast<T *>(cur ? I.f0 : I.f1);
     } else {
