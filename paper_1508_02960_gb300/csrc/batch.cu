@@ -312,6 +312,52 @@ long long Batch::fluid_cells() const
     return s;
 }
 
+// The constants of CollPar (lbm_device.cuh): single precision ...
+static void collision_constants(CollPar<float> &c, double wp, double wm, double rho0, double delta_rho, int s,
+                                const double *rates)
+{
+    const float r = (float)rho0;
+    const float wa = (float)weight(1), wd = (float)weight(7);
+    auto twice = [](float v) { return make_float2(v, v); };
+    c.omega = (float)wp;
+    c.wp = twice(-(float)wp);
+    c.wm = twice(-(float)wm);
+    c.wmb = twice((float)wm);
+    c.rho0 = std::ldexp(r, s);
+    c.irho0 = std::ldexp(1.0f / r, -s);
+    c.r15 = std::ldexp(1.5f * r, s);
+    c.r45 = twice(std::ldexp(4.5f * r, s));
+    c.w3a = twice(-std::ldexp((wa * 3.0f) * r, s));
+    c.w3d = twice(-std::ldexp((wd * 3.0f) * r, s));
+    c.dshift = std::ldexp((float)delta_rho, s);
+    for (int i = 0; i < Q; ++i) c.rate[i] = (float)rates[i] / (float)mrt_norm2(i);
+    c.hash_off = (uint32_t)s << 23;
+}
+
+// ... and double.  alpha and c1, beta and c3 are rounded together, so that the rounded
+// collision conserves mass, 24 c1d + c10 = omega+ = 1 - a0, and momentum,
+// 2 beta + 2 c3a + 8 c3d = 1, to one rounding of the smallest of them.
+static void collision_constants(CollPar<double> &c, double wp, double wm, double rho0, double delta_rho,
+                                const double *rates)
+{
+    c.a0 = 1.0 - wp;
+    c.alpha = 0.5 * c.a0;
+    const double w = 1.0 - c.a0;
+    c.c1d = w / 36.0;
+    c.c1a = 2.0 * c.c1d;
+    c.c10 = w - 24.0 * c.c1d;
+    c.beta = 0.5 - 0.5 * wm;
+    c.c3d = (0.5 - c.beta) / 6.0;
+    c.c3a = (0.5 - c.beta) - 4.0 * c.c3d;
+    c.c2a = w / (4.0 * rho0);
+    c.c2d = 0.5 * c.c2a;
+    c.kap = -1.5 / rho0;
+    c.rho0 = rho0;
+    c.irho0 = 1.0 / rho0;
+    c.dshift = delta_rho;
+    for (int i = 0; i < Q; ++i) c.rate[i] = rates[i] / (double)mrt_norm2(i);
+}
+
 static void fill_dev(const Instance &in, InstanceDev &D)
 {
     const lbm_desc &d = in.desc;
@@ -352,33 +398,25 @@ static void fill_dev(const Instance &in, InstanceDev &D)
     D.scale = std::ldexp(1.0f, in.dev_scale_log2);
     D.inv_scale = std::ldexp(1.0f, -in.dev_scale_log2);
     const double tau = d.tau;
-    D.omega = 1.0 / tau;
-    D.omega_m = 1.0 / (0.5 + d.magic_lambda / (tau - 0.5));
+    const double omega = 1.0 / tau;
+    const double omega_m = d.collision == LBM_SRT ? omega : 1.0 / (0.5 + d.magic_lambda / (tau - 0.5));
+    double rates[Q];
     if (!in.mrt_rates.empty()) {
-        for (int i = 0; i < Q; ++i) D.s[i] = in.mrt_rates[i];
+        for (int i = 0; i < Q; ++i) rates[i] = in.mrt_rates[i];
     } else {
         // Sec. 2.1: s_nu = 1/tau on the viscous modes, s_zeta = 8(2-s_nu)/(8-s_nu) on the
         // kinetic modes, energy modes by the ratio rule, conserved modes 0.
         const double snu = 1.0 / tau;
         const double sz = 8.0 * (2.0 - snu) / (8.0 - snu);
         const double se = 1.0 / (0.5 + (tau - 0.5) / d.mrt_energy_ratio);
-        for (int i = 0; i < Q; ++i) D.s[i] = sz;
-        D.s[0] = D.s[3] = D.s[5] = D.s[7] = 0.0;
-        D.s[9] = D.s[11] = D.s[13] = D.s[14] = D.s[15] = snu;
-        D.s[1] = D.s[2] = se;
+        for (int i = 0; i < Q; ++i) rates[i] = sz;
+        rates[0] = rates[3] = rates[5] = rates[7] = 0.0;
+        rates[9] = rates[11] = rates[13] = rates[14] = rates[15] = snu;
+        rates[1] = rates[2] = se;
     }
-    D.delta_rho = d.delta_rho;
     D.rho0 = d.rho0;
-    D.omega_f = (float)D.omega;
-    D.omega_m_f = (float)D.omega_m;
-    D.rho0_f = (float)D.rho0;
-    D.irho0_f = 1.0f / D.rho0_f;
-    D.delta_rho_f = (float)D.delta_rho;
-    D.irho0 = 1.0 / D.rho0;
-    for (int i = 0; i < Q; ++i) {
-        D.rate_f[i] = (float)D.s[i] / (float)mrt_norm2(i);
-        D.rate_d[i] = D.s[i] / (double)mrt_norm2(i);
-    }
+    collision_constants(D.cf, omega, omega_m, d.rho0, d.delta_rho, in.dev_scale_log2, rates);
+    collision_constants(D.cd, omega, omega_m, d.rho0, d.delta_rho, rates);
 }
 
 // cuTensorMapEncodeTiled, looked up once through the runtime (no link to the driver library)

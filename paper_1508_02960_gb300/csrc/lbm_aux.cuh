@@ -97,7 +97,7 @@ __global__ void init_kernel(const InstanceDev *__restrict__ table, int inst, int
         T *f = reinterpret_cast<T *>(layout == 0 ? (cur ? I.f1 : I.f0) : I.f0);
         if ((meta.x >> lane) & 1u) {
 #pragma unroll
-            for (int k = 0; k < Q; ++k) f[(long long)k * I.ks + cell] = S::pack(0.0f, I.scale);
+            for (int k = 0; k < Q; ++k) f[(long long)k * I.ks + cell] = S::pack(0.0f);
             continue;
         }
         double u[3] = {0.0, 0.0, 0.0};
@@ -108,7 +108,7 @@ __global__ void init_kernel(const InstanceDev *__restrict__ table, int inst, int
         for (int k = 0; k < Q; ++k) {
             const double eu = ex(k) * u[0] + ey(k) * u[1] + ez(k) * u[2];
             const double g = weight(k) * I.rho0 * (3.0 * eu + 4.5 * eu * eu - 1.5 * uu);
-            f[(long long)(layout == 0 ? k : opp(k)) * I.ks + cell] = S::pack((typename S::R)g, I.scale);
+            f[(long long)(layout == 0 ? k : opp(k)) * I.ks + cell] = S::pack((typename S::R)g * I.scale);
         }
     }
 }
@@ -131,13 +131,12 @@ __global__ void wall_prepare_kernel(const InstanceDev *__restrict__ table, int i
     T *f = reinterpret_cast<T *>(layout == 0 && cur ? I.f1 : I.f0);
     const R *linkc = reinterpret_cast<const R *>(I.linkc);
     const long long ks = I.ks, nx = I.nx, ny = I.ny, nz = I.nz;
-    constexpr bool sr = sizeof(T) == 2;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nb;
          b += (long long)gridDim.x * blockDim.x) {
         const long long cell = bcell[b];
         const uint32_t wm = I.bmask[b], off = I.boff[b];
         const long long x = cell % nx, yz = cell / nx, y = yz % ny, z = yz / ny;
-        const uint32_t h = sr ? cell_hash((uint32_t)cell) : 0u;
+        const RoundKey key = round_key<STORE>((uint32_t)cell, I.cf.hash_off);
         // the cell's moments at t (for IEBB): the post-collision state conserves them
         R drho = R(0), u[3] = {R(0), R(0), R(0)};
         if (I.wall == 4) {
@@ -175,8 +174,7 @@ __global__ void wall_prepare_kernel(const InstanceDev *__restrict__ table, int i
                 sv = wall_own_part(I.wall, cq, C, B);
             }
             const long long src = (x - ex(k) + nx) % nx + nx * ((y - ey(k) + ny) % ny + ny * ((z - ez(k) + nz) % nz));
-            f[(long long)(layout == 0 ? k : kb) * ks + src] =
-                sr ? S::pack_sr(sv, I.scale, round_bits(h, k, float(sv))) : S::pack(sv, I.scale);
+            put1<STORE>(f + (long long)(layout == 0 ? k : kb) * ks + src, sv * R(I.scale), key, k);
         }
     }
 }
@@ -198,10 +196,10 @@ __global__ void import_kernel(const InstanceDev *__restrict__ table, int inst, i
         T *f = reinterpret_cast<T *>(layout == 0 ? (cur ? I.f1 : I.f0) : I.f0);
         const long long slot = (long long)(layout == 0 ? k : opp(k)) * I.ks + cell;
         if ((meta.x >> lane) & 1u) {
-            f[slot] = S::pack(0.0f, I.scale);
+            f[slot] = S::pack(0.0f);
             continue;
         }
-        f[slot] = S::pack((typename S::R)(fk[cell] - wr), I.scale);
+        f[slot] = S::pack((typename S::R)(fk[cell] - wr) * I.scale);
     }
 }
 

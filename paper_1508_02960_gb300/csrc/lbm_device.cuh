@@ -136,45 +136,53 @@ template <> struct Store<ST_F64> {
     using T = double;
     using R = double;
     __device__ static R load(const T *p, float) { return __ldg(p); }
-    __device__ static R cvt(T v, float) { return v; }
-    __device__ static T pack(R v, float) { return v; }
-    __device__ static T pack_sr(R v, float, uint32_t) { return v; }
+    __device__ static R cvt(T v) { return v; }
+    __device__ static T pack(R v) { return v; }
 };
 template <> struct Store<ST_F32> {
     using T = float;
     using R = float;
     __device__ static R load(const T *p, float) { return __ldg(p); }
-    __device__ static R cvt(T v, float) { return v; }
-    __device__ static T pack(R v, float) { return v; }
-    __device__ static T pack_sr(R v, float, uint32_t) { return v; }
+    __device__ static R cvt(T v) { return v; }
+    __device__ static T pack(R v) { return v; }
 };
+// Stochastic rounding of the 16-bit formats: random bits (the upper ones of ra, rb) are added
+// below the format's mantissa and the sum truncated.  pack2_sr rounds two values, a to the
+// upper half of the result and b to the lower.
 // FP16 deviation with a power-of-two scale 2^s: stored = g * 2^s (exact scaling).
 template <> struct Store<ST_F16> {
     using T = __half;
     using R = float;
     __device__ static R load(const T *p, float inv_scale) { return __half2float(__ldg(p)) * inv_scale; }
-    __device__ static R cvt(T v, float inv_scale) { return __half2float(v) * inv_scale; }
-    __device__ static T pack(R v, float scale) { return __float2half_rn(v * scale); }
-    // stochastic rounding: 13 random bits added below the FP16 mantissa, then truncation
-    __device__ static T pack_sr(R v, float scale, uint32_t rnd)
+    __device__ static R cvt(T v) { return __half2float(v); }
+    __device__ static T pack(R v) { return __float2half_rn(v); }
+    // 13 random bits; one packed conversion (the scalar one to FP16 runs at an eighth of it)
+    __device__ static uint32_t pack2_sr(R a, R b, uint32_t ra, uint32_t rb)
     {
-        const float x = v * scale;
-        return __float2half_rz(__uint_as_float(__float_as_uint(x) + (rnd >> 19)));
+        uint32_t d;
+        asm("cvt.rz.f16x2.f32 %0, %1, %2;"
+            : "=r"(d)
+            : "f"(__uint_as_float(__float_as_uint(a) + (ra >> 19))), "f"(__uint_as_float(__float_as_uint(b) + (rb >> 19))));
+        return d;
     }
+    __device__ static T half_of(uint32_t d, int hi) { return __ushort_as_half((unsigned short)(hi ? d >> 16 : d)); }
 };
 template <> struct Store<ST_BF16> {
     using T = __nv_bfloat16;
     using R = float;
     __device__ static R load(const T *p, float) { return __bfloat162float(__ldg(p)); }
-    __device__ static R cvt(T v, float) { return __bfloat162float(v); }
-    __device__ static T pack(R v, float) { return __float2bfloat16_rn(v); }
-    // stochastic rounding: 16 random bits added below the BF16 mantissa, then truncation
-    __device__ static T pack_sr(R v, float, uint32_t rnd)
+    __device__ static R cvt(T v) { return __bfloat162float(v); }
+    __device__ static T pack(R v) { return __float2bfloat16_rn(v); }
+    // 16 random bits, added and truncated by the conversion itself
+    __device__ static uint32_t pack2_sr(R a, R b, uint32_t ra, uint32_t rb)
     {
-        const uint32_t b = __float_as_uint(v) + (rnd >> 16);
-        return __ushort_as_bfloat16((unsigned short)(b >> 16));
+        uint32_t d;
+        asm("cvt.rs.bf16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(a), "f"(b), "r"(__byte_perm(rb, ra, 0x7632)));
+        return d;
     }
+    __device__ static T half_of(uint32_t d, int hi) { return __ushort_as_bfloat16((unsigned short)(hi ? d >> 16 : d)); }
 };
+template <int S> constexpr bool kStochastic = S == ST_F16 || S == ST_BF16;
 
 // Random bits for the stochastic rounding of population k of a cell: cell_hash mixes the
 // cell index once (SplitMix-style finaliser), then one multiply per direction folds in the
@@ -188,9 +196,46 @@ __device__ __forceinline__ uint32_t cell_hash(uint32_t cell)
     h *= 0xC2B2AE35u;
     return h ^ (h >> 16);
 }
-__device__ __forceinline__ uint32_t round_bits(uint32_t h, int k, float v)
+// (bits: those of the deviation in FP32; h ^ bits is one instruction, the multiply the other)
+__device__ __forceinline__ uint32_t round_bits(uint32_t h, int k, uint32_t bits)
 {
-    return (h ^ __float_as_uint(v)) * (0x9E3779B1u + 0x6A09E666u * (uint32_t)k);
+    return (h ^ bits) * (0x9E3779B1u + 0x6A09E666u * (uint32_t)k);
+}
+
+// Hash of a cell for the stochastic rounding of its values; off: CollPar::hash_off.
+struct RoundKey {
+    uint32_t h, off;
+};
+template <int STORE> __device__ __forceinline__ RoundKey round_key(uint32_t cell, uint32_t off)
+{
+    if constexpr (kStochastic<STORE>) return {cell_hash(cell), STORE == ST_F16 ? off : 0u};
+    else return {0u, 0u};
+}
+
+// Store the values a and b of directions k and l of a cell to pa and pb, or a alone to pa:
+// rounded stochastically in the 16-bit formats, as they are in the wider ones.
+template <int STORE>
+__device__ __forceinline__ void put2(typename Store<STORE>::T *pa, typename Store<STORE>::T *pb,
+                                     typename Store<STORE>::R a, typename Store<STORE>::R b, RoundKey key, int k, int l)
+{
+    using S = Store<STORE>;
+    if constexpr (kStochastic<STORE>) {
+        const uint32_t d = S::pack2_sr(a, b, round_bits(key.h, k, __float_as_uint(a) - key.off),
+                                       round_bits(key.h, l, __float_as_uint(b) - key.off));
+        *pa = S::half_of(d, 1);
+        *pb = S::half_of(d, 0);
+    } else {
+        *pa = S::pack(a);
+        *pb = S::pack(b);
+    }
+}
+template <int STORE>
+__device__ __forceinline__ void put1(typename Store<STORE>::T *pa, typename Store<STORE>::R a, RoundKey key, int k)
+{
+    using S = Store<STORE>;
+    if constexpr (kStochastic<STORE>)
+        *pa = S::half_of(S::pack2_sr(0.0f, a, 0u, round_bits(key.h, k, __float_as_uint(a) - key.off)), 0);
+    else *pa = S::pack(a);
 }
 
 inline size_t storage_bytes(int s) { return s == ST_F64 ? 8 : (s == ST_F32 ? 4 : 2); }
@@ -254,6 +299,41 @@ enum { STATUS_DIVERGED = 1u, STATUS_TIMEOUT = 2u, STATUS_BOUNDS = 4u };
 // the wall), boff[b] the index of its first link; its links are ordered by k.  Link l:
 // linkc[l] = CLI coefficient (1-2q)/(1+2q) (0 where CLI falls back to SBB).
 // ------------------------------------------------------------------------------------
+
+// Constants of the collision as the step kernels use them, computed on the host so that no
+// thread converts or divides.
+//
+// Single precision, for the formats that collide in FP32: the parameters rounded to single
+// and the products of them that Eqs. SRT, TRT, MRT and equilibrium begin with.  FP16 storage
+// collides the stored values, deviations times 2^s (every product with a power of two is
+// exact), so rho0 and the pressure shift carry 2^s and 1/rho0 carries 2^-s; the other formats
+// have s = 0.
+template <typename R> struct CollPar;
+template <> struct CollPar<float> {
+    // twice over, for packed FP32 instructions: -omega+, -+ omega-, 9/2 rho0 2^s, and
+    // -3 w rho0 2^s of the axis and diagonal directions
+    float2 wp, wm, wmb, r45, w3a, w3d;
+    float omega;            // SRT omega = 1/tau, TRT omega+
+    float rho0, irho0;      // rho0 2^s, 2^-s / rho0
+    float r15;              // 3/2 rho0 2^s
+    float dshift;           // delta_rho 2^s
+    float rate[Q];          // MRT: s_i / |M_i|^2
+    uint32_t hash_off;      // FP16: s << 23 (round_bits hashes the deviation itself)
+};
+// Double precision, for FP64 storage (SRT is TRT with omega- = omega+).  With j = sum e_k g_k,
+// s = g_k + g_kbar and d = g_k - g_kbar of an opposite pair and B = drho - 3/2 j.j / rho0,
+//   (g~_k + g~_kbar) / 2 = alpha s + c2 (e.j)^2 + c1 B,   alpha = (1 - omega+) / 2,
+//   (g~_k - g~_kbar) / 2 = beta d + c3 e.j,               beta = (1 - omega-) / 2,
+//   g~_0 = (1 - omega+) g_0 + c10 B,
+// c1 = omega+ w, c2 = 9/2 omega+ w / rho0, c3 = 3 omega- w for the axis (a) and diagonal (d)
+// pairs.
+template <> struct CollPar<double> {
+    double a0, alpha, beta, c1a, c1d, c10, c2a, c2d, c3a, c3d;
+    double kap;             // -3/2 / rho0
+    double rho0, irho0, dshift;
+    double rate[Q];         // MRT: s_i / |M_i|^2
+};
+
 struct InstanceDev {
     void *f0, *f1;           // populations [19][ks] (direction k at k * ks); AA uses f0 only
     const uint4 *seg;        // [nseg]
@@ -280,18 +360,9 @@ struct InstanceDev {
     int wall;                // 0 = SBB, 1 = CLI, 2 = LIBB, 3 = QIBB, 4 = IEBB, 5 = MR
     int phase;               // A-B: buffer holding the current state when flip == 0
     float scale, inv_scale;  // FP16 deviation scaling
-    double omega;            // SRT omega = 1/tau; TRT omega+
-    double omega_m;          // TRT omega-
-    double s[Q];             // MRT relaxation rates
-    double delta_rho, rho0;
-    // the same parameters as the step kernels use them, computed on the host so that no
-    // thread converts or divides them: single precision for the formats that collide in FP32
-    // (each the correctly rounded single of the double above, 1/rho0 the correctly rounded
-    // quotient), and the MRT rates divided by |M_i|^2 in both precisions
-    float omega_f, omega_m_f, rho0_f, irho0_f, delta_rho_f;
-    double irho0;
-    float rate_f[Q];
-    double rate_d[Q];
+    double rho0;
+    CollPar<float> cf;       // the collision of the formats that collide in FP32
+    CollPar<double> cd;      // that of FP64 storage
     // sizes the checked build tests indices against, and the batch's sticky error word
     // (STATUS_BOUNDS, STATUS_TIMEOUT), which the host reads with the reductions
     uint32_t n_fwarps_padded, n_boundary, n_links;

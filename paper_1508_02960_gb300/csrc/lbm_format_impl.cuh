@@ -32,6 +32,9 @@ cudaError_t launch_step(void (*kernel)(P...), const Launch &L, A &&...args)
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// The collision a format's kernels run: FP64 SRT is TRT with both rates equal.
+template <int STORE> constexpr int kSrt = STORE == ST_F64 ? (int)COLL_TRT : (int)COLL_SRT;
+
 template <int STORE, int COLL, int KIND, bool RED, bool WX, int WARPS>
 cudaError_t step_red(const Launch &L, int flip, unsigned *status, const InstanceDev *one)
 {
@@ -76,11 +79,11 @@ cudaError_t step(int coll, int kind, const Launch &L, int flip, int reduce, unsi
                  int wx, int warps)
 {
     switch (coll * 3 + kind) {
-    case COLL_SRT * 3 + KIND_AB: return step_one<STORE, COLL_SRT, KIND_AB>(L, flip, reduce, status, one, wx, warps);
+    case COLL_SRT * 3 + KIND_AB: return step_one<STORE, kSrt<STORE>, KIND_AB>(L, flip, reduce, status, one, wx, warps);
     case COLL_SRT * 3 + KIND_AA_PULL:
-        return step_one<STORE, COLL_SRT, KIND_AA_PULL>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, kSrt<STORE>, KIND_AA_PULL>(L, flip, reduce, status, one, wx, warps);
     case COLL_SRT * 3 + KIND_AA_LOCAL:
-        return step_one<STORE, COLL_SRT, KIND_AA_LOCAL>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, kSrt<STORE>, KIND_AA_LOCAL>(L, flip, reduce, status, one, wx, warps);
     case COLL_TRT * 3 + KIND_AB: return step_one<STORE, COLL_TRT, KIND_AB>(L, flip, reduce, status, one, wx, warps);
     case COLL_TRT * 3 + KIND_AA_PULL:
         return step_one<STORE, COLL_TRT, KIND_AA_PULL>(L, flip, reduce, status, one, wx, warps);
@@ -120,8 +123,8 @@ template <int STORE>
 cudaError_t step_tma(int coll, int wx, const TmaLaunch &T, const InstanceDev &one, int flip)
 {
     switch (coll * 2 + (wx ? 1 : 0)) {
-    case COLL_SRT * 2: return step_tma_one<STORE, COLL_SRT, false>(T, one, flip);
-    case COLL_SRT * 2 + 1: return step_tma_one<STORE, COLL_SRT, true>(T, one, flip);
+    case COLL_SRT * 2: return step_tma_one<STORE, kSrt<STORE>, false>(T, one, flip);
+    case COLL_SRT * 2 + 1: return step_tma_one<STORE, kSrt<STORE>, true>(T, one, flip);
     case COLL_TRT * 2: return step_tma_one<STORE, COLL_TRT, false>(T, one, flip);
     case COLL_TRT * 2 + 1: return step_tma_one<STORE, COLL_TRT, true>(T, one, flip);
     case COLL_MRT * 2: return step_tma_one<STORE, COLL_MRT, false>(T, one, flip);
@@ -146,8 +149,8 @@ template <int STORE, int COLL, bool WX> int tma_prepare_one()
 template <int STORE> int tma_prepare(int coll, int wx)
 {
     switch (coll * 2 + (wx ? 1 : 0)) {
-    case COLL_SRT * 2: return tma_prepare_one<STORE, COLL_SRT, false>();
-    case COLL_SRT * 2 + 1: return tma_prepare_one<STORE, COLL_SRT, true>();
+    case COLL_SRT * 2: return tma_prepare_one<STORE, kSrt<STORE>, false>();
+    case COLL_SRT * 2 + 1: return tma_prepare_one<STORE, kSrt<STORE>, true>();
     case COLL_TRT * 2: return tma_prepare_one<STORE, COLL_TRT, false>();
     case COLL_TRT * 2 + 1: return tma_prepare_one<STORE, COLL_TRT, true>();
     case COLL_MRT * 2: return tma_prepare_one<STORE, COLL_MRT, false>();

@@ -62,10 +62,17 @@ inline size_t step_smem_bytes(int, int) { return 0; }
 template <typename R> struct Par {
     uint32_t ks, nx, ny, nz;
     FastDiv dnx, dny;
-    R omega, omega_m, rho0, irho0, dshift;
-    float sc, isc;
+    CollPar<R> c;
+    float isc;
+    uint32_t hash_off;
     int wall;
 };
+
+template <typename R> __device__ __forceinline__ const CollPar<R> &coll_par(const InstanceDev &I)
+{
+    if constexpr (sizeof(R) == sizeof(float)) return I.cf;
+    else return I.cd;
+}
 
 template <typename R> __device__ __forceinline__ Par<R> load_par(const InstanceDev &I)
 {
@@ -76,21 +83,9 @@ template <typename R> __device__ __forceinline__ Par<R> load_par(const InstanceD
     p.nz = I.nz;
     p.dnx = I.div_nx;
     p.dny = I.div_ny;
-    if constexpr (sizeof(R) == sizeof(float)) {
-        p.omega = I.omega_f;
-        p.omega_m = I.omega_m_f;
-        p.rho0 = I.rho0_f;
-        p.irho0 = I.irho0_f;
-        p.dshift = I.delta_rho_f;
-    } else {
-        p.omega = I.omega;
-        p.omega_m = I.omega_m;
-        p.rho0 = I.rho0;
-        p.irho0 = I.irho0;
-        p.dshift = I.delta_rho;
-    }
-    p.sc = I.scale;
+    p.c = coll_par<R>(I);
     p.isc = I.inv_scale;
+    p.hash_off = I.cf.hash_off;
     p.wall = I.wall;
     return p;
 }
@@ -168,19 +163,285 @@ __device__ __forceinline__ uint2 ld_keep(const uint2 *a, uint64_t pol)
 template <int STORE, int COLL, bool RED, bool WX, int WARPS = kStepWarps, int KIND = KIND_AB, bool BATCH = false>
 constexpr int step_min_blocks()
 {
-    // the in-place steps of the 16-bit formats (stochastic rounding, scaling) spill at 56
-    // registers: 32 warps, measured 0.3-3 % faster than 36; so does a batch's local step,
-    // whose parameters come from the instance table instead of the constant bank (60 bytes
-    // at 56 registers; 32 warps measured 3-6 % faster on batches of 2-4 cells)
-    constexpr bool wide = RED || WX || COLL == COLL_MRT || ((STORE == ST_F16 || STORE == ST_BF16) && KIND != KIND_AB) ||
-                          (BATCH && KIND == KIND_AA_LOCAL);
+    // the in-place steps of the 16-bit formats (stochastic rounding) spill at 56 registers: 32
+    // warps, measured 0.3-3 % faster than 36; so do a batch's steps, whose parameters come
+    // from the instance table instead of the constant bank
+    constexpr bool wide = RED || WX || COLL == COLL_MRT || BATCH ||
+                          ((STORE == ST_F16 || STORE == ST_BF16) && KIND != KIND_AB);
     return (STORE == ST_F64 ? 8 : wide ? 32 : LBM_STEP_WARPS_PER_SM) / WARPS;
 }
 
-// Moments of the incoming populations (Eq. Macro), in deviation form.
-template <typename R>
-__device__ __forceinline__ void moments(const R (&g)[Q], R irho0, R &drho, R &ux, R &uy, R &uz)
+// Two values of the compute type side by side.  FP32: a register pair and Blackwell's packed
+// FP32 instructions (add, sub, mul, fma .f32x2: both values by one instruction, each rounded
+// as by the scalar one), which halve the issue slots of the collision; FP64: two scalars.
+template <typename R> struct Pair;
+template <> struct Pair<float> {
+    unsigned long long v;
+};
+template <> struct Pair<double> {
+    double x, y;
+};
+__device__ __forceinline__ Pair<float> pair_of(float x, float y)
 {
+    Pair<float> p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p.v) : "f"(x), "f"(y));
+    return p;
+}
+__device__ __forceinline__ Pair<double> pair_of(double x, double y) { return {x, y}; }
+__device__ __forceinline__ void split(const Pair<float> &p, float &x, float &y)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(p.v));
+}
+__device__ __forceinline__ void split(const Pair<double> &p, double &x, double &y)
+{
+    x = p.x;
+    y = p.y;
+}
+__device__ __forceinline__ Pair<float> operator+(const Pair<float> &a, const Pair<float> &b)
+{
+    Pair<float> d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+__device__ __forceinline__ Pair<float> operator-(const Pair<float> &a, const Pair<float> &b)
+{
+    Pair<float> d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+__device__ __forceinline__ Pair<float> operator*(const Pair<float> &a, const Pair<float> &b)
+{
+    Pair<float> d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+__device__ __forceinline__ Pair<float> fma_r(const Pair<float> &a, const Pair<float> &b, const Pair<float> &c)
+{
+    Pair<float> d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return d;
+}
+__device__ __forceinline__ Pair<double> operator+(const Pair<double> &a, const Pair<double> &b)
+{
+    return {a.x + b.x, a.y + b.y};
+}
+__device__ __forceinline__ Pair<double> operator-(const Pair<double> &a, const Pair<double> &b)
+{
+    return {a.x - b.x, a.y - b.y};
+}
+__device__ __forceinline__ Pair<double> operator*(const Pair<double> &a, const Pair<double> &b)
+{
+    return {a.x * b.x, a.y * b.y};
+}
+__device__ __forceinline__ Pair<double> fma_r(const Pair<double> &a, const Pair<double> &b, const Pair<double> &c)
+{
+    return {fma_r(a.x, b.x, c.x), fma_r(a.y, b.y, c.y)};
+}
+__device__ __forceinline__ Pair<float> pair_of(const float2 &a) { return pair_of(a.x, a.y); }
+template <typename R> __device__ __forceinline__ Pair<R> both(R a) { return pair_of(a, a); }
+template <typename R> __device__ __forceinline__ R sum_of(const Pair<R> &p)
+{
+    R x, y;
+    split(p, x, y);
+    return x + y;
+}
+
+// Moments and collision of one cell, in place on the pulled values g[] (deviations, in the
+// units of CollPar): Eqs. Macro, SRT, TRT, MRT with the equilibrium of Eq. equilibrium.
+// Returns drho = sum g_k and u = rho0^-1 sum e_k g_k.
+//
+// Three forms.
+//  - relax_pairs, TRT: on the sums s and differences d of opposite pairs, the directions 1, 3
+//    (axis x, y), 7, 9 (diagonals of the xy plane), 11, 13 (xz) and 15, 17 (yz) two to a
+//    Pair, 5 (axis z) alone.  FP64: the bound is the FP64 pipe (a warp instruction per 19
+//    cycles a multiprocessor, 64 cycles for a warp alone), so the count is what matters: 116
+//    (CollPar<double>) where the pair form of the equations takes about 150; SRT runs it with
+//    omega- = omega+.  FP32: Eq. TRT operation by operation, 97 instructions for 147
+//    operations; its values are those of the scalar form, bit for bit (the 16-bit formats'
+//    stochastic rounding hashes them).
+//  - relax_rows, MRT of FP64 and FP32 storage: g~ = g - M^T delta, delta_i = s_i / |M_i|^2
+//    (m_i - m_i^eq).  The rows of M are combinations of the same few sums per axis and per
+//    plane (checked against mrt_m at compile time below), so the moments and the way back take
+//    177 operations instead of the 19 x 19 products; the equilibrium moments follow from Eq.
+//    equilibrium: e -11 drho + 19 j.j/rho0, eps 3 drho - 11/2 j.j/rho0, 3p_xx
+//    (3 jx^2 - j.j)/rho0, 3pi_xx -1/2 of it, p_ww (jy^2 - jz^2)/rho0, pi_ww -1/2 of it, p_ab
+//    ja jb/rho0, q -2/3 j, m 0.
+//  - relax_plain, FP32 SRT and the MRT of the 16-bit formats, whose FP32 values (hashed by the
+//    stochastic rounding) are those of these expressions.
+template <typename R> struct PairSums {
+    Pair<R> s1, s7, s11, s15, d1, d7, d11, d15;
+    R s5, d5;
+    __device__ __forceinline__ explicit PairSums(const R (&g)[Q])
+    {
+        const Pair<R> a1 = pair_of(g[1], g[3]), b1 = pair_of(g[2], g[4]);
+        const Pair<R> a7 = pair_of(g[7], g[9]), b7 = pair_of(g[8], g[10]);
+        const Pair<R> a11 = pair_of(g[11], g[13]), b11 = pair_of(g[12], g[14]);
+        const Pair<R> a15 = pair_of(g[15], g[17]), b15 = pair_of(g[16], g[18]);
+        s1 = a1 + b1, s7 = a7 + b7, s11 = a11 + b11, s15 = a15 + b15;
+        d1 = a1 - b1, d7 = a7 - b7, d11 = a11 - b11, d15 = a15 - b15;
+        s5 = g[5] + g[6], d5 = g[5] - g[6];
+    }
+};
+
+__device__ __forceinline__ void relax_pairs(double (&g)[Q], const CollPar<double> &c, double &drho, double &ux,
+                                            double &uy, double &uz)
+{
+    using R = double;
+    using V = Pair<double>;
+    const auto [s1, s7, s11, s15, d1, d7, d11, d15, s5, d5] = PairSums<double>(g);
+    // per plane: the x (or y) and the y or z momentum of its four diagonals
+    R jx, jy, jz, u, v;
+    split(d7, u, v);
+    const R x7 = u + v, y7 = u - v;
+    split(d11, u, v);
+    const R x11 = u + v, z11 = u - v;
+    split(d15, u, v);
+    const R y15 = u + v, z15 = u - v;
+    drho = sum_of((s1 + s7) + (s11 + s15)) + (s5 + g[0]);
+    const V jxy = (d1 + pair_of(x7, y7)) + pair_of(x11, y15);
+    split(jxy, jx, jy);
+    jz = d5 + (z11 + z15);
+    const V q1 = jxy * jxy;
+    const R q5 = jz * jz;
+    const R B = fma_r(c.kap, sum_of(q1) + q5, drho);
+    const R E1 = c.c1a * B, E7 = c.c1d * B;
+    const V al = both(c.alpha), be = both(c.beta), c2d = both(c.c2d), c3d = both(c.c3d), E7v = both(E7);
+    auto give = [&](int k, const V &s, const V &d, const V &ej, const V &qc, const V &c3) {
+        const V h = fma_r(al, s, qc), t = fma_r(be, d, c3 * ej);
+        split(h + t, g[k], g[k + 2]);
+        split(h - t, g[k + 1], g[k + 3]);
+    };
+    g[0] = fma_r(c.a0, g[0], c.c10 * B);
+    give(1, s1, d1, jxy, fma_r(both(c.c2a), q1, both(E1)), both(c.c3a));
+    {
+        const R h = fma_r(c.alpha, s5, fma_r(c.c2a, q5, E1)), t = fma_r(c.beta, d5, c.c3a * jz);
+        g[5] = h + t;
+        g[6] = h - t;
+    }
+    const V e7 = pair_of(jx + jy, jx - jy), e11 = pair_of(jx + jz, jx - jz), e15 = pair_of(jy + jz, jy - jz);
+    give(7, s7, d7, e7, fma_r(c2d, e7 * e7, E7v), c3d);
+    give(11, s11, d11, e11, fma_r(c2d, e11 * e11, E7v), c3d);
+    give(15, s15, d15, e15, fma_r(c2d, e15 * e15, E7v), c3d);
+    ux = jx * c.irho0;
+    uy = jy * c.irho0;
+    uz = jz * c.irho0;
+}
+
+__device__ __forceinline__ void relax_pairs(float (&g)[Q], const CollPar<float> &c, float &drho, float &ux, float &uy,
+                                            float &uz)
+{
+    using R = float;
+    using V = Pair<float>;
+    const auto [s1, s7, s11, s15, d1, d7, d11, d15, s5, d5] = PairSums<float>(g);
+    R sx, sy, s7x, s7y, s11x, s11y, s15x, s15y, dx, dy, d7x, d7y, d11x, d11y, d15x, d15y;
+    split(s1, sx, sy);
+    split(s7, s7x, s7y);
+    split(s11, s11x, s11y);
+    split(s15, s15x, s15y);
+    split(d1, dx, dy);
+    split(d7, d7x, d7y);
+    split(d11, d11x, d11y);
+    split(d15, d15x, d15y);
+    drho = ((((((((g[0] + sx) + sy) + s5) + s7x) + s7y) + s11x) + s11y) + s15x) + s15y;
+    ux = ((((dx + d7x) + d7y) + d11x) + d11y) * c.irho0;
+    uy = ((((dy + d7x) - d7y) + d15x) + d15y) * c.irho0;
+    uz = ((((d5 + d11x) - d11y) + d15x) - d15y) * c.irho0;
+    const R uu = fma_r(uz, uz, fma_r(ux, ux, __fmul_rn(uy, uy)));
+    const R base = fma_r(-c.r15, uu, drho);  // drho - 3/2 rho0 u.u
+    const V wp = pair_of(c.wp), wm = pair_of(c.wm), wmb = pair_of(c.wmb), r45 = pair_of(c.r45), basev = both(base);
+    // Y, Z: the symmetric and antisymmetric parts less their equilibria
+    auto give = [&](int k, const V &eu, R w, const V &w3) {
+        const V a = pair_of(g[k], g[k + 2]), b = pair_of(g[k + 1], g[k + 3]), half = both(R(0.5));
+        const V Y = fma_r(half, a + b, both(-w) * fma_r(r45 * eu, eu, basev));
+        const V Z = fma_r(half, a - b, w3 * eu);
+        split(fma_r(wm, Z, fma_r(wp, Y, a)), g[k], g[k + 2]);
+        split(fma_r(wmb, Z, fma_r(wp, Y, b)), g[k + 1], g[k + 3]);
+    };
+    constexpr R wa = R(weight(1)), wd = R(weight(7));
+    g[0] = fma_r(-c.omega, fma_r(-R(weight(0)), base, g[0]), g[0]);
+    give(1, pair_of(ux, uy), wa, pair_of(c.w3a));
+    {
+        const R Y = fma_r(R(0.5), g[5] + g[6], -__fmul_rn(wa, fma_r(__fmul_rn(c.r45.x, uz), uz, base)));
+        const R Z = fma_r(R(0.5), g[5] - g[6], __fmul_rn(c.w3a.x, uz));
+        g[5] = fma_r(c.wm.x, Z, fma_r(c.wp.x, Y, g[5]));
+        g[6] = fma_r(c.wmb.x, Z, fma_r(c.wp.x, Y, g[6]));
+    }
+    give(7, pair_of(ux + uy, ux - uy), wd, pair_of(c.w3d));
+    give(11, pair_of(ux + uz, ux - uz), wd, pair_of(c.w3d));
+    give(15, pair_of(uy + uz, uy - uz), wd, pair_of(c.w3d));
+}
+
+template <typename R>
+__device__ __forceinline__ void relax_rows(R (&g)[Q], const CollPar<R> &c, R &drho, R &ux, R &uy, R &uz)
+{
+    const auto [s1, s7, s11, s15, d1, d7, d11, d15, s5, d5] = PairSums<R>(g);
+    R u, v;
+    split(d7, u, v);
+    const R x7 = u + v, y7 = u - v;
+    split(d11, u, v);
+    const R x11 = u + v, z11 = u - v;
+    split(d15, u, v);
+    const R y15 = u + v, z15 = u - v;
+    R sx, sy, pxy, pxz, pyz, mxy, mxz, myz, dx, dy;
+    split(s1, sx, sy);
+    split(d1, dx, dy);
+    split(s7, u, v);
+    pxy = u + v, mxy = u - v;
+    split(s11, u, v);
+    pxz = u + v, mxz = u - v;
+    split(s15, u, v);
+    pyz = u + v, myz = u - v;
+    const R yz = sy + s5, A = sx + yz, px = pxy + pxz, D = px + pyz;
+    drho = g[0] + (A + D);
+    const R tx = x7 + x11, ty = y7 + y15, tz = z11 + z15;
+    const R jx = dx + tx, jy = dy + ty, jz = d5 + tz;
+    ux = c.irho0 * jx;
+    uy = c.irho0 * jy;
+    uz = c.irho0 * jz;
+    const R qxx = ux * jx, qyy = uy * jy, qzz = uz * jz;
+    const R qq = qxx + (qyy + qzz), n9 = fma_r(R(3), qxx, -qq), n11 = qyy - qzz;
+    const R x9 = fma_r(R(2), sx, -yz), w9 = fma_r(R(-2), pyz, px), x11m = sy - s5, w11 = pxy - pxz;
+    const R D1 = c.rate[1] * fma_r(R(-11), A, fma_r(R(8), D, fma_r(R(-30), g[0], fma_r(R(11), drho, R(-19) * qq))));
+    const R D2 = c.rate[2] * fma_r(R(-4), A, fma_r(R(12), g[0], fma_r(R(-3), drho, fma_r(R(5.5), qq, D))));
+    const R D9 = c.rate[9] * (x9 + (w9 - n9)), D11 = c.rate[11] * (x11m + (w11 - n11));
+    const R D10 = c.rate[10] * fma_r(R(-2), x9, fma_r(R(0.5), n9, w9));
+    const R D12 = c.rate[12] * fma_r(R(-2), x11m, fma_r(R(0.5), n11, w11));
+    const R D13 = c.rate[13] * fma_r(-ux, jy, mxy);
+    const R D14 = c.rate[14] * fma_r(-uy, jz, myz);
+    const R D15 = c.rate[15] * fma_r(-ux, jz, mxz);
+    const R D4 = c.rate[4] * fma_r(R(-4), dx, fma_r(R(2.0 / 3.0), jx, tx));
+    const R D6 = c.rate[6] * fma_r(R(-4), dy, fma_r(R(2.0 / 3.0), jy, ty));
+    const R D8 = c.rate[8] * fma_r(R(-4), d5, fma_r(R(2.0 / 3.0), jz, tz));
+    const R D16 = c.rate[16] * (x7 - x11), D17 = c.rate[17] * (y15 - y7), D18 = c.rate[18] * (z11 - z15);
+    // back: the even part is taken off both values of a pair, the odd part off one and
+    // added to the other
+    g[0] -= fma_r(R(12), D2, R(-30) * D1);
+    auto give = [&](int k, R ev, R od) {
+        g[k] = (g[k] - ev) - od;
+        g[k + 1] = (g[k + 1] - ev) + od;
+    };
+    const R a = fma_r(R(-11), D1, R(-4) * D2), b = fma_r(R(8), D1, D2);
+    const R u9 = fma_r(R(-2), D10, D9), u11 = fma_r(R(-2), D12, D11), v9 = D9 + D10, v11 = D11 + D12;
+    give(1, fma_r(R(2), u9, a), R(-4) * D4);
+    const R ay = a - u9;
+    give(3, ay + u11, R(-4) * D6);
+    give(5, ay - u11, R(-4) * D8);
+    const R xa = D4 + D16, ya = D6 - D17, xb = D4 - D16, za = D8 + D18, yb = D6 + D17, zb = D8 - D18;
+    const R bv = b + v9, b7 = bv + v11, b11m = bv - v11, b15m = fma_r(R(-2), v9, b);
+    give(7, b7 + D13, xa + ya);
+    give(9, b7 - D13, xa - ya);
+    give(11, b11m + D15, xb + za);
+    give(13, b11m - D15, xb - za);
+    give(15, b15m + D14, yb + zb);
+    give(17, b15m - D14, yb - zb);
+}
+
+template <int COLL>
+__device__ __forceinline__ void relax_plain(float (&g)[Q], const CollPar<float> &p, float &drho, float &ux, float &uy,
+                                            float &uz)
+{
+    using R = float;
+    const R irho0 = p.irho0, rho0 = p.rho0;
     // sums and differences of opposite pairs: drho = g_0 + sum s_p, j = sum e_p d_p
     R d_sum = g[0], jx = R(0), jy = R(0), jz = R(0);
 #pragma unroll
@@ -195,15 +456,7 @@ __device__ __forceinline__ void moments(const R (&g)[Q], R irho0, R &drho, R &ux
     ux = jx * irho0;
     uy = jy * irho0;
     uz = jz * irho0;
-}
-
-// Collision of one cell, in place on g[] (deviations), Eqs. SRT, TRT, MRT with the
-// equilibrium of Eq. equilibrium.  rates: the 19 MRT rates (MRT only).
-template <int COLL, typename R>
-__device__ __forceinline__ void collide(R (&g)[Q], const Par<R> &p, const R *rates, R drho, R ux, R uy, R uz)
-{
-    const R rho0 = p.rho0;
-    const R uu = ux * ux + uy * uy + uz * uz;
+    const R uu = fma_r(uz, uz, fma_r(ux, ux, __fmul_rn(uy, uy)));
     if constexpr (COLL == COLL_SRT) {
         const R om = p.omega;
 #pragma unroll
@@ -212,24 +465,7 @@ __device__ __forceinline__ void collide(R (&g)[Q], const Par<R> &p, const R *rat
             const R geq = R(weight(k)) * (drho + rho0 * (R(3) * eu + R(4.5) * eu * eu - R(1.5) * uu));
             g[k] = g[k] - om * (g[k] - geq);
         }
-    } else if constexpr (COLL == COLL_TRT) {
-        // symmetric part relaxes with omega+, antisymmetric part with omega- (Eq. TRT)
-        const R wp = p.omega, wm = p.omega_m;
-        const R base = drho - R(1.5) * rho0 * uu;     // drho + rho0 (-3/2 u.u)
-        g[0] = g[0] - wp * (g[0] - R(weight(0)) * base);
-#pragma unroll
-        for (int k = 1; k < Q; k += 2) {
-            const int kb = k + 1;
-            const R w = R(weight(k));
-            const R eu = R(ex(k)) * ux + R(ey(k)) * uy + R(ez(k)) * uz;
-            const R eqp = w * (base + R(4.5) * rho0 * eu * eu);   // (f_k^eq + f_kbar^eq) / 2
-            const R eqm = (w * R(3) * rho0) * eu;                  // (f_k^eq - f_kbar^eq) / 2
-            const R dp = wp * (R(0.5) * (g[k] + g[kb]) - eqp);
-            const R dm = wm * (R(0.5) * (g[k] - g[kb]) - eqm);
-            g[k] = g[k] - dp - dm;
-            g[kb] = g[kb] - dp + dm;
-        }
-    } else {  // MRT: g~ = g - M^-1 S M (g - g^eq), M^-1 = M^T diag(1/|M_i|^2)
+    } else {  // MRT
         // Every row of M is even or odd in e (mrt_even), so a moment takes the sums (even
         // rows) or the differences (odd rows) of the opposite pairs of g - g^eq, and the
         // relaxation goes back to a pair as its even part plus or minus its odd part: the
@@ -254,18 +490,18 @@ __device__ __forceinline__ void collide(R (&g)[Q], const Par<R> &p, const R *rat
             if (i == 0 || i == 3 || i == 5 || i == 7) continue;  // conserved: m^neq = 0
             R m = R(0);
 #pragma unroll
-            for (int p = 0; p <= Q / 2; ++p) {
-                const int c = mrt_m(i, p == 0 ? 0 : 2 * p - 1);
-                const R v = mrt_even(i) ? sp[p] : dp[p];
+            for (int h = 0; h <= Q / 2; ++h) {
+                const int c = mrt_m(i, h == 0 ? 0 : 2 * h - 1);
+                const R v = mrt_even(i) ? sp[h] : dp[h];
                 if (c == 1) m += v;
                 else if (c == -1) m -= v;
                 else if (c != 0) m += R(c) * v;
             }
-            dm[i] = rates[i] * m;  // rates[] already divided by |M_i|^2
+            dm[i] = p.rate[i] * m;  // rates[] already divided by |M_i|^2
         }
 #pragma unroll
-        for (int p = 0; p <= Q / 2; ++p) {
-            const int k = p == 0 ? 0 : 2 * p - 1;
+        for (int h = 0; h <= Q / 2; ++h) {
+            const int k = h == 0 ? 0 : 2 * h - 1;
             R ev = R(0), od = R(0);
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
@@ -276,7 +512,7 @@ __device__ __forceinline__ void collide(R (&g)[Q], const Par<R> &p, const R *rat
                 if (mrt_even(i)) ev += t;
                 else od += t;
             }
-            if (p == 0) {
+            if (h == 0) {
                 g[0] -= ev;
             } else {
                 g[k] -= ev + od;
@@ -285,6 +521,32 @@ __device__ __forceinline__ void collide(R (&g)[Q], const Par<R> &p, const R *rat
         }
     }
 }
+
+template <int COLL, int STORE, typename R>
+__device__ __forceinline__ void relax(R (&g)[Q], const CollPar<R> &c, R &drho, R &ux, R &uy, R &uz)
+{
+    static_assert(STORE != ST_F64 || COLL != COLL_SRT, "FP64 SRT runs as TRT");
+    if constexpr (COLL == COLL_TRT) relax_pairs(g, c, drho, ux, uy, uz);
+    else if constexpr (COLL == COLL_MRT && !kStochastic<STORE>) relax_rows(g, c, drho, ux, uy, uz);
+    else relax_plain<COLL>(g, c, drho, ux, uy, uz);
+}
+// The combinations of relax_rows against the rows of M.
+constexpr bool mrt_combinations_hold()
+{
+    for (int k = 0; k < Q; ++k) {
+        const int x = ex(k), y = ey(k), z = ez(k), n2 = speed2(k);
+        const int A = n2 == 1, D = n2 == 2, xy = D && !z, xz = D && !y, yz = D && !x;
+        const int x9 = A * (2 * x * x - y * y - z * z), w9 = xy + xz - 2 * yz;
+        const int x11 = A * (y * y - z * z), w11 = xy - xz;
+        const int m[Q] = {1, -30 * (n2 == 0) - 11 * A + 8 * D, 12 * (n2 == 0) - 4 * A + D, x, x * (D - 4 * A), y,
+                          y * (D - 4 * A), z, z * (D - 4 * A), x9 + w9, -2 * x9 + w9, x11 + w11, -2 * x11 + w11,
+                          x * y, y * z, x * z, x * (xy - xz), y * (yz - xy), z * (xz - yz)};
+        for (int i = 0; i < Q; ++i)
+            if (m[i] != mrt_m(i, k)) return false;
+    }
+    return true;
+}
+static_assert(mrt_combinations_hold(), "the combinations of relax_rows are the rows of M");
 
 // Periodic wrap of c + d into [0, n) for |d| <= 2 (any n >= 1).
 __device__ __forceinline__ int wrap2(int c, int n)
@@ -336,10 +598,10 @@ __device__ __forceinline__ R wall_neighbour_terms(const Par<R> &P, int wall, con
         int xv2, xv3;
         uint32_t c2, c3;
         link_neighbours(P, cell, k, c2, xv2, c3, xv3);
-        const R b2 = shifted(S::load(fs + ((uint32_t)k * P.ks + c2), P.isc), xv2, (int)P.nx,
-                             R(weight(k)) * P.dshift);
-        const R p3 = shifted(S::load(fs + ((uint32_t)kb * P.ks + c3), P.isc), xv3, (int)P.nx,
-                             R(weight(kb)) * P.dshift);
+        const R b2 = shifted(S::cvt(__ldg(fs + ((uint32_t)k * P.ks + c2))), xv2, (int)P.nx,
+                             R(weight(k)) * P.c.dshift);
+        const R p3 = shifted(S::cvt(__ldg(fs + ((uint32_t)kb * P.ks + c3))), xv3, (int)P.nx,
+                             R(weight(kb)) * P.c.dshift);
         v = fma_r(ld_keep(lw + LW_ALPHA, keep), g[kb], v);
         v = fma_r(ld_keep(lw + LW_BETA, keep), p3, v);
         v = fma_r(ld_keep(lw + LW_DELTA, keep), b2, v);
@@ -352,7 +614,7 @@ __device__ __forceinline__ R wall_neighbour_terms(const Par<R> &P, int wall, con
         for (int m = 1; m < Q; ++m) {
             const int d = ex(kb) * ex(m) + ey(kb) * ey(m) + ez(kb) * ez(m);
             if (d == 0) continue;
-            const R gm = S::load(fs + ((uint32_t)m * P.ks + c2), P.isc);
+            const R gm = S::cvt(__ldg(fs + ((uint32_t)m * P.ks + c2)));
             j2 += d > 0 ? (d == 1 ? gm : R(d) * gm) : (d == -1 ? -gm : R(d) * gm);
         }
         v = fma_r(ld_keep(lw + LW_ZETA, keep), j2, v);
@@ -375,7 +637,7 @@ __device__ __forceinline__ R wall_own_part_w(const Par<R> &P, const R *lw, int k
     if (X != R(0)) {
         const R eu = R(ex(kb)) * ux + R(ey(kb)) * uy + R(ez(kb)) * uz;
         const R uu = ux * ux + uy * uy + uz * uz;
-        const R fst = drho + P.rho0 * (ld_keep(lw + LW_THETA, keep) * eu + R(4.5) * eu * eu - R(1.5) * uu);
+        const R fst = drho + P.c.rho0 * (ld_keep(lw + LW_THETA, keep) * eu + R(4.5) * eu * eu - R(1.5) * uu);
         sv = fma_r(X * R(weight(kb)), fst, sv);
     }
     return sv;
@@ -396,7 +658,7 @@ __device__ __forceinline__ R wall_own_part_w(const Par<R> &P, const R *lw, int k
 // imported populations) gets these slots from wall_prepare_kernel.
 // Walls in the AA layout: the same, with S where the AA layout's pull reads (see above).
 template <int COLL, int STORE, int KIND, bool RED, bool WX, typename R>
-__device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], const Par<R> &P, const R *rates,
+__device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], const Par<R> &P,
                                             uint32_t cell, uint32_t xf,
                                             bool inner, const uint32_t *pull_off, const uint32_t *push_off,
                                             uint32_t wm, uint32_t off, const typename Store<STORE>::T *fs,
@@ -427,7 +689,7 @@ __device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], con
                 else if constexpr (KIND == KIND_AA_PULL) ci = (uint32_t)k * KS + cell;
                 else ci = (uint32_t)kb * KS + coord_of(P, cell).pull(k);
                 C = checked(I, ci - (KIND == KIND_AA_PULL ? (uint32_t)k : (uint32_t)kb) * KS, I.n32)
-                        ? S::cvt(ld_pop<KIND>(fs + ci), P.isc)
+                        ? S::cvt(ld_pop<KIND>(fs + ci))
                         : R(0);
             }
             g[k] = v;
@@ -441,45 +703,48 @@ __device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], con
     }
 
     R drho, ux, uy, uz;
-    moments(g, P.irho0, drho, ux, uy, uz);
+    relax<COLL, STORE>(g, P.c, drho, ux, uy, uz);
     if constexpr (RED) {
-        rd = drho;
+        const R unit = STORE == ST_F16 ? R(P.isc) : R(1);  // FP16: from the stored units
+        rd = drho * unit;
         rx = ux;
         ry = uy;
         rz = uz;
         const R uu = ux * ux + uy * uy + uz * uz;
         if (!(uu < R(1)) || !(drho == drho)) atomicOr(status, STATUS_DIVERGED);
+        for (int d = 0; d < 3; ++d) fm[d] *= unit;
     }
 
-    collide<COLL, R>(g, P, rates, drho, ux, uy, uz);
-
-    // 16-bit formats round stochastically (see Store); wider formats round to nearest
-    constexpr bool sr = sizeof(T) == 2;
-    const uint32_t h = sr ? cell_hash(cell) : 0u;
-    T packed[Q];
-#pragma unroll
-    for (int k = 0; k < Q; ++k)
-        packed[k] = sr ? S::pack_sr(g[k], P.sc, round_bits(h, k, float(g[k]))) : S::pack(g[k], P.sc);
+    // 16-bit formats round stochastically (put2); wider formats to nearest
+    const RoundKey key = round_key<STORE>(cell, P.hash_off);
     if constexpr (KIND == KIND_AA_PULL) {
         if (push_off) {  // interior cell: x + e_k is cell + e_k, except across the x faces
             const uint32_t cxm = (xf & 1u) ? P.nx : 0u, cxp = (xf & 2u) ? P.nx : 0u;
-#pragma unroll
-            for (int k = 0; k < Q; ++k) {
+            auto at = [&](int k) {
                 uint32_t idx = cell + push_off[k];
                 if (ex(k) == 1) idx -= cxp;
                 if (ex(k) == -1) idx += cxm;
-                if (checked(I, idx - (uint32_t)k * KS, I.n32)) fd[idx] = packed[k];
-            }
+                return idx;
+            };
+            auto ok = [&](int k) { return checked(I, at(k) - (uint32_t)k * KS, I.n32); };
+            if (ok(0)) put1<STORE>(fd + at(0), g[0], key, 0);
+#pragma unroll
+            for (int k = 1; k < Q; k += 2)
+                if (ok(k) && ok(k + 1)) put2<STORE>(fd + at(k), fd + at(k + 1), g[k], g[k + 1], key, k, k + 1);
         } else {
             const Coord co = coord_of(P, cell);
+            put1<STORE>(fd + co.push(0), g[0], key, 0);
 #pragma unroll
-            for (int k = 0; k < Q; ++k) fd[(uint32_t)k * KS + co.push(k)] = packed[k];
+            for (int k = 1; k < Q; k += 2)
+                put2<STORE>(fd + ((uint32_t)k * KS + co.push(k)), fd + ((uint32_t)(k + 1) * KS + co.push(k + 1)), g[k],
+                            g[k + 1], key, k, k + 1);
         }
     } else {
+        put1<STORE>(fd + cell, g[0], key, 0);
 #pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            if constexpr (KIND == KIND_AB) fd[(uint32_t)k * KS + cell] = packed[k];
-            else fd[(uint32_t)opp(k) * KS + cell] = packed[k];
+        for (int k = 1; k < Q; k += 2) {  // A-B: slot k; AA: slot kbar
+            const int ka = KIND == KIND_AB ? k : k + 1, kb = KIND == KIND_AB ? k + 1 : k;
+            put2<STORE>(fd + ((uint32_t)ka * KS + cell), fd + ((uint32_t)kb * KS + cell), g[k], g[k + 1], key, k, k + 1);
         }
     }
     if constexpr (KIND == KIND_AA_PULL) {
@@ -492,7 +757,7 @@ __device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], con
                 const uint32_t l = off + __popc(wm & ((1u << k) - 1u));
                 const R cq = P.wall == 1 ? ld_keep(linkc + l, l2_keep_policy()) : R(0);
                 const R sv = wall_own_part(P.wall, cq, g[opp(k)], g[k]);
-                fd[(uint32_t)k * KS + cell] = sr ? S::pack_sr(sv, P.sc, round_bits(h, k, float(sv))) : S::pack(sv, P.sc);
+                put1<STORE>(fd + ((uint32_t)k * KS + cell), sv, key, k);
             }
         }
     }
@@ -526,8 +791,7 @@ __device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], con
                 } else {
                     idx = d * KS + co.pull(k);
                 }
-                if (checked(I, idx - d * KS, I.n32))
-                    fd[idx] = sr ? S::pack_sr(sv, P.sc, round_bits(h, k, float(sv))) : S::pack(sv, P.sc);
+                if (checked(I, idx - d * KS, I.n32)) put1<STORE>(fd + idx, sv, key, k);
             }
         }
     }
@@ -607,7 +871,7 @@ template <typename R> struct RedAcc {
 // crossed the x boundary, walls, collision, stores; with RED, add the lane's moments and
 // momentum exchange to acc.
 template <int COLL, int STORE, int KIND, bool RED, bool WX, typename R>
-__device__ __forceinline__ void finish_item(const InstanceDev &I, const Par<R> &P, const R *rates,
+__device__ __forceinline__ void finish_item(const InstanceDev &I, const Par<R> &P,
                                             const typename Store<STORE>::T (&raw)[Q], const WarpItem &it, int lane,
                                             const typename Store<STORE>::T *fs, typename Store<STORE>::T *fd,
                                             unsigned *status, RedAcc<R> &acc)
@@ -617,23 +881,23 @@ __device__ __forceinline__ void finish_item(const InstanceDev &I, const Par<R> &
     if (it.cell == 0xFFFFFFFFu) return;
     R g[Q];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) g[k] = S::cvt(raw[k], P.isc);
+    for (int k = 0; k < Q; ++k) g[k] = S::cvt(raw[k]);
     // pressure shift of the pulls that crossed the x boundary (wall directions take their
     // value from the wall rule instead)
     const uint32_t wm = it.wm;
     if (it.xf & 1u) {
 #pragma unroll
         for (int k = 0; k < Q; ++k)
-            if (ex(k) == 1 && !((wm >> k) & 1u)) g[k] += R(weight(k)) * P.dshift;
+            if (ex(k) == 1 && !((wm >> k) & 1u)) g[k] += R(weight(k)) * P.c.dshift;
     }
     if (it.xf & 2u) {
 #pragma unroll
         for (int k = 0; k < Q; ++k)
-            if (ex(k) == -1 && !((wm >> k) & 1u)) g[k] -= R(weight(k)) * P.dshift;
+            if (ex(k) == -1 && !((wm >> k) & 1u)) g[k] -= R(weight(k)) * P.c.dshift;
     }
     R rd = R(0), rx = R(0), ry = R(0), rz = R(0);
     R fm[3] = {R(0), R(0), R(0)};
-    finish_cell<COLL, STORE, KIND, RED, WX, R>(I, g, P, rates, it.cell, it.xf, it.inner, I.pull_off,
+    finish_cell<COLL, STORE, KIND, RED, WX, R>(I, g, P, it.cell, it.xf, it.inner, I.pull_off,
                                                it.inner ? I.push_off : nullptr, wm, it.off, fs, fd,
                                                reinterpret_cast<const R *>(I.linkc),
                                                reinterpret_cast<const R *>(I.linkw), status, rd, rx, ry, rz, fm);
@@ -702,17 +966,6 @@ __device__ __forceinline__ void reduce_tile(const RedAcc<R> &acc, double *partia
     }
 }
 
-template <int COLL, typename R> __device__ __forceinline__ void load_rates(const InstanceDev &I, R (&rates)[Q])
-{
-    if constexpr (COLL == COLL_MRT) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            if constexpr (sizeof(R) == sizeof(float)) rates[i] = I.rate_f[i];
-            else rates[i] = I.rate_d[i];
-        }
-    }
-}
-
 // Programmatic dependent launch (sm_90 and later): a step lets the next step's blocks be
 // scheduled as soon as all of its own blocks are running, and a step waits for the
 // previous one to complete (with its memory visible) only before its first population
@@ -772,8 +1025,6 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
     }
     const InstanceDev &I = instance_of<BATCH>(table, one, tile.inst);
     const Par<R> P = load_par<R>(I);
-    R rates[Q];
-    load_rates<COLL>(I, rates);
     const T *fs;  // state read this step
     T *fd;        // state written this step
     if constexpr (KIND == KIND_AB) {
@@ -791,7 +1042,7 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
     T raw[Q];
     pull_item<STORE, KIND, R>(I, P, fs, it, raw);
     RedAcc<R> acc{};
-    finish_item<COLL, STORE, KIND, RED, WX, R>(I, P, rates, raw, it, lane, fs, fd, status + tile.inst, acc);
+    finish_item<COLL, STORE, KIND, RED, WX, R>(I, P, raw, it, lane, fs, fd, status + tile.inst, acc);
     if constexpr (RED) reduce_tile(acc, I.partials, tile.local);
 }
 

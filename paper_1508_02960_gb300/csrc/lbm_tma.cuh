@@ -112,8 +112,6 @@ __global__ void __launch_bounds__(kBrickCells, tma_min_blocks<STORE>())
     }
     __syncthreads();
     const Par<R> P = load_par<R>(I);
-    R rates[Q];
-    load_rates<COLL>(I, rates);
     const int cur = I.phase ^ flip;
     const T *fs = reinterpret_cast<const T *>(cur ? I.f1 : I.f0);
     T *fd = reinterpret_cast<T *>(cur ? I.f0 : I.f1);
@@ -223,7 +221,7 @@ __global__ void __launch_bounds__(kBrickCells, tma_min_blocks<STORE>())
         const WarpItem now = meta;
         if (brick + (int)gridDim.x < nbricks) locate(brick + (int)gridDim.x, meta);
         RedAcc<R> acc{};
-        finish_item<COLL, STORE, KIND_AB, false, WX, R>(I, P, rates, raw, now, cx, fs, fd, nullptr, acc);
+        finish_item<COLL, STORE, KIND_AB, false, WX, R>(I, P, raw, now, cx, fs, fd, nullptr, acc);
     }
 }
 
