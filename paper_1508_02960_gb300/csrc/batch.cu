@@ -742,7 +742,7 @@ Launch Batch::shaped_launch(const StepShape &sh, int kind) const
     while (w < kShapeWarpsN && kShapeWarps[w] != sh.warps) ++w;
     (void)kind;
     const int nt = nwtiles_[w];
-    return Launch{d_table_, d_wtiles_[w], nt, sh.warps, std::max(1, nt), sh.warps * 32, stream_, &maps_[w]};
+    return Launch{d_table_, d_wtiles_[w], nt, sh.warps, std::max(1, nt), sh.warps * 32, stream_, sms_, &maps_[w]};
 }
 
 // Every other step takes its tiles from the last to the first, so that it begins with the
@@ -779,7 +779,7 @@ lbm_status Batch::graph_for(long long m, bool red, const StepShape &sh, int wx, 
         graphs_.erase(lru);
     }
     StepQueue q{&ops(),
-                Launch{d_table_, d_stiles_, nstiles_, kTileSegs, grid_, kStepWarps * 32, stream_, &maps_[0]},
+                Launch{d_table_, d_stiles_, nstiles_, kTileSegs, grid_, kStepWarps * 32, stream_, sms_, &maps_[0]},
                 {shaped_launch(sh, layout_ == LBM_LAYOUT_AB ? KIND_AB : KIND_AA_PULL),
                  shaped_launch(sh, KIND_AA_LOCAL)},
                 sh.warps,

@@ -13,11 +13,11 @@
 namespace lbm {
 namespace detail {
 
-// Launch of a step kernel with programmatic stream serialisation: the kernel may start
-// (up to its wait on the previous step) while the previous kernel of the stream is still
-// running.  Captured into a graph, this becomes a programmatic dependency edge.
+// Launch of a step kernel.  overlap: with programmatic stream serialisation, the kernel may
+// start (up to its wait on the previous step) while the previous kernel of the stream is still
+// running; captured into a graph, this becomes a programmatic dependency edge.
 template <typename... P, typename... A>
-cudaError_t launch_step(void (*kernel)(P...), const Launch &L, A &&...args)
+cudaError_t launch_step(void (*kernel)(P...), const Launch &L, bool overlap, A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)L.grid);
@@ -28,7 +28,7 @@ cudaError_t launch_step(void (*kernel)(P...), const Launch &L, A &&...args)
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
@@ -39,13 +39,21 @@ template <int STORE, int COLL, int KIND, bool RED, bool WX, int WARPS>
 cudaError_t step_red(const Launch &L, int flip, unsigned *status, const InstanceDev *one)
 {
     cudaError_t e;
+    // A grid that the multiprocessors hold at once starts after the previous step has ended:
+    // launched into it, its blocks are placed around the running ones, several to one
+    // multiprocessor and none to another, and the step takes as long as the fullest one (FP64
+    // 24^3 29.4 us overlapped, 10.0 after; 48^3 30.4 / 24.2; FP32 AA 32^3 5.2 / 3.7, 64^3
+    // 7.0 / 6.3).  A larger grid refills every multiprocessor as it goes, and overlapping its
+    // start hides the launch (FP32 AA 96^3 11.9 / 12.1, 80^3 8.3 both; FP64 80^3 87.0 / 87.3).
+    constexpr int resident = STORE == ST_F64 ? 16 : step_min_blocks<STORE, COLL, RED, WX, WARPS, KIND>() * WARPS;
+    const bool overlap = (long long)L.grid * WARPS > (long long)L.sms * resident;
     if (one) {  // a single instance: parameters travel in the constant bank
-        e = launch_step(step_kernel<COLL, STORE, KIND, false, RED, WX, WARPS>, L, L.table, *one, NoBatchMap{}, L.tiles,
+        e = launch_step(step_kernel<COLL, STORE, KIND, false, RED, WX, WARPS>, L, overlap, L.table, *one, NoBatchMap{}, L.tiles,
                         L.ntiles, flip, status);
     } else {  // a batch: parameters from the device table, the tiles' instances from the map
         static const InstanceDev unused{};
         static const BatchMap no_map{};  // n = 0: tile records
-        e = launch_step(step_kernel<COLL, STORE, KIND, true, RED, WX, WARPS>, L, L.table, unused,
+        e = launch_step(step_kernel<COLL, STORE, KIND, true, RED, WX, WARPS>, L, overlap, L.table, unused,
                         L.map ? *L.map : no_map, L.tiles, L.ntiles, flip, status);
     }
     if (e != cudaSuccess) return e;

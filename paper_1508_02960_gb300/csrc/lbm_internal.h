@@ -36,6 +36,7 @@ struct Launch {
     int chunk_segs;
     int grid, block;
     cudaStream_t stream;
+    int sms = 0;                    // multiprocessors of the device (step launches)
     const BatchMap *map = nullptr;  // a batched step launch: its tiles' instances (n = 0: none)
 };
 

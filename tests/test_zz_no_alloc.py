@@ -94,3 +94,65 @@ def test_noalloc_rejects_oversized_and_bad_arguments(capi):
     assert "limit" in capi.last_error()
     assert L.lbm_moment_sums_f64_noalloc(None, None, 8, 1.0, buf.data_ptr(), None) == capi.ERR_ARG
     assert L.lbm_moment_sums_f64_noalloc(buf.data_ptr(), None, 0, 1.0, buf.data_ptr(), None) == capi.ERR_ARG
+
+
+@pytest.mark.parametrize("n", [1, 31, 255, 257, 311_296, 311_297, 400_003])
+@pytest.mark.parametrize("kind", ["flow", "tiny", "huge", "uneven", "signed"])
+def test_noalloc_integer_sums(capi, n, kind):
+    """The fixed-point sums at the edges of a block's rounds and of the block count, on values
+    far from 1 (scaled by 1e-280, summed in FP64, and 1e+200), on cells of very different
+    sizes side by side, and on signed values, against exact sums (math.fsum).  Tolerance: an
+    FP64 sum of each cell's 19 values rounds at 2^-53 of their sum at most 18 times; 19 * 2^-53
+    of the sum of the absolute values bounds it, and the sums over the cells are no worse."""
+    import math
+
+    import torch
+    rng = np.random.default_rng(n)
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+    f = w[:, None] * (1.0 + 1e-3 * rng.uniform(-1, 1, size=(19, n)))
+    rho0 = 1.0
+    if kind == "tiny":
+        f, rho0 = f * 1e-300, 1e-300
+    elif kind == "huge":
+        f, rho0 = f * 1e200, 1.25e200
+    elif kind == "uneven":
+        f = f * 2.0 ** rng.integers(-30, 30, size=n)
+    elif kind == "signed":
+        f = f * rng.choice([-1.0, 1.0], size=(19, n)) * 2.0 ** rng.integers(-8, 8, size=(19, n))
+    solid = (rng.uniform(size=n) < 0.25).astype(np.uint8)
+    solid[0] = 0
+    fl = f[:, solid == 0]
+    e = np.array([[0, 0, 0], [1, 0, 0], [-1, 0, 0], [0, 1, 0], [0, -1, 0], [0, 0, 1], [0, 0, -1],
+                  [1, 1, 0], [-1, -1, 0], [1, -1, 0], [-1, 1, 0], [1, 0, 1], [-1, 0, -1], [1, 0, -1],
+                  [-1, 0, 1], [0, 1, 1], [0, -1, -1], [0, 1, -1], [0, -1, 1]])
+    ref = [math.fsum(fl.ravel().tolist() + [-rho0] * fl.shape[1])]
+    ref += [math.fsum((fl[e[:, a] == 1]).ravel().tolist() + (-fl[e[:, a] == -1]).ravel().tolist()) / rho0
+            for a in range(3)]
+    out = torch.full((4,), float("nan"), dtype=torch.float64, device="cuda")
+    fd, sd = torch.from_numpy(f).cuda(), torch.from_numpy(solid).cuda()
+    capi.moment_sums_f64_noalloc(fd.data_ptr(), sd.data_ptr(), n, rho0, out.data_ptr(), torch.cuda.current_stream())
+    got = out.cpu().numpy()
+    size = np.abs(fl).sum() + rho0 * fl.shape[1]
+    for d in range(4):
+        assert abs(got[d] - ref[d]) <= 19 * 2.0 ** -53 * (size if d == 0 else np.abs(fl).sum() / rho0), (d, got, ref)
+
+
+def test_noalloc_sums_of_infinities_and_nan(capi):
+    import torch
+    f = np.full((19, 300), 0.05)
+    solid = np.zeros(300, dtype=np.uint8)
+    for bad, at in ((np.inf, 17), (np.nan, 299)):
+        g = f.copy()
+        g[1, at] = bad
+        for masked in (False, True):
+            solid[:] = 0
+            solid[at] = masked
+            out = torch.zeros(4, dtype=torch.float64, device="cuda")
+            fd, sd = torch.from_numpy(g).cuda(), torch.from_numpy(solid).cuda()
+            capi.moment_sums_f64_noalloc(fd.data_ptr(), sd.data_ptr(), 300, 1.0, out.data_ptr(),
+                                         torch.cuda.current_stream())
+            got = out.cpu().numpy()
+            if masked:  # a solid cell's entries are ignored
+                assert np.isfinite(got).all()
+            else:       # direction 1 moves along x: the density and x sums take it over
+                assert not np.isfinite(got[:2]).any() and np.isfinite(got[2:]).all()
