@@ -356,7 +356,7 @@ LBM_API lbm_status lbm_synchronize(lbm_ctx *ctx);
  *   cuda_stream  stream the two kernels are queued on (NULL = legacy default stream)
  * Calls no cudaMalloc or cudaFree: block sums go to a fixed 256 KiB scratch array inside
  * the library, held by every GPU that loads it.  n_cells is limited to 268,435,456
- * (8192 blocks of 32768 cells); larger fields return LBM_ERR_ARG.  The first call on
+ * (32768 times the 8192 slots); larger fields return LBM_ERR_ARG.  The first call on
  * each device looks up the scratch address (cudaGetSymbolAddress) and should come before
  * any stream capture.  The address is kept, per device ordinal, for the life of the
  * process: after cudaDeviceReset on a device it is stale, so a process that resets a

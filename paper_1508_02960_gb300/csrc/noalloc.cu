@@ -26,46 +26,197 @@ namespace {
 
 constexpr int kNoAllocMaxBlocks = 8192;      // scratch slots: 8192 * 4 doubles = 256 KiB
 constexpr int kNoAllocThreads = 256;
-constexpr long long kNoAllocCellsPerBlock = 32768;  // fixed cells per block: 128 per thread
-constexpr long long kNoAllocMaxCells = (long long)kNoAllocMaxBlocks * kNoAllocCellsPerBlock;
+constexpr long long kNoAllocMaxCells = (long long)kNoAllocMaxBlocks * 32768;
 
 static __device__ __align__(256) double g_noalloc_partials[kNoAllocMaxBlocks * 4];
 
-// Block b sums cells [b * kNoAllocCellsPerBlock, ...) of the fluid cells: threads stride
-// over the range in a fixed order, then a fixed tree; partial -> partials[b].
-__global__ void __launch_bounds__(kNoAllocThreads) noalloc_partials_kernel(const double *__restrict__ f,
+// Blocks of a call: 8 to a multiprocessor (its full complement of threads), each over one
+// contiguous range of whole rounds of its threads; small fields take a round a block.  Fixed
+// by the cell count alone, so that the order of the sums is.
+constexpr long long kNoAllocBlocks = 152 * 8;
+__host__ __device__ inline long long noalloc_cells_per_block(long long n)
+{
+    return ((n + kNoAllocBlocks - 1) / kNoAllocBlocks + kNoAllocThreads - 1) / kNoAllocThreads * kNoAllocThreads;
+}
+
+// Fixed-point sums.  A cell's 19 values, the largest of which has the exponent field E, are
+// taken as integers in units of 2^(E - 1080): 1.52-bit mantissas at bit 57 and
+// below, so that 19 of them fit 63 bits and values down to 2^-5 of the largest power lose
+// nothing (equilibrium populations span 2^4).  Smaller ones are truncated below 2^-57 of it,
+// where an FP64 sum of the cell would round at 2^-53.
+constexpr int kFixedTop = 57;
+
+struct FixedSum {           // sum = hi 2^32 + lo, as the sums of the halves of the terms
+    long long hi;
+    unsigned long long lo;
+    __device__ __forceinline__ void add(long long x)
+    {
+        lo += (unsigned long long)(unsigned)x;
+        hi += x >> 32;
+    }
+};
+
+__device__ __forceinline__ double to_double(__int128 t)
+{
+    return (double)(long long)(t >> 64) * 18446744073709551616.0 + (double)(unsigned long long)t;
+}
+
+// Sums of m cells held in units of exponent field E, as FP64: .v[0] = sum rho - m rho0,
+// .v[1..3] = sum j.  Out of line: rare in a warp's loop, once at the end of a block.
+struct Sums4 {
+    double v[4];
+};
+__device__ __noinline__ Sums4 to_sums(FixedSum s0, FixedSum s1, FixedSum s2, FixedSum s3, int E, unsigned m,
+                                      double rho0)
+{
+    Sums4 a = {};
+    if (m == 0) return a;
+    const double unit = __longlong_as_double((long long)(E - kFixedTop) << 52);
+    auto whole = [](const FixedSum &s) { return ((__int128)s.hi << 32) + (__int128)s.lo; };
+    const double r = rho0 / unit;  // rho0 in units: its whole part is taken off exactly
+    if (r < 4.6e18) {
+        const long long w = (long long)r;
+        a.v[0] = (to_double(whole(s0) - (__int128)w * m) - (r - (double)w) * m) * unit;
+    } else {
+        a.v[0] = to_double(whole(s0)) * unit - rho0 * m;
+    }
+    a.v[1] = to_double(whole(s1)) * unit;
+    a.v[2] = to_double(whole(s2)) * unit;
+    a.v[3] = to_double(whole(s3)) * unit;
+    return a;
+}
+
+// Block b sums its range of the fluid cells; partial -> partials[b].  Bound: one read of the
+// field.  The sums are integer sums because FP64 arithmetic is slow on GB300 (a warp
+// instruction per 19 cycles a multiprocessor): the 49 FP64 additions of a cell would take four
+// times as long as its loads, the 340 integer instructions they become take 0.8 of it.
+// 160^3 cells, 43 % of them solid at random: 1044 us with FP64 sums in 125 blocks of fixed
+// size -> 160 us.  Values out of the integers' reach (infinities, NaN, a cell's
+// largest value below 2^-959) are summed in FP64.
+__global__ void __launch_bounds__(kNoAllocThreads, 2) noalloc_partials_kernel(const double *__restrict__ f,
                                                                           const uint8_t *__restrict__ solid,
                                                                           long long n, double rho0,
                                                                           double *__restrict__ partials)
 {
-    __shared__ double sm[kNoAllocThreads][4];
-    const long long c0 = (long long)blockIdx.x * kNoAllocCellsPerBlock;
-    const long long c1 = c0 + kNoAllocCellsPerBlock < n ? c0 + kNoAllocCellsPerBlock : n;
+    __shared__ double sm[kNoAllocThreads / 32][4];
+    __shared__ FixedSum fs[kNoAllocThreads / 32][4];
+    __shared__ unsigned cnt[kNoAllocThreads / 32];
+    __shared__ int exps[kNoAllocThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long per = noalloc_cells_per_block(n);
+    const long long c0 = (long long)blockIdx.x * per, c1 = c0 + per < n ? c0 + per : n;
     double a[4] = {0.0, 0.0, 0.0, 0.0};
-    for (long long c = c0 + threadIdx.x; c < c1; c += kNoAllocThreads) {
-        if (solid && solid[c]) continue;
-        double rho = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
+    FixedSum s[4] = {};
+    unsigned m = 0;
+    int Ecur = 0;  // exponent field of s (0: none yet)
+    for (long long cw = c0 + warp * 32; cw < c1; cw += kNoAllocThreads) {
+        const long long c = cw + lane;
+        const bool live = c < c1 && !(solid && solid[c]);
+        unsigned long long v[Q];
 #pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            const double v = f[(long long)k * n + c];
-            rho += v;
-            jx += ex(k) * v;
-            jy += ey(k) * v;
-            jz += ez(k) * v;
+        for (int k = 0; k < Q; ++k)
+            v[k] = live ? __ldg(reinterpret_cast<const unsigned long long *>(f) + ((long long)k * n + c)) : 0ull;
+        unsigned top = 0u;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) top = max(top, (unsigned)(v[k] >> 32) & 0x7ff00000u);
+        const int E = (int)(top >> 20);
+        if (E >= 64 && E < 0x7ff) {
+            if (E != Ecur) {
+                const Sums4 w = to_sums(s[0], s[1], s[2], s[3], Ecur, m, rho0);
+                for (int d = 0; d < 4; ++d) a[d] += w.v[d];
+                for (int d = 0; d < 4; ++d) s[d] = FixedSum{0, 0ull};
+                m = 0;
+                Ecur = E;
+            }
+            long long x[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                const unsigned hi = (unsigned)(v[k] >> 32), lo = (unsigned)v[k];
+                const unsigned sh = (unsigned)(E + 62 - kFixedTop) - ((hi >> 20) & 0x7ffu);
+                const unsigned mh = (__funnelshift_l(lo, hi, 10) & 0x3fffffffu) | 0x40000000u;
+                unsigned long long t = (unsigned long long)mh << 32 | (unsigned long long)(lo << 10);
+                asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(t), "r"(sh));  // 0 from 64 on
+                const long long sg = (long long)v[k] >> 63;
+                const long long q = ((long long)t ^ sg) - sg;
+                x[0] += q;
+                if (ex(k)) x[1] += ex(k) > 0 ? q : -q;
+                if (ey(k)) x[2] += ey(k) > 0 ? q : -q;
+                if (ez(k)) x[3] += ez(k) > 0 ? q : -q;
+            }
+            for (int d = 0; d < 4; ++d) s[d].add(x[d]);
+            ++m;
+        } else if (live) {
+            double x[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                const double g = __longlong_as_double((long long)v[k]);
+                x[0] += g;
+                if (ex(k)) x[1] += ex(k) > 0 ? g : -g;
+                if (ey(k)) x[2] += ey(k) > 0 ? g : -g;
+                if (ez(k)) x[3] += ez(k) > 0 ? g : -g;
+            }
+            a[0] += x[0] - rho0;
+            for (int d = 1; d < 4; ++d) a[d] += x[d];
         }
-        a[0] += rho - rho0;
-        a[1] += jx / rho0;
-        a[2] += jy / rho0;
-        a[3] += jz / rho0;
     }
-    for (int d = 0; d < 4; ++d) sm[threadIdx.x][d] = a[d];
+    // the warp's sums, then the block's: in integers where they have one unit, as they have in
+    // a flow, whose largest population (at rest, about 1/3 rho0) keeps its exponent
+    const int Etop = (int)__reduce_max_sync(0xffffffffu, (unsigned)Ecur);
+    if (!__all_sync(0xffffffffu, m == 0 || Ecur == Etop)) {
+        const Sums4 w = to_sums(s[0], s[1], s[2], s[3], Ecur, m, rho0);
+        for (int d = 0; d < 4; ++d) {
+            a[d] += w.v[d];
+            s[d] = FixedSum{0, 0ull};
+        }
+        m = 0;
+    }
+    Ecur = Etop;
+    for (int o = 16; o > 0; o >>= 1) {
+        m += __shfl_xor_sync(0xffffffffu, m, o);
+        for (int d = 0; d < 4; ++d) {
+            s[d].hi += __shfl_xor_sync(0xffffffffu, s[d].hi, o);
+            s[d].lo += __shfl_xor_sync(0xffffffffu, s[d].lo, o);
+        }
+    }
+    bool any = false;
+    for (int d = 0; d < 4; ++d) any |= a[d] != 0.0;  // (NaN too)
+    if (__any_sync(0xffffffffu, any))
+        for (int d = 0; d < 4; ++d)
+            for (int o = 16; o > 0; o >>= 1) a[d] += __shfl_xor_sync(0xffffffffu, a[d], o);
+    if (lane == 0) {
+        for (int d = 0; d < 4; ++d) {
+            sm[warp][d] = a[d];
+            fs[warp][d] = s[d];
+        }
+        cnt[warp] = m;
+        exps[warp] = Ecur;
+    }
     __syncthreads();
-    for (int w = kNoAllocThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int d = 0; d < 4; ++d) sm[threadIdx.x][d] += sm[threadIdx.x + w][d];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double b[4] = {0.0, 0.0, 0.0, 0.0};
+        FixedSum t[4] = {};
+        unsigned mt = 0;
+        int Et = 0;
+        for (int w = 0; w < kNoAllocThreads / 32; ++w) {
+            if (cnt[w] > 0 && exps[w] != Et) {
+                const Sums4 v = to_sums(t[0], t[1], t[2], t[3], Et, mt, rho0);
+                for (int d = 0; d < 4; ++d) b[d] += v.v[d];
+                for (int d = 0; d < 4; ++d) t[d] = FixedSum{0, 0ull};
+                mt = 0;
+                Et = exps[w];
+            }
+            for (int d = 0; d < 4; ++d) {
+                t[d].hi += fs[w][d].hi;
+                t[d].lo += fs[w][d].lo;
+                b[d] += sm[w][d];
+            }
+            mt += cnt[w];
+        }
+        const Sums4 v = to_sums(t[0], t[1], t[2], t[3], Et, mt, rho0);
+        for (int d = 0; d < 4; ++d) b[d] += v.v[d];
+        partials[(long long)blockIdx.x * 4] = b[0];
+        for (int d = 1; d < 4; ++d) partials[(long long)blockIdx.x * 4 + d] = b[d] / rho0;
     }
-    if (threadIdx.x < 4) partials[(long long)blockIdx.x * 4 + threadIdx.x] = sm[0][threadIdx.x];
 }
 
 // One block: out[d] = sum over blocks of partials[b][d], in a fixed order.
@@ -129,7 +280,8 @@ extern "C" lbm_status lbm_moment_sums_f64_noalloc(const double *f_dev, const uin
     lbm_status st = noalloc_scratch(&scratch);
     if (st != LBM_OK) return st;
     const cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const int nblocks = (int)((n_cells + kNoAllocCellsPerBlock - 1) / kNoAllocCellsPerBlock);
+    const long long per = noalloc_cells_per_block(n_cells);
+    const int nblocks = (int)((n_cells + per - 1) / per);
     noalloc_partials_kernel<<<nblocks, kNoAllocThreads, 0, s>>>(f_dev, solid_dev, (long long)n_cells, rho0, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "no-allocation moment sums (partials)");
