@@ -383,6 +383,10 @@ static void fill_dev(const Instance &in, InstanceDev &D)
     D.bmask = in.geo.bmask;
     D.boff = in.geo.boff;
     D.linkc = in.geo.linkc;
+    D.linkr = in.geo.linkr;
+    D.ilinkr = in.geo.ilinkr;
+    D.ilinkc = in.geo.ilinkc;
+    D.ilink = in.geo.ilink;
     D.linkw = in.geo.linkw;
     D.partials = in.partials;
     D.ncells = in.geo.ncells;

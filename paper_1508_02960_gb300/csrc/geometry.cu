@@ -149,22 +149,18 @@ __global__ void fluid_scatter_kernel(long long n, const uint4 *__restrict__ seg,
     }
 }
 
-// The step kernels' per-lane work-list entries, one warp per work item w (its cells
-// icell[32w .. 32w+31] in cell order, padding lanes 0xFFFFFFFF), so that a step finds what
-// it needs of a cell without a dependent load or a division: flane[32w + l] = {x, y},
+// The step kernels' work-list entries, one warp per work item w (its cells icell[32w ..
+// 32w+31] in cell order, padding lanes 0xFFFFFFFF), so that a step finds what it needs of a
+// cell without a dependent load or a division: flane[32w + l] = {x, y},
 //   x: the cell (bits 0-27; cells < 2^28 since 19 direction strides fit 32 bits), bit 28
 //      x = 0, bit 29 x = nx - 1 (the pulls and pushes that cross the x faces), bit 30 every
 //      cell of the item away from the y and z faces (the same in all its lanes);
 //      0xFFFFFFFF for a padding lane;
-//   y: bits 0-18 the wall mask (bit k: x - e_k solid), bits 19-31 the cell's first link
-//      minus the item's first link;
-// and fwarp[w] = {boundary bits of the lanes, the item's first link (0 when it has no
-// boundary cell)}.  Links are numbered in cell order, and an item's cells lie within
-// kItemSpan + 1 consecutive cells of at most 18 links each, so the offset fits 13 bits.
-static_assert(18 * (kItemSpan + 1) < (1 << 13), "link offset field of the work-list entries");
+//   y: the wall mask (bit k: x - e_k solid).
+// count[w] = number of cut links of the item's cells.
 __global__ void flane_kernel(long long nw, int nx, int ny, int nz, const uint32_t *__restrict__ icell,
                              const uint4 *__restrict__ seg, const uint32_t *__restrict__ bmask,
-                             const uint32_t *__restrict__ boff, uint2 *__restrict__ fwarp, uint2 *__restrict__ flane)
+                             uint2 *__restrict__ flane, unsigned long long *__restrict__ count)
 {
     const int lane = threadIdx.x & 31;
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -172,26 +168,59 @@ __global__ void flane_kernel(long long nw, int nx, int ny, int nz, const uint32_
         const uint32_t c = icell[w * 32 + lane];
         const bool live = c != 0xFFFFFFFFu;
         const uint4 m = live ? seg[c >> 5] : make_uint4(0u, 0u, 0u, 0u);
-        const bool bnd = live && ((m.y >> (c & 31u)) & 1u);
-        uint32_t wm = 0u, off = 0u;
-        if (bnd) {  // the boundary table lists boundary cells in cell order
-            const uint32_t b = m.z + __popc(m.y & ((1u << (c & 31u)) - 1u));
-            wm = bmask[b];
-            off = boff[b];
-        }
-        const unsigned bb = __ballot_sync(0xffffffffu, bnd);
-        const uint32_t base = bb ? __shfl_sync(0xffffffffu, off, __ffs(bb) - 1) : 0u;
-        uint32_t ex = 0xFFFFFFFFu;
+        uint32_t wm = 0u;
+        if (live && ((m.y >> (c & 31u)) & 1u))  // the boundary table lists boundary cells in cell order
+            wm = bmask[m.z + __popc(m.y & ((1u << (c & 31u)) - 1u))];
+        const unsigned links = __reduce_add_sync(0xffffffffu, (unsigned)__popc(wm));
+        uint32_t ce = 0xFFFFFFFFu;
         bool in_yz = true;
         if (live) {
             const uint32_t x = c % (uint32_t)nx, yz = c / (uint32_t)nx;
             const uint32_t y = yz % (uint32_t)ny, z = yz / (uint32_t)ny;
-            ex = c | (x == 0 ? 1u << 28 : 0u) | (x == (uint32_t)nx - 1u ? 1u << 29 : 0u);
+            ce = c | (x == 0 ? 1u << 28 : 0u) | (x == (uint32_t)nx - 1u ? 1u << 29 : 0u);
             in_yz = y >= 1 && y + 2 <= (uint32_t)ny && z >= 1 && z + 2 <= (uint32_t)nz;
         }
-        if (__all_sync(0xffffffffu, in_yz) && live) ex |= 1u << 30;
-        flane[w * 32 + lane] = make_uint2(ex, wm | ((bnd ? off - base : 0u) << 19));
-        if (lane == 0) fwarp[w] = make_uint2(bb, base);
+        if (__all_sync(0xffffffffu, in_yz) && live) ce |= 1u << 30;
+        flane[w * 32 + lane] = make_uint2(ce, wm);
+        if (lane == 0) count[w] = links;
+    }
+}
+
+// The links of the work items, item by item (an item's cells may have other items' between
+// them): fwarp[w] = {the item's links, the first of them}, and for link i of this order
+// ilinkr[i] = k | lane << 8, ilinkc[i] its CLI coefficient and, where
+// given, ilink[i] its index in cell order (linkw's).
+template <typename R>
+__global__ void item_links_kernel(long long nw, const uint2 *__restrict__ flane,
+                                  const uint4 *__restrict__ seg, const uint32_t *__restrict__ boff,
+                                  const unsigned long long *__restrict__ base, const R *__restrict__ linkc,
+                                  uint2 *__restrict__ fwarp, uint16_t *__restrict__ ilinkr, R *__restrict__ ilinkc,
+                                  uint32_t *__restrict__ ilink)
+{
+    const int lane = threadIdx.x & 31;
+    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+    for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nw; w += warps) {
+        const uint2 e = flane[w * 32 + lane];
+        const uint32_t n = (uint32_t)__popc(e.y);
+        uint32_t at = n;  // inclusive sum over the lanes
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += v;
+        }
+        const uint32_t first = (uint32_t)base[w], total = __shfl_sync(0xffffffffu, at, 31);
+        if (lane == 0) fwarp[w] = make_uint2(total, first);
+        if (n == 0) continue;
+        at += first - n;
+        const uint32_t c = e.x & 0x0FFFFFFFu;
+        const uint4 m = seg[c >> 5];
+        uint32_t l = boff[m.z + __popc(m.y & ((1u << (c & 31u)) - 1u))];
+        for (int k = 1; k < Q; ++k) {
+            if (!((e.y >> k) & 1u)) continue;
+            ilinkr[at] = (uint16_t)(k | lane << 8);
+            ilinkc[at] = linkc[l];
+            if (ilink) ilink[at] = l;
+            ++at, ++l;
+        }
     }
 }
 
@@ -199,7 +228,7 @@ __global__ void flane_kernel(long long nw, int nx, int ny, int nz, const uint32_
 // box segment of 32 cells that are all fluid is an item of its own: aligned to 128-byte
 // lines, each of its loads and stores touches one line (two for the directions with
 // e_kx != 0).  The fluid cells of the other segments are packed 32 to an item in cell
-// order, an item spanning at most kItemSpan + 1 cells (the link-offset field above).  On
+// order, an item spanning at most kItemSpan + 1 cells.  On
 // the r = 60 sphere cell this cuts the cache lines a step touches by a fifth at the same
 // number of items, where 32 consecutive fluid cells to an item straddle two lines almost
 // always.
@@ -352,7 +381,8 @@ __global__ void link_kernel(long long nb, int nx, int ny, int nz, const double4 
                             const double *__restrict__ qfield, const uint8_t *__restrict__ solid,
                             const uint32_t *__restrict__ bmask, const uint32_t *__restrict__ boff,
                             const long long *__restrict__ bcell, double *__restrict__ linkq, R *__restrict__ linkc,
-                            unsigned long long *__restrict__ ncli, int wall, double tau, R *__restrict__ linkw)
+                            unsigned long long *__restrict__ ncli, int wall, double tau, R *__restrict__ linkw,
+                            uint16_t *__restrict__ linkr)
 {
     const long long n = (long long)nx * ny * nz;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nb;
@@ -402,6 +432,7 @@ __global__ void link_kernel(long long nb, int nx, int ny, int nz, const double4 
             const double cq = f2 ? __ddiv_rn(__dsub_rn(1.0, 2.0 * q), __dadd_rn(1.0, 2.0 * q)) : 0.0;
             linkq[l] = q;
             linkc[l] = (R)cq;
+            linkr[l] = (uint16_t)(k | (int)(c & 31) << 8);
             if (linkw) {  // x_f3 = x + 2 e_k
                 const int x3 = (x + 2 * ex(k) + 2 * nx) % nx, y3 = (y + 2 * ey(k) + 2 * ny) % ny,
                           z3 = (z + 2 * ez(k) + 2 * nz) % nz;
@@ -520,6 +551,10 @@ void free_geometry(GeometryDev *g)
     cudaFree(g->bcell);
     cudaFree(g->linkq);
     cudaFree(g->linkc);
+    cudaFree(g->linkr);
+    cudaFree(g->ilinkr);
+    cudaFree(g->ilinkc);
+    cudaFree(g->ilink);
     cudaFree(g->linkw);
     *g = GeometryDev();
 }
@@ -552,6 +587,7 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
     double *d_q = nullptr;
     uint32_t *d_wm = nullptr, *d_icell = nullptr;  // d_icell: the work items' cells, [32 n_fwarps_padded]
     unsigned long long *d_cnt = nullptr, *d_base = nullptr, *d_nl = nullptr, *d_lbase = nullptr, *d_ctr = nullptr;
+    unsigned long long *d_icnt = nullptr, *d_ibase = nullptr;
     unsigned long long h_ctr[2] = {0ull, 0ull};
     unsigned long long h_last[2];
     *g = GeometryDev();
@@ -662,6 +698,10 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
         if (g->n_links > 0) {
             GEO_CHECK(dev_alloc(&g->linkq, sizeof(double) * g->n_links));
             GEO_CHECK(dev_alloc(&g->linkc, (c_double ? 8 : 4) * g->n_links));
+            GEO_CHECK(dev_alloc(&g->linkr, sizeof(uint16_t) * g->n_links));
+            GEO_CHECK(dev_alloc(&g->ilinkr, sizeof(uint16_t) * g->n_links));
+            GEO_CHECK(dev_alloc(&g->ilinkc, (c_double ? 8 : 4) * g->n_links));
+            if (wall >= 2) GEO_CHECK(dev_alloc(&g->ilink, sizeof(uint32_t) * g->n_links));
             if (wall >= 2) GEO_CHECK(dev_alloc(&g->linkw, (c_double ? 8 : 4) * kLinkW * g->n_links));
             if (q_host && !(spheres && n_spheres > 0)) {
                 GEO_CHECK(dev_alloc(&d_q, sizeof(double) * Q * n));
@@ -672,20 +712,32 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
                 link_kernel<double><<<grid_for(nb, 128), 128, 0, s>>>(nb, nx, ny, nz, sp, n_spheres, d_q, g->solid,
                                                                       g->bmask, g->boff, g->bcell, g->linkq,
                                                                       (double *)g->linkc, d_ctr + 1, wall, tau,
-                                                                      (double *)g->linkw);
+                                                                      (double *)g->linkw, g->linkr);
             else
                 link_kernel<float><<<grid_for(nb, 128), 128, 0, s>>>(nb, nx, ny, nz, sp, n_spheres, d_q, g->solid,
                                                                      g->bmask, g->boff, g->bcell, g->linkq,
                                                                      (float *)g->linkc, d_ctr + 1, wall, tau,
-                                                                     (float *)g->linkw);
+                                                                     (float *)g->linkw, g->linkr);
             GEO_CHECK(cudaGetLastError());
         }
     }
-    // per-lane entries of the step kernels' work list (needs the boundary table's links)
+    // the step kernels' work list: per-lane entries, then the items' links (boundary table and
+    // coefficients are there)
     GEO_CHECK(dev_alloc(&g->flane, sizeof(uint2) * 32 * g->n_fwarps_padded));
+    GEO_CHECK(dev_alloc(&d_icnt, sizeof(unsigned long long) * g->n_fwarps_padded));
+    GEO_CHECK(dev_alloc(&d_ibase, sizeof(unsigned long long) * g->n_fwarps_padded));
     flane_kernel<<<grid_for(g->n_fwarps_padded * 32, 256), 256, 0, s>>>(g->n_fwarps_padded, nx, ny, nz, d_icell,
-                                                                          g->seg, g->bmask, g->boff, g->fwarp,
-                                                                          g->flane);
+                                                                          g->seg, g->bmask, g->flane, d_icnt);
+    GEO_CHECK(cudaGetLastError());
+    GEO_CHECK(exclusive_scan(d_icnt, d_ibase, g->n_fwarps_padded, s));
+    if (c_double)
+        item_links_kernel<double><<<grid_for(g->n_fwarps_padded * 32, 256), 256, 0, s>>>(
+            g->n_fwarps_padded, g->flane, g->seg, g->boff, d_ibase, (const double *)g->linkc, g->fwarp,
+            g->ilinkr, (double *)g->ilinkc, g->ilink);
+    else
+        item_links_kernel<float><<<grid_for(g->n_fwarps_padded * 32, 256), 256, 0, s>>>(
+            g->n_fwarps_padded, g->flane, g->seg, g->boff, d_ibase, (const float *)g->linkc, g->fwarp,
+            g->ilinkr, (float *)g->ilinkc, g->ilink);
     GEO_CHECK(cudaGetLastError());
     GEO_CHECK(cudaMemcpyAsync(h_ctr, d_ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost, s));
     GEO_CHECK(cudaStreamSynchronize(s));
@@ -694,7 +746,8 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
     g->bytes = n + sizeof(uint4) * (g->nseg_padded + g->n_active_padded) + sizeof(uint32_t) * g->n_fcell_padded +
                (sizeof(uint2) * 32 + sizeof(uint2)) * g->n_fwarps_padded +
                (sizeof(uint32_t) * 2 + sizeof(long long)) * g->n_boundary +
-               (sizeof(double) + (c_double ? 8 : 4) * (wall >= 2 ? 1 + kLinkW : 1)) * g->n_links;
+               (sizeof(double) + 2 * sizeof(uint16_t) + (wall >= 2 ? sizeof(uint32_t) : 0) +
+                (c_double ? 8 : 4) * (wall >= 2 ? 2 + kLinkW : 2)) * g->n_links;
 
     cudaFree(d_sph);
     cudaFree(d_q);
@@ -705,6 +758,8 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
     cudaFree(d_lbase);
     cudaFree(d_ctr);
     cudaFree(d_icell);
+    cudaFree(d_icnt);
+    cudaFree(d_ibase);
     return cudaSuccess;
 fail:
     cudaStreamSynchronize(s);
@@ -717,6 +772,8 @@ fail:
     cudaFree(d_lbase);
     cudaFree(d_ctr);
     cudaFree(d_icell);
+    cudaFree(d_icnt);
+    cudaFree(d_ibase);
     free_geometry(g);
     return e == cudaSuccess ? cudaErrorUnknown : e;
 }

@@ -288,16 +288,17 @@ enum { STATUS_DIVERGED = 1u, STATUS_TIMEOUT = 2u, STATUS_BOUNDS = 4u };
 // fcell[j] is the j-th fluid cell in cell order (the state kernels' list).  The step kernels
 // take work items of one warp each (geometry.cu, pack_items): a box segment whose 32 cells
 // are all fluid, or up to 32 fluid cells of partly solid segments in cell order, the lanes
-// after an item's last cell padding.  For item w: fwarp[w].x bit l set when lane l's cell is
-// a boundary cell, fwarp[w].y the index of the item's first link; flane[32w + l] = {x, y}:
-// x the cell (bits 0-27) with bit 28 x = 0, bit 29 x = nx - 1, bit 30 all the item's cells
-// away from the y and z faces (0xFFFFFFFF: padding lane); y the wall mask (bits 0-18, as
-// bmask below, 0 for other cells) and the cell's first link - fwarp[w].y (bits 19-31), so
-// that a step needs no dependent load and no division to find a cell's walls and its
-// periodic fix-ups.
+// after an item's last cell padding.  For item w: flane[32w + l] = {x, y}: x the cell (bits
+// 0-27) with bit 28 x = 0, bit 29 x = nx - 1, bit 30 all the item's cells away from the y and
+// z faces (0xFFFFFFFF: padding lane); y the wall mask (as bmask below, 0 for other cells).
+// The cut links again in item order (an item's cells may have other items' between them):
+// fwarp[w] = {the item's links, the first of them}, ilinkr[i] = k | lane << 8, ilinkc[i] = its
+// linkc, ilink[i] = its index in cell order.  So a step needs no
+// dependent load and no division to find a cell's walls and its periodic fix-ups.
 // Boundary cell b: bmask[b] bit k set when x - e_k is solid (the pull of direction k hits
 // the wall), boff[b] the index of its first link; its links are ordered by k.  Link l:
-// linkc[l] = CLI coefficient (1-2q)/(1+2q) (0 where CLI falls back to SBB).
+// linkc[l] = CLI coefficient (1-2q)/(1+2q) (0 where CLI falls back to SBB), linkr[l] = k | the
+// cell's lane in its segment << 8.
 // ------------------------------------------------------------------------------------
 
 // Constants of the collision as the step kernels use them, computed on the host so that no
@@ -334,7 +335,7 @@ template <> struct CollPar<double> {
     double rate[Q];         // MRT: s_i / |M_i|^2
 };
 
-struct InstanceDev {
+struct alignas(16) InstanceDev {
     void *f0, *f1;           // populations [19][ks] (direction k at k * ks); AA uses f0 only
     const uint4 *seg;        // [nseg]
     const uint4 *aseg;       // [n_active_padded]: seg entries of segments holding fluid, .w = segment
@@ -344,6 +345,10 @@ struct InstanceDev {
     const uint32_t *bmask;   // [n_boundary]
     const uint32_t *boff;    // [n_boundary]
     const void *linkc;       // [n_links], type R
+    const uint16_t *linkr;   // [n_links]
+    const uint16_t *ilinkr;  // [n_links]
+    const void *ilinkc;      // [n_links], type R
+    const uint32_t *ilink;   // [n_links] (walls >= LBM_LIBB), else NULL
     const void *linkw;       // [n_links][kLinkW], type R (walls >= LBM_LIBB), else NULL
     double *partials;        // [n_tiles of this instance][kRedSlots]
     long long ncells;

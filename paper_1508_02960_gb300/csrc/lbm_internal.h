@@ -98,14 +98,18 @@ struct GeometryDev {
     uint32_t *fcell = nullptr;     // [n_fcell_padded] fluid cells in cell order (pad 0xFFFFFFFF)
     long long n_fcell = 0, n_fcell_padded = 0;
     uint2 *flane = nullptr;        // [32 n_fwarps_padded] the step work items' cells with their
-                                   // wall masks, link offsets and face flags (lbm_device.cuh)
-    uint2 *fwarp = nullptr;        // [n_fwarps_padded] per work item: boundary bits, first link
+                                   // wall masks and face flags (lbm_device.cuh)
+    uint2 *fwarp = nullptr;        // [n_fwarps_padded] per work item: links, first link
     long long n_fwarps = 0, n_fwarps_padded = 0;
     uint32_t *bmask = nullptr;     // [n_boundary]
     uint32_t *boff = nullptr;      // [n_boundary]
     long long *bcell = nullptr;    // [n_boundary] cell index of each boundary cell
     double *linkq = nullptr;       // [n_links] wall distance q (FP64)
     void *linkc = nullptr;         // [n_links] CLI coefficient, compute type
+    uint16_t *linkr = nullptr;     // [n_links] direction and lane in its segment
+    uint16_t *ilinkr = nullptr;    // [n_links] in work-item order: direction and lane
+    void *ilinkc = nullptr;        // [n_links] ... the CLI coefficient, compute type
+    uint32_t *ilink = nullptr;     // [n_links] ... the link (walls >= LBM_LIBB)
     void *linkw = nullptr;         // [n_links][kLinkW] rule coefficients (LIBB, QIBB, IEBB, MR)
     size_t bytes = 0;
 };

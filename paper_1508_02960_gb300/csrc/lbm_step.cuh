@@ -55,14 +55,11 @@ template <int KIND, typename T> __device__ __forceinline__ T ld_pop(const T *p)
     else return *p;
 }
 
-// The step kernel uses no dynamic shared memory.
-inline size_t step_smem_bytes(int, int) { return 0; }
-
 // Instance parameters held in registers for the duration of a chunk.
 template <typename R> struct Par {
     uint32_t ks, nx, ny, nz;
     FastDiv dnx, dny;
-    CollPar<R> c;
+    const CollPar<R> &c;  // read where it is used
     float isc;
     uint32_t hash_off;
     int wall;
@@ -76,18 +73,8 @@ template <typename R> __device__ __forceinline__ const CollPar<R> &coll_par(cons
 
 template <typename R> __device__ __forceinline__ Par<R> load_par(const InstanceDev &I)
 {
-    Par<R> p;
-    p.ks = I.ks;
-    p.nx = I.nx;
-    p.ny = I.ny;
-    p.nz = I.nz;
-    p.dnx = I.div_nx;
-    p.dny = I.div_ny;
-    p.c = coll_par<R>(I);
-    p.isc = I.inv_scale;
-    p.hash_off = I.cf.hash_off;
-    p.wall = I.wall;
-    return p;
+    return Par<R>{I.ks,      (uint32_t)I.nx, (uint32_t)I.ny, (uint32_t)I.nz, I.div_nx,
+                  I.div_ny,  coll_par<R>(I), I.inv_scale,    I.cf.hash_off,  I.wall};
 }
 
 // Cell coordinates with the periodic x-1/x/x+1 offsets, row offsets y-1/y/y+1 and plane
@@ -143,6 +130,12 @@ __device__ __forceinline__ double ld_keep(const double *a, uint64_t pol)
 {
     double v;
     asm("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(a), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_keep(const uint16_t *a, uint64_t pol)
+{
+    unsigned short v;
+    asm("ld.global.nc.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(a), "l"(pol));
     return v;
 }
 __device__ __forceinline__ uint2 ld_keep(const uint2 *a, uint64_t pol)
@@ -578,150 +571,96 @@ __device__ __forceinline__ void link_neighbours(const Par<R> &P, uint32_t cell, 
 
 // Population of direction m read at a virtual x coordinate: the pressure shift of a value
 // that crossed an x face (Sec. 2.2.2, as for the pulls).
-template <typename R> __device__ __forceinline__ R shifted(R v, int xv, int nx, R w_dshift)
+template <typename R> __device__ __forceinline__ R shifted(R v, int xv, int nx, R w, R dshift)
 {
-    return xv < 0 ? v + w_dshift : (xv >= nx ? v - w_dshift : v);
+    return xv < 0 ? fma_r(w, dshift, v) : (xv >= nx ? fma_r(-w, dshift, v) : v);
 }
 
 // The neighbour terms alpha P2 + beta P3 + delta B2 + zeta J2 of an interpolated wall rule
-// (kLinkW) of link (x, kbar), x - e_k solid, added to v (which holds S).  The loads the
-// rule may need are issued before its coefficients arrive (a coefficient of 0 -- a
-// fallback -- multiplies a finite value read from a solid cell's slot).
+// (kLinkW) of link (x, kbar), x - e_k solid, added to v (which holds S); p2 is the cell's
+// ordinary pull of direction kbar.  The loads the rule may need are issued before its
+// coefficients arrive (a coefficient of 0 -- a fallback -- multiplies a finite value read
+// from a solid cell's slot).
 template <int STORE, typename R>
-__device__ __forceinline__ R wall_neighbour_terms(const Par<R> &P, int wall, const R *lw, int k, uint32_t cell,
-                                                  const R (&g)[Q], const typename Store<STORE>::T *fs, R v)
+__device__ __forceinline__ R wall_neighbour_terms(const Par<R> &P, int wall, const R *lw, int k, uint32_t cell, R p2,
+                                                  const typename Store<STORE>::T *fs, R v)
 {
     using S = Store<STORE>;
-    const int kb = opp(k);
+    const int kb = opp_rt(k);
     const uint64_t keep = l2_keep_policy();
     if (wall == 3 || wall == 5) {  // QIBB, MR: P3 = g~_kbar(x_f3), B2 = g~_k(x_f2)
         int xv2, xv3;
         uint32_t c2, c3;
         link_neighbours(P, cell, k, c2, xv2, c3, xv3);
-        const R b2 = shifted(S::cvt(__ldg(fs + ((uint32_t)k * P.ks + c2))), xv2, (int)P.nx,
-                             R(weight(k)) * P.c.dshift);
-        const R p3 = shifted(S::cvt(__ldg(fs + ((uint32_t)kb * P.ks + c3))), xv3, (int)P.nx,
-                             R(weight(kb)) * P.c.dshift);
-        v = fma_r(ld_keep(lw + LW_ALPHA, keep), g[kb], v);
+        const R w = k < 7 ? R(weight(1)) : R(weight(7));
+        const R b2 = shifted(S::cvt(__ldg(fs + ((uint32_t)k * P.ks + c2))), xv2, (int)P.nx, w, P.c.dshift);
+        const R p3 = shifted(S::cvt(__ldg(fs + ((uint32_t)kb * P.ks + c3))), xv3, (int)P.nx, w, P.c.dshift);
+        v = fma_r(ld_keep(lw + LW_ALPHA, keep), p2, v);
         v = fma_r(ld_keep(lw + LW_BETA, keep), p3, v);
         v = fma_r(ld_keep(lw + LW_DELTA, keep), b2, v);
     } else if (wall == 4) {  // IEBB: J2 = e_kbar . (momentum of x_f2); the shift carries none
         int xv2, xv3;
         uint32_t c2, c3;
         link_neighbours(P, cell, k, c2, xv2, c3, xv3);
+        const int x = -ex_rt(k), y = -ey_rt(k), z = -ez_rt(k);
         R j2 = R(0);
 #pragma unroll
         for (int m = 1; m < Q; ++m) {
-            const int d = ex(kb) * ex(m) + ey(kb) * ey(m) + ez(kb) * ez(m);
-            if (d == 0) continue;
-            const R gm = S::cvt(__ldg(fs + ((uint32_t)m * P.ks + c2)));
-            j2 += d > 0 ? (d == 1 ? gm : R(d) * gm) : (d == -1 ? -gm : R(d) * gm);
+            const int d = x * ex(m) + y * ey(m) + z * ez(m);
+            if (d != 0) j2 = fma_r(R(d), S::cvt(__ldg(fs + ((uint32_t)m * P.ks + c2))), j2);
         }
         v = fma_r(ld_keep(lw + LW_ZETA, keep), j2, v);
     } else {  // LIBB
-        v = fma_r(ld_keep(lw + LW_ALPHA, keep), g[kb], v);
+        v = fma_r(ld_keep(lw + LW_ALPHA, keep), p2, v);
     }
     return v;
 }
 
 // The own-cell part S of an interpolated wall rule (kLinkW) from the cell's post-collision
-// values g[] and its moments drho, u at this step.
+// values B = g~_k, C = g~_kbar and its moments drho, u at this step.
 template <typename R>
-__device__ __forceinline__ R wall_own_part_w(const Par<R> &P, const R *lw, int k, const R (&g)[Q], R drho, R ux, R uy,
-                                             R uz)
+__device__ __forceinline__ R wall_own_part_w(const Par<R> &P, const R *lw, int k, R B, R C, R drho, R ux, R uy, R uz)
 {
-    const int kb = opp(k);
     const uint64_t keep = l2_keep_policy();
-    R sv = fma_r(ld_keep(lw + LW_GAMMA, keep), g[k], ld_keep(lw + LW_EPS, keep) * g[kb]);
+    R sv = fma_r(ld_keep(lw + LW_GAMMA, keep), B, ld_keep(lw + LW_EPS, keep) * C);
     const R X = ld_keep(lw + LW_X, keep);
     if (X != R(0)) {
-        const R eu = R(ex(kb)) * ux + R(ey(kb)) * uy + R(ez(kb)) * uz;
+        const R eu = R(-ex_rt(k)) * ux + R(-ey_rt(k)) * uy + R(-ez_rt(k)) * uz;
         const R uu = ux * ux + uy * uy + uz * uz;
         const R fst = drho + P.c.rho0 * (ld_keep(lw + LW_THETA, keep) * eu + R(4.5) * eu * eu - R(1.5) * uu);
-        sv = fma_r(X * R(weight(kb)), fst, sv);
+        sv = fma_r(X * (k < 7 ? R(weight(1)) : R(weight(7))), fst, sv);
     }
     return sv;
 }
 
-// Process one cell whose 19 pulled populations are in g[] (already shifted, except the
-// wall directions): walls, moments, collision, stores.  When RED is set, returns the
-// moments through rd..rz and the momentum the cell's wall links hand to the solid in this
-// step through fm[3]: a link (x, kbar) with x - e_k solid carries g~_kbar(x) into the wall
-// and brings the new g_k back, so the solid gains e_kbar (g~_kbar(x) + g_k).  (Deviations
-// suffice: the 2 w rho0 of full populations sums to zero over a periodic domain.)
-//
-// Walls in the A-B layout.  The pull of a wall direction k reads slot k of the solid cell
-// x - e_k, which no fluid cell owns; every step leaves there the own-cell part S of the
-// wall rule for the next step (wall_own_part, from its post-collision values in
-// registers), so SBB needs no wall code at all and CLI adds c g_kbar^in, g_kbar^in being
-// the cell's ordinary pull from x_f2 = x + e_k.  A state set from outside (initial state,
-// imported populations) gets these slots from wall_prepare_kernel.
-// Walls in the AA layout: the same, with S where the AA layout's pull reads (see above).
-template <int COLL, int STORE, int KIND, bool RED, bool WX, typename R>
-__device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], const Par<R> &P,
-                                            uint32_t cell, uint32_t xf,
-                                            bool inner, const uint32_t *pull_off, const uint32_t *push_off,
-                                            uint32_t wm, uint32_t off, const typename Store<STORE>::T *fs,
-                                            typename Store<STORE>::T *fd, const R *linkc, const R *linkw,
-                                            unsigned *status, R &rd, R &rx, R &ry, R &rz, R (&fm)[3])
+// Pressure shift of the pulls that crossed the x boundary (wall directions take their value
+// from the wall rule instead).
+template <typename R> __device__ __forceinline__ void pressure_shift(R (&g)[Q], const Par<R> &P, uint32_t xf, uint32_t wm)
 {
-    using S = Store<STORE>;
-    using T = typename S::T;
-    const uint32_t KS = P.ks;
-    if (wm) {
+    if (xf & 1u) {
 #pragma unroll
-        for (int k = 1; k < Q; ++k) {
-            if (!((wm >> k) & 1u)) continue;
-            const int kb = opp(k);
-            const uint32_t l = off + __popc(wm & ((1u << k) - 1u));
-            const R cq = P.wall == 1 ? ld_keep(linkc + l, l2_keep_policy()) : R(0);
-            R v, C;
-            v = g[k];  // S, left by the previous step where this pull reads
-            if (WX && KIND == KIND_AB && P.wall >= 2)
-                v = wall_neighbour_terms<STORE>(P, P.wall, linkw + (size_t)l * kLinkW, k, cell, g, fs, v);
-            else if (cq != R(0)) v = fma_r(cq, g[kb], v);
-            if constexpr (RED) {
-                // the own post-collision g~_kbar(x) of the previous step (momentum exchange):
-                // A-B: own slot kbar; AA after a LOCAL step: own slot k; AA after a PULL
-                // step: where it was pushed, slot kbar of x - e_k
-                uint32_t ci;
-                if constexpr (KIND == KIND_AB) ci = (uint32_t)kb * KS + cell;
-                else if constexpr (KIND == KIND_AA_PULL) ci = (uint32_t)k * KS + cell;
-                else ci = (uint32_t)kb * KS + coord_of(P, cell).pull(k);
-                C = checked(I, ci - (KIND == KIND_AA_PULL ? (uint32_t)k : (uint32_t)kb) * KS, I.n32)
-                        ? S::cvt(ld_pop<KIND>(fs + ci))
-                        : R(0);
-            }
-            g[k] = v;
-            if constexpr (RED) {  // e_kbar = -e_k
-                const R m = C + v;
-                if (ex(k)) fm[0] += ex(k) > 0 ? -m : m;
-                if (ey(k)) fm[1] += ey(k) > 0 ? -m : m;
-                if (ez(k)) fm[2] += ez(k) > 0 ? -m : m;
-            }
-        }
+        for (int k = 0; k < Q; ++k)
+            if (ex(k) == 1 && !((wm >> k) & 1u)) g[k] += R(weight(k)) * P.c.dshift;
     }
-
-    R drho, ux, uy, uz;
-    relax<COLL, STORE>(g, P.c, drho, ux, uy, uz);
-    if constexpr (RED) {
-        const R unit = STORE == ST_F16 ? R(P.isc) : R(1);  // FP16: from the stored units
-        rd = drho * unit;
-        rx = ux;
-        ry = uy;
-        rz = uz;
-        const R uu = ux * ux + uy * uy + uz * uz;
-        if (!(uu < R(1)) || !(drho == drho)) atomicOr(status, STATUS_DIVERGED);
-        for (int d = 0; d < 3; ++d) fm[d] *= unit;
+    if (xf & 2u) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+            if (ex(k) == -1 && !((wm >> k) & 1u)) g[k] -= R(weight(k)) * P.c.dshift;
     }
+}
 
-    // 16-bit formats round stochastically (put2); wider formats to nearest
-    const RoundKey key = round_key<STORE>(cell, P.hash_off);
+// Stores of one cell's post-collision values: A-B slot k, AA LOCAL slot kbar of the cell, AA
+// PULL slot k of x + e_k.
+template <int STORE, int KIND, typename R>
+__device__ __forceinline__ void store_cell(const InstanceDev &I, const Par<R> &P, const R (&g)[Q], uint32_t cell,
+                                           uint32_t xf, bool inner, RoundKey key, typename Store<STORE>::T *fd)
+{
+    const uint32_t KS = P.ks;
     if constexpr (KIND == KIND_AA_PULL) {
-        if (push_off) {  // interior cell: x + e_k is cell + e_k, except across the x faces
+        if (inner) {  // interior cell: x + e_k is cell + e_k, except across the x faces
             const uint32_t cxm = (xf & 1u) ? P.nx : 0u, cxp = (xf & 2u) ? P.nx : 0u;
             auto at = [&](int k) {
-                uint32_t idx = cell + push_off[k];
+                uint32_t idx = cell + I.push_off[k];
                 if (ex(k) == 1) idx -= cxp;
                 if (ex(k) == -1) idx += cxm;
                 return idx;
@@ -740,59 +679,14 @@ __device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], con
                             g[k + 1], key, k, k + 1);
         }
     } else {
+        // AA LOCAL: the slots the pull read; their addresses are computed again here, not kept
+        // in 38 registers since (kept, the step spilled 196 bytes at 56 registers)
+        asm volatile("" : "+r"(cell));
         put1<STORE>(fd + cell, g[0], key, 0);
 #pragma unroll
-        for (int k = 1; k < Q; k += 2) {  // A-B: slot k; AA: slot kbar
+        for (int k = 1; k < Q; k += 2) {
             const int ka = KIND == KIND_AB ? k : k + 1, kb = KIND == KIND_AB ? k + 1 : k;
             put2<STORE>(fd + ((uint32_t)ka * KS + cell), fd + ((uint32_t)kb * KS + cell), g[k], g[k + 1], key, k, k + 1);
-        }
-    }
-    if constexpr (KIND == KIND_AA_PULL) {
-        // the own-cell part of every wall rule into the own slot k, which the next (LOCAL)
-        // step's pull of direction k reads
-        if (wm) {
-#pragma unroll
-            for (int k = 1; k < Q; ++k) {
-                if (!((wm >> k) & 1u)) continue;
-                const uint32_t l = off + __popc(wm & ((1u << k) - 1u));
-                const R cq = P.wall == 1 ? ld_keep(linkc + l, l2_keep_policy()) : R(0);
-                const R sv = wall_own_part(P.wall, cq, g[opp(k)], g[k]);
-                put1<STORE>(fd + ((uint32_t)k * KS + cell), sv, key, k);
-            }
-        }
-    }
-    if constexpr (KIND != KIND_AA_PULL) {
-        // A-B, and AA LOCAL steps: the own-cell part of every wall rule into the solid slot
-        // the next step's pull of direction k reads (A-B: slot k of x - e_k in the other
-        // buffer; AA: slot kbar of x - e_k)
-        if (wm) {
-            const uint32_t cxm = (xf & 1u) ? P.nx : 0u, cxp = (xf & 2u) ? P.nx : 0u;
-            Coord co;
-            if (!inner) co = coord_of(P, cell);
-#pragma unroll
-            for (int k = 1; k < Q; ++k) {
-                if (!((wm >> k) & 1u)) continue;
-                const uint32_t l = off + __popc(wm & ((1u << k) - 1u));
-                R sv;
-                if (WX && P.wall >= 2) {
-                    sv = wall_own_part_w(P, linkw + (size_t)l * kLinkW, k, g, drho, ux, uy, uz);
-                } else {
-                    const R cq = P.wall == 1 ? ld_keep(linkc + l, l2_keep_policy()) : R(0);
-                    sv = wall_own_part(P.wall, cq, g[opp(k)], g[k]);
-                }
-                // the slot direction: k in A-B, kbar in AA (pull_off of an AA instance
-                // addresses slot kbar of x - e_k)
-                const uint32_t d = KIND == KIND_AB ? (uint32_t)k : (uint32_t)opp(k);
-                uint32_t idx;
-                if (inner) {
-                    idx = cell + pull_off[k];
-                    if (ex(k) == 1) idx += cxm;
-                    if (ex(k) == -1) idx -= cxp;
-                } else {
-                    idx = d * KS + co.pull(k);
-                }
-                if (checked(I, idx - d * KS, I.n32)) put1<STORE>(fd + idx, sv, key, k);
-            }
         }
     }
 }
@@ -802,31 +696,196 @@ __device__ __forceinline__ void finish_cell(const InstanceDev &I, R (&g)[Q], con
 struct WarpItem {
     uint32_t cell;     // this lane's cell (0xFFFFFFFF: padding lane)
     uint32_t xf;       // bit 0: x = 0, bit 1: x = nx - 1 (pulls and pushes across the x faces)
-    uint32_t wm, off;  // boundary cell: wall mask (bit k: x - e_k solid) and first link; else 0
-    uint2 wd;          // tiles: the warp's entry (.y its first link); bricks: y and z of the cell
-    bool inner;        // every lane away from the y and z faces
+    uint32_t wm;       // boundary cell: wall mask (bit k: x - e_k solid); else 0
+    bool inner;        // every live lane away from the y and z faces (padding lanes: undefined)
 };
 
-// Locate one work item: this lane's cell, its x-face flags, wall mask and links, and
-// whether every lane is away from the y and z faces, all precomputed in the work list (one
-// entry per warp and one per lane, no dependent load and no division), which no step writes.
+// Walls.  The pull of a wall direction k reads, in the A-B layout, slot k of the solid cell
+// x - e_k, which no fluid cell owns; every step leaves there the own-cell part S of the wall
+// rule for the next step (wall_own_part, from its post-collision values in registers), so
+// SBB needs no wall code before the collision at all and CLI adds c g_kbar^in, g_kbar^in
+// being the cell's ordinary pull from x_f2 = x + e_k.  AA: the same, with S where the AA
+// layout's pull reads (see above).  A state set from outside (initial state, imported
+// populations) gets these slots from wall_prepare_kernel.  Momentum exchange: a link (x,
+// kbar) with x - e_k solid carries g~_kbar(x) into the wall and brings the new g_k back, so
+// the solid gains e_kbar (g~_kbar(x) + g_k).  (Deviations suffice: the 2 w rho0 of full
+// populations sums to zero over a periodic domain.)
+//
+// A work item's links are handled one to a lane, not one direction after the other by the
+// lanes of the cells: on the r = 60 sphere in 128^3 an item with walls has 24 links, of 9
+// directions, at 5.4 of its cells, so a loop over the directions would run 9 times, each
+// with its own coefficient load, for a third of a lane's work each.  The cells' values go
+// through shared memory: the lanes of boundary cells write their 18 values, the links' lanes
+// take the two of theirs, and, before the collision, write the new g_k back for the cells'
+// lanes to read.
+// Per step against the loop over the directions: FP64 20^3 9.9 -> 6.9 us, 128^3 311 -> 278;
+// BF16 AA 48^3 4.48 -> 4.07, 128^3 25.7 -> 23.7; FP16 A-B 48^3 4.56 -> 4.30, 128^3 33.3 -> 32.0;
+// FP32 A-B 80^3 9.06 -> 8.42, MR walls 128^3 67 -> 46; FP32 AA 48^3 to 256^3 within 1 %.
+template <typename R> struct WallStage {
+    static constexpr int kStride = 33;  // two links of one cell meet different banks
+    R *v;                               // [18 directions, then drho, u_x, u_y, u_z (WX)][kStride]
+    __device__ __forceinline__ R &at(int k, int lane) const { return v[(k - 1) * kStride + lane]; }
+};
+template <typename R, bool WX> constexpr int kWallStage = (WX ? Q + 3 : Q - 1) * WallStage<R>::kStride;
+
+// A lane's link of the item: n = the item's links, first = the first of them, and of link
+// first + lane (the first 32) its direction, its cell's lane, its CLI coefficient and its
+// index in cell order (interpolated rules).
+template <typename R> struct LinkOfLane {
+    uint32_t n, first;
+    uint32_t dir, lane;
+    R c;
+    uint32_t index;
+};
+// BRICK: the warp's cells are a 32-cell segment of the box, its links counted in cell order.
+template <bool WX, bool BRICK, typename R>
+__device__ __forceinline__ void load_link(const InstanceDev &I, const Par<R> &P, uint32_t l, LinkOfLane<R> &L)
+{
+    const uint64_t keep = l2_keep_policy();
+    const uint32_t r = ld_keep((BRICK ? I.linkr : I.ilinkr) + l, keep);
+    L.dir = r & 31u;
+    L.lane = r >> 8;
+    if (P.wall == 1) L.c = ld_keep(reinterpret_cast<const R *>(BRICK ? I.linkc : I.ilinkc) + l, keep);
+    if (WX && P.wall >= 2) L.index = BRICK ? l : ld_keep(I.ilink + l, keep);
+}
+// The first 32 links of an item (n of them, from first): lane by lane, the others none.
+template <bool WX, bool BRICK, typename R>
+__device__ __forceinline__ LinkOfLane<R> first_links(const InstanceDev &I, const Par<R> &P, uint32_t n, uint32_t first,
+                                                     int lane)
+{
+    LinkOfLane<R> L{n, first, 1u, 0u, R(0), 0u};
+    // every link of the item within the link tables
+    if (n && !checked(I, first + n, I.n_links + 1u)) L.n = 0u;
+    if ((uint32_t)lane < L.n) load_link<WX, BRICK>(I, P, first + (uint32_t)lane, L);
+    return L;
+}
+
+// The solid cell x - e_k of a link of a cell with face flags xf (as WarpItem's, bit 2: inner).
+template <typename R>
+__device__ __forceinline__ uint32_t solid_of(const Par<R> &P, uint32_t cell, uint32_t xf, int k)
+{
+    const int dx = ex_rt(k), dy = ey_rt(k), dz = ez_rt(k);
+    if (xf & 4u) {
+        uint32_t s = cell - (uint32_t)(dx + (int)P.nx * (dy + (int)P.ny * dz));
+        if (dx == 1 && (xf & 1u)) s += P.nx;
+        if (dx == -1 && (xf & 2u)) s -= P.nx;
+        return s;
+    }
+    const uint32_t yz = fast_div(cell, P.dnx), zz = fast_div(yz, P.dny);
+    const int x = (int)(cell - yz * P.nx), y = (int)(yz - zz * P.ny), z = (int)zz;
+    return (uint32_t)wrap2(x - dx, (int)P.nx) +
+           P.nx * ((uint32_t)wrap2(y - dy, (int)P.ny) + P.ny * (uint32_t)wrap2(z - dz, (int)P.nz));
+}
+
+// Before the collision: the rule's neighbour terms, and with RED the momentum exchange.
+template <int STORE, int KIND, bool RED, bool WX, bool BRICK, typename R>
+__device__ __forceinline__ void walls_in(const InstanceDev &I, const Par<R> &P, R (&g)[Q], const WarpItem &it,
+                                         LinkOfLane<R> L, const WallStage<R> &st, int lane,
+                                         const typename Store<STORE>::T *fs, R (&fm)[3])
+{
+    using S = Store<STORE>;
+    if (L.n == 0 || (!RED && P.wall == 0)) return;  // the same in all lanes
+    if (it.wm) {
+#pragma unroll
+        for (int k = 1; k < Q; ++k) st.at(k, lane) = g[k];
+    }
+    __syncwarp();
+    for (uint32_t b = 0; b < L.n; b += 32) {
+        const uint32_t j = b + (uint32_t)lane;
+        const bool mine = j < L.n;
+        if (mine && b > 0) load_link<WX, BRICK>(I, P, L.first + j, L);
+        const int k = (int)L.dir, kb = opp_rt(k), from = (int)L.lane;
+        const uint32_t lc = __shfl_sync(0xffffffffu, it.cell, from);
+        const uint32_t lx = RED && KIND == KIND_AA_LOCAL ? __shfl_sync(0xffffffffu, it.xf | (it.inner ? 4u : 0u), from) : 0u;
+        if (mine) {
+            R v = st.at(k, from);  // S, left by the previous step where this pull reads
+            if (WX && KIND == KIND_AB && P.wall >= 2)
+                v = wall_neighbour_terms<STORE>(P, P.wall,
+                                                reinterpret_cast<const R *>(I.linkw) + (size_t)L.index * kLinkW, k,
+                                                lc, st.at(kb, from), fs, v);
+            else if (L.c != R(0)) v = fma_r(L.c, st.at(kb, from), v);
+            st.at(k, from) = v;
+            if constexpr (RED) {
+                // the own post-collision g~_kbar(x) of the previous step: A-B: own slot kbar; AA
+                // after a LOCAL step: own slot k; AA after a PULL step: where it was pushed,
+                // slot kbar of x - e_k
+                const uint32_t d = (uint32_t)(KIND == KIND_AA_PULL ? k : kb);
+                const uint32_t at = KIND == KIND_AA_LOCAL ? solid_of(P, lc, lx, k) : lc;
+                if (checked(I, at, I.n32)) {
+                    const R m = S::cvt(ld_pop<KIND>(fs + (d * P.ks + at))) + v;  // e_kbar = -e_k
+                    fm[0] -= R(ex_rt(k)) * m;
+                    fm[1] -= R(ey_rt(k)) * m;
+                    fm[2] -= R(ez_rt(k)) * m;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (it.wm) {
+#pragma unroll
+        for (int k = 1; k < Q; ++k) g[k] = st.at(k, lane);
+    }
+}
+
+// After it: the own-cell part of every link's rule from the post-collision values, where the
+// next step's pull of direction k reads it: A-B slot k of x - e_k in the buffer written; AA
+// LOCAL slot kbar of x - e_k; AA PULL the own slot k.
+template <int STORE, int KIND, bool WX, bool BRICK, typename R>
+__device__ __forceinline__ void walls_out(const InstanceDev &I, const Par<R> &P, const R (&g)[Q], R drho, R ux, R uy,
+                                          R uz, const WarpItem &it, LinkOfLane<R> L, const WallStage<R> &st, int lane,
+                                          typename Store<STORE>::T *fd)
+{
+    if (L.n == 0) return;
+    if (it.wm) {
+#pragma unroll
+        for (int k = 1; k < Q; ++k) st.at(k, lane) = g[k];
+        if constexpr (WX) {
+            st.at(Q, lane) = drho;
+            st.at(Q + 1, lane) = ux;
+            st.at(Q + 2, lane) = uy;
+            st.at(Q + 3, lane) = uz;
+        }
+    }
+    __syncwarp();
+    for (uint32_t b = 0; b < L.n; b += 32) {
+        const uint32_t j = b + (uint32_t)lane;
+        const bool mine = j < L.n;
+        if (mine && b > 0) load_link<WX, BRICK>(I, P, L.first + j, L);
+        const int k = (int)L.dir, kb = opp_rt(k), from = (int)L.lane;
+        const uint32_t lc = __shfl_sync(0xffffffffu, it.cell, from);
+        const uint32_t lx = KIND != KIND_AA_PULL ? __shfl_sync(0xffffffffu, it.xf | (it.inner ? 4u : 0u), from) : 0u;
+        if (mine) {
+            const R B = st.at(k, from), C = st.at(kb, from);
+            R sv;
+            if (WX && P.wall >= 2)
+                sv = wall_own_part_w(P, reinterpret_cast<const R *>(I.linkw) + (size_t)L.index * kLinkW, k, B, C,
+                                     st.at(Q, from), st.at(Q + 1, from), st.at(Q + 2, from), st.at(Q + 3, from));
+            else sv = wall_own_part(P.wall, L.c, C, B);
+            const uint32_t d = (uint32_t)(KIND == KIND_AA_LOCAL ? kb : k);
+            const uint32_t at = KIND == KIND_AA_PULL ? lc : solid_of(P, lc, lx, k);
+            if (checked(I, at, I.n32))
+                put1<STORE>(fd + (d * P.ks + at), sv, round_key<STORE>(lc, P.hash_off), k);
+        }
+    }
+}
+
+// Locate one work item: this lane's cell, its x-face flags and wall mask, whether every lane
+// is away from the y and z faces, and the item's links (number and first), all precomputed in
+// tables that no step writes (no dependent load and no division).
 template <typename R>
 __device__ __forceinline__ void locate_item(const InstanceDev &I, const Par<R> &P, const uint2 *flane,
-                                            const uint2 *fwarp, uint32_t w, int lane, WarpItem &it)
+                                            const uint2 *fwarp, uint32_t w, int lane, WarpItem &it, uint2 &links)
 {
     const uint64_t keep = l2_keep_policy();
     const bool w_ok = checked(I, w, I.n_fwarps_padded);
-    it.wd = w_ok ? ld_keep(fwarp + w, keep) : make_uint2(0u, 0u);
+    links = w_ok ? ld_keep(fwarp + w, keep) : make_uint2(0u, 0u);
     const uint2 e = w_ok ? ld_keep(flane + (w * 32u + (uint32_t)lane), keep) : make_uint2(0xFFFFFFFFu, 0u);
     const bool live = e.x != 0xFFFFFFFFu;
     it.cell = live ? (e.x & 0x0FFFFFFFu) : 0xFFFFFFFFu;
     if (live && !checked(I, it.cell, I.n32)) it.cell = 0xFFFFFFFFu;
-    it.xf = (e.x >> 28) & 3u;
+    it.xf = live ? (e.x >> 28) & 3u : 0u;
     it.inner = ((e.x >> 30) & 1u) != 0u;  // the same in all live lanes of the item
-    it.wm = e.y & 0x7FFFFu;
-    it.off = it.wd.y + (e.y >> 19);
-    // every link of the cell within the link tables
-    if (it.wm && !checked(I, it.off + __popc(it.wm), I.n_links + 1u)) it.wm = 0u;
+    it.wm = e.y;
 }
 
 // Issue the 19 pulls of a located work item into raw[] (storage type, converted in
@@ -837,7 +896,11 @@ template <int STORE, int KIND, typename R>
 __device__ __forceinline__ void pull_item(const InstanceDev &I, const Par<R> &P, const typename Store<STORE>::T *fs,
                                           const WarpItem &it, typename Store<STORE>::T (&raw)[Q])
 {
-    if (it.cell == 0xFFFFFFFFu) return;
+    if (it.cell == 0xFFFFFFFFu) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) raw[k] = typename Store<STORE>::T{};
+        return;
+    }
     if (KIND != KIND_AA_LOCAL && it.inner) {
         const uint32_t cxm = (it.xf & 1u) ? P.nx : 0u, cxp = (it.xf & 2u) ? P.nx : 0u;
 #pragma unroll
@@ -868,47 +931,41 @@ template <typename R> struct RedAcc {
 };
 
 // Finish one work item pulled by pull_item: convert, pressure shift of the pulls that
-// crossed the x boundary, walls, collision, stores; with RED, add the lane's moments and
-// momentum exchange to acc.
-template <int COLL, int STORE, int KIND, bool RED, bool WX, typename R>
+// crossed the x boundary, walls, moments and collision, stores; with RED, add the lane's
+// moments and momentum exchange to acc.  Padding lanes take part (they may hold a link) on
+// zeros and store nothing.
+template <int COLL, int STORE, int KIND, bool RED, bool WX, bool BRICK, typename R>
 __device__ __forceinline__ void finish_item(const InstanceDev &I, const Par<R> &P,
-                                            const typename Store<STORE>::T (&raw)[Q], const WarpItem &it, int lane,
+                                            const typename Store<STORE>::T (&raw)[Q], const WarpItem &it,
+                                            const LinkOfLane<R> &L, const WallStage<R> &st, int lane,
                                             const typename Store<STORE>::T *fs, typename Store<STORE>::T *fd,
                                             unsigned *status, RedAcc<R> &acc)
 {
     using S = Store<STORE>;
-    using T = typename S::T;
-    if (it.cell == 0xFFFFFFFFu) return;
+    const bool live = it.cell != 0xFFFFFFFFu;
     R g[Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) g[k] = S::cvt(raw[k]);
-    // pressure shift of the pulls that crossed the x boundary (wall directions take their
-    // value from the wall rule instead)
-    const uint32_t wm = it.wm;
-    if (it.xf & 1u) {
-#pragma unroll
-        for (int k = 0; k < Q; ++k)
-            if (ex(k) == 1 && !((wm >> k) & 1u)) g[k] += R(weight(k)) * P.c.dshift;
-    }
-    if (it.xf & 2u) {
-#pragma unroll
-        for (int k = 0; k < Q; ++k)
-            if (ex(k) == -1 && !((wm >> k) & 1u)) g[k] -= R(weight(k)) * P.c.dshift;
-    }
-    R rd = R(0), rx = R(0), ry = R(0), rz = R(0);
+    pressure_shift(g, P, it.xf, it.wm);
     R fm[3] = {R(0), R(0), R(0)};
-    finish_cell<COLL, STORE, KIND, RED, WX, R>(I, g, P, it.cell, it.xf, it.inner, I.pull_off,
-                                               it.inner ? I.push_off : nullptr, wm, it.off, fs, fd,
-                                               reinterpret_cast<const R *>(I.linkc),
-                                               reinterpret_cast<const R *>(I.linkw), status, rd, rx, ry, rz, fm);
+    walls_in<STORE, KIND, RED, WX, BRICK>(I, P, g, it, L, st, lane, fs, fm);
+    R drho, ux, uy, uz;
+    relax<COLL, STORE>(g, P.c, drho, ux, uy, uz);
     if constexpr (RED) {
-        acc.v[RED_DRHO] += rd;
-        acc.v[RED_U + 0] += rx;
-        acc.v[RED_U + 1] += ry;
-        acc.v[RED_U + 2] += rz;
+        const R unit = STORE == ST_F16 ? R(P.isc) : R(1);  // FP16: from the stored units
+        if (live) {
+            const R uu = ux * ux + uy * uy + uz * uz;
+            if (!(uu < R(1)) || !(drho == drho)) atomicOr(status, STATUS_DIVERGED);
+            acc.v[RED_DRHO] += drho * unit;
+            acc.v[RED_U + 0] += ux;
+            acc.v[RED_U + 1] += uy;
+            acc.v[RED_U + 2] += uz;
+        }
 #pragma unroll
-        for (int d = 0; d < 3; ++d) acc.v[RED_F + d] += fm[d];
+        for (int d = 0; d < 3; ++d) acc.v[RED_F + d] += fm[d] * unit;
     }
+    if (live) store_cell<STORE, KIND>(I, P, g, it.cell, it.xf, it.inner, round_key<STORE>(it.cell, P.hash_off), fd);
+    walls_out<STORE, KIND, WX, BRICK>(I, P, g, drho, ux, uy, uz, it, L, st, lane, fd);
 }
 
 // Error-free sum (Knuth's TwoSum): s + e == a + b exactly, s = fl(a + b).
@@ -974,9 +1031,9 @@ __device__ __forceinline__ void allow_next_step() { asm volatile("griddepcontrol
 __device__ __forceinline__ void wait_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <bool BATCH>
-__device__ __forceinline__ const InstanceDev &instance_of(const InstanceDev *table, const InstanceDev &one, int i)
+__device__ __forceinline__ const InstanceDev &instance_of(const InstanceDev *copied, const InstanceDev &one)
 {
-    if constexpr (BATCH) return table[i];
+    if constexpr (BATCH) return *copied;
     else return one;
 }
 
@@ -1023,7 +1080,16 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
     } else {
         tile = TileDev{0, t, (long long)t * WARPS, nullptr, nullptr};
     }
-    const InstanceDev &I = instance_of<BATCH>(table, one, tile.inst);
+    // a batch's block copies its instance's parameters to shared memory, where they are read as
+    // a single instance's are in the constant bank: at their use, not held in registers
+    __shared__ uint4 params[BATCH ? sizeof(InstanceDev) / sizeof(uint4) : 1];
+    static_assert(sizeof(InstanceDev) % sizeof(uint4) == 0, "copied in 16-byte pieces");
+    if constexpr (BATCH) {
+        for (int i = threadIdx.x; i < (int)(sizeof(InstanceDev) / sizeof(uint4)); i += WARPS * 32)
+            params[i] = __ldg(reinterpret_cast<const uint4 *>(table + tile.inst) + i);
+        __syncthreads();
+    }
+    const InstanceDev &I = instance_of<BATCH>(reinterpret_cast<const InstanceDev *>(params), one);
     const Par<R> P = load_par<R>(I);
     const T *fs;  // state read this step
     T *fd;        // state written this step
@@ -1035,14 +1101,19 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
         fd = reinterpret_cast<T *>(I.f0);
         fs = fd;
     }
+    __shared__ R stage[WARPS * kWallStage<R, WX>];
+    const WallStage<R> st{stage + warp * kWallStage<R, WX>};
     WarpItem it;
+    uint2 links;
     locate_item<R>(I, P, BATCH ? tile.flane : I.flane, BATCH ? tile.fwarp : I.fwarp,
-                   (uint32_t)tile.seg0 + (uint32_t)warp, lane, it);
+                   (uint32_t)tile.seg0 + (uint32_t)warp, lane, it, links);
     wait_previous_step();
     T raw[Q];
     pull_item<STORE, KIND, R>(I, P, fs, it, raw);
+    // issued behind the pulls (before them its registers cost FP32 AA 256^3 2 %)
+    const LinkOfLane<R> L = first_links<WX, false, R>(I, P, links.x, links.y, lane);
     RedAcc<R> acc{};
-    finish_item<COLL, STORE, KIND, RED, WX, R>(I, P, raw, it, lane, fs, fd, status + tile.inst, acc);
+    finish_item<COLL, STORE, KIND, RED, WX, false, R>(I, P, raw, it, L, st, lane, fs, fd, status + tile.inst, acc);
     if constexpr (RED) reduce_tile(acc, I.partials, tile.local);
 }
 

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kBrickCells, tma_min_blocks<STORE>())
     };
     // what a thread needs of its cell in a brick, read from tables no step writes: loaded
     // one brick ahead, while the previous brick is being finished
-    auto locate = [&](int brick, WarpItem &m) {
+    auto locate = [&](int brick, WarpItem &m, LinkOfLane<R> &L, uint2 &yz) {
         int x0, y0, z0;
         brick_origin(bricks[brick], x0, y0, z0);
         const uint32_t x = (uint32_t)(x0 + cx), y = (uint32_t)(y0 + cy), z = (uint32_t)(z0 + cz);
@@ -148,23 +148,31 @@ __global__ void __launch_bounds__(kBrickCells, tma_min_blocks<STORE>())
         m.cell = live ? cell : 0xFFFFFFFFu;
         m.xf = (x == 0 ? 1u : 0u) | (x == P.nx - 1 ? 2u : 0u);
         m.wm = 0u;
-        m.off = 0u;
+        uint32_t off = 0u;
         m.inner = (y - 1u < P.ny - 2u) && (z - 1u < P.nz - 2u);
-        m.wd = make_uint2(y, z);
+        yz = make_uint2(y, z);
         if (live && ((sg.y >> cx) & 1u)) {
             const uint32_t bi = sg.z + __popc(sg.y & ((1u << cx) - 1u));
             if (checked(I, bi, I.n_boundary)) {
                 m.wm = I.bmask[bi];
-                m.off = I.boff[bi];
-                if (!checked(I, m.off + __popc(m.wm), I.n_links + 1u)) m.wm = 0u;
+                off = I.boff[bi];
+                if (!checked(I, off + __popc(m.wm), I.n_links + 1u)) m.wm = 0u;
             }
         }
+        // the links of the warp's cells (a segment of the box) are consecutive
+        const unsigned bb = __ballot_sync(0xffffffffu, m.wm != 0u);
+        const uint32_t n = __reduce_add_sync(0xffffffffu, (unsigned)__popc(m.wm));
+        L = first_links<WX, true, R>(I, P, n, __shfl_sync(0xffffffffu, off, bb ? __ffs(bb) - 1 : 0), cx);
     };
 
     __shared__ int failed;
     if (tid == 0) failed = 0;
+    __shared__ R stage_w[kBrickCells / 32 * kWallStage<R, WX>];
+    const WallStage<R> wst{stage_w + (tid >> 5) * kWallStage<R, WX>};
     WarpItem meta;
-    if ((int)blockIdx.x < nbricks) locate((int)blockIdx.x, meta);
+    LinkOfLane<R> link;
+    uint2 meta_yz;
+    if ((int)blockIdx.x < nbricks) locate((int)blockIdx.x, meta, link, meta_yz);
     wait_previous_step();  // the copies read what the previous step wrote
     if (tid == 0)
         for (int s = 0; s < kBrickStages; ++s)
@@ -175,9 +183,9 @@ __global__ void __launch_bounds__(kBrickCells, tma_min_blocks<STORE>())
         const int s = it % kBrickStages;
         const uint32_t parity = (uint32_t)(it / kBrickStages) & 1u;
         const bool live = meta.cell != 0xFFFFFFFFu;
-        const uint32_t xf = meta.xf, y = meta.wd.x, z = meta.wd.y;
+        const uint32_t xf = meta.xf, y = meta_yz.x, z = meta_yz.y;
         // pulls whose source lies across a face: outside the box, read directly
-        T raw[Q];
+        T raw[Q] = {};
         uint32_t wrap = 0u;
         if (live && (xf != 0u || y == 0 || y == P.ny - 1 || z == 0 || z == P.nz - 1)) {
 #pragma unroll
@@ -219,9 +227,10 @@ __global__ void __launch_bounds__(kBrickCells, tma_min_blocks<STORE>())
             }
         }
         const WarpItem now = meta;
-        if (brick + (int)gridDim.x < nbricks) locate(brick + (int)gridDim.x, meta);
+        const LinkOfLane<R> now_link = link;
+        if (brick + (int)gridDim.x < nbricks) locate(brick + (int)gridDim.x, meta, link, meta_yz);
         RedAcc<R> acc{};
-        finish_item<COLL, STORE, KIND_AB, false, WX, R>(I, P, raw, now, cx, fs, fd, nullptr, acc);
+        finish_item<COLL, STORE, KIND_AB, false, WX, true, R>(I, P, raw, now, now_link, wst, cx, fs, fd, nullptr, acc);
     }
 }
 
