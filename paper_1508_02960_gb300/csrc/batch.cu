@@ -216,16 +216,20 @@ Instance::~Instance()
     free_geometry(&geo);
 }
 
+StepGroup::~StepGroup()
+{
+    for (auto &kv : graphs) cudaGraphExecDestroy(kv.second.exec);
+    cudaFree(d_table);
+    for (TileDev *t : d_tiles) cudaFree(t);
+}
+
 Batch::~Batch()
 {
     if (stream_ || cap_) cudaStreamSynchronize(stream_);
-    for (auto &kv : graphs_) cudaGraphExecDestroy(kv.second.exec);
+    groups_.clear();
     inst_.clear();
-    for (int w = 0; w < kShapeWarpsN; ++w) cudaFree(d_wtiles_[w]);
     cudaFree(d_table_);
-    cudaFree(d_tiles_);
     cudaFree(d_tile_count_);
-    cudaFree(d_stiles_);
     cudaFree(d_stile_count_);
     cudaFree(d_bricks_);
     cudaFree(d_error_);
@@ -525,85 +529,11 @@ lbm_status Batch::rebuild()
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    sms_ = sms;
     if (!d_error_) {  // the batch's sticky error word (bounded waits, checked build)
         CK(dev_alloc(&d_error_, sizeof(unsigned)));
         CK(cudaMemset(d_error_, 0, sizeof(unsigned)));
     }
-    std::vector<InstanceDev> table(std::max(n, 1));
-    std::vector<TileDev> tiles, stiles, wtiles[kShapeWarpsN];
-    std::vector<int> tc(std::max(n, 1)), sc(std::max(n, 1));  // tiles of each instance
-    for (int i = 0; i < n; ++i) {
-        Instance &in = *inst_[i];
-        fill_dev(in, table[i]);
-        table[i].error = d_error_;
-        // state kernels: chunks of the active-segment list
-        const long long nt = std::max(1ll, (in.geo.n_active + CS - 1) / CS);
-        // step kernels: kTileSegs fluid warps per tile (the list is padded to whole tiles)
-        const long long ns = std::max(1ll, (in.geo.n_fwarps + kTileSegs - 1) / kTileSegs);
-        if (nt > in.partial_capacity || ns > in.partial_capacity) return fail(LBM_ERR_STATE, "partials too small");
-        if (ns * kTileSegs > in.geo.n_fwarps_padded) return fail(LBM_ERR_STATE, "fluid work list too short");
-        tc[i] = (int)nt;
-        for (long long t = 0; t < nt; ++t) tiles.push_back(TileDev{i, (int)t, t * CS, nullptr, nullptr});
-        sc[i] = (int)ns;
-        for (long long t = 0; t < ns; ++t)
-            stiles.push_back(TileDev{i, (int)t, t * kTileSegs, in.geo.flane, in.geo.fwarp});
-        // tiles of the other block shapes of the non-reducing step (no partial sums)
-        for (int w = 0; w < kShapeWarpsN; ++w) {
-            const int W = kShapeWarps[w];
-            // at least one tile, as for the reducing step, whose tiles the kShapeWarps[0]
-            // map also describes (an instance without fluid has one tile of padding)
-            const long long nw = std::max(1ll, (in.geo.n_fwarps + W - 1) / W);
-            if (i < kBatchMapMax) {
-                maps_[w].tile_start[i] = (int)wtiles[w].size();
-                maps_[w].flane[i] = in.geo.flane;
-                maps_[w].fwarp[i] = in.geo.fwarp;
-            }
-            if (nw * W > in.geo.n_fwarps_padded) return fail(LBM_ERR_STATE, "fluid work list too short");
-            for (long long t = 0; t < nw; ++t)
-                wtiles[w].push_back(TileDev{i, (int)t, t * W, in.geo.flane, in.geo.fwarp});
-        }
-    }
-    if (tiles.size() > (size_t)INT32_MAX || stiles.size() > (size_t)INT32_MAX)
-        return fail(LBM_ERR_ARG, "too many tiles");
-    for (int w = 0; w < kShapeWarpsN; ++w) {  // maps for batches of 2 .. kBatchMapMax instances
-        maps_[w].n = (n >= 2 && n <= kBatchMapMax) ? n : 0;
-        if (maps_[w].n) maps_[w].tile_start[n] = (int)wtiles[w].size();
-    }
-    ntiles_ = (int)tiles.size();
-    nstiles_ = (int)stiles.size();
-    cudaFree(d_table_);
-    cudaFree(d_tiles_);
-    cudaFree(d_tile_count_);
-    cudaFree(d_stiles_);
-    cudaFree(d_stile_count_);
-    d_table_ = nullptr;
-    d_tiles_ = d_stiles_ = nullptr;
-    d_tile_count_ = d_stile_count_ = nullptr;
-    h_table_ = table;
-    CK(dev_alloc(&d_table_, sizeof(InstanceDev) * table.size()));
-    CK(cudaMemcpy(d_table_, table.data(), sizeof(InstanceDev) * table.size(), cudaMemcpyHostToDevice));
-    if (ntiles_ > 0) {
-        CK(dev_alloc(&d_tiles_, sizeof(TileDev) * tiles.size()));
-        CK(cudaMemcpy(d_tiles_, tiles.data(), sizeof(TileDev) * tiles.size(), cudaMemcpyHostToDevice));
-    }
-    CK(dev_alloc(&d_tile_count_, sizeof(int) * tc.size()));
-    CK(cudaMemcpy(d_tile_count_, tc.data(), sizeof(int) * tc.size(), cudaMemcpyHostToDevice));
-    if (nstiles_ > 0) {
-        CK(dev_alloc(&d_stiles_, sizeof(TileDev) * stiles.size()));
-        CK(cudaMemcpy(d_stiles_, stiles.data(), sizeof(TileDev) * stiles.size(), cudaMemcpyHostToDevice));
-    }
-    for (int w = 0; w < kShapeWarpsN; ++w) {
-        cudaFree(d_wtiles_[w]);
-        d_wtiles_[w] = nullptr;
-        nwtiles_[w] = (int)wtiles[w].size();
-        if (nwtiles_[w] > 0) {
-            CK(dev_alloc(&d_wtiles_[w], sizeof(TileDev) * wtiles[w].size()));
-            CK(cudaMemcpy(d_wtiles_[w], wtiles[w].data(), sizeof(TileDev) * wtiles[w].size(),
-                          cudaMemcpyHostToDevice));
-        }
-    }
-    CK(dev_alloc(&d_stile_count_, sizeof(int) * sc.size()));
-    CK(cudaMemcpy(d_stile_count_, sc.data(), sizeof(int) * sc.size(), cudaMemcpyHostToDevice));
     if (n > capacity_) {
         cudaFree(d_sums_);
         cudaFree(d_status_);
@@ -627,18 +557,124 @@ lbm_status Batch::rebuild()
         CK(cudaMallocHost(&h_sums_, sizeof(double) * kRedSlots * capacity_));
         CK(cudaMallocHost(&h_status_, sizeof(unsigned) * capacity_));
     }
-    // one step block per tile; the hardware block scheduler balances the tiles
-    grid_ = std::max(1, nstiles_);
-    sms_ = sms;
-    for (auto &kv : graphs_) cudaGraphExecDestroy(kv.second.exec);
-    graphs_.clear();
-    shape_ = StepShape{};
-    shape_src_ = 0;
-    aux_grid_ = std::max(1, std::min(sms * 8, (ntiles_ + 7) / 8));
-    lbm_status st = setup_tma();
+    std::vector<InstanceDev> table(std::max(n, 1));
+    std::vector<int> tc(std::max(n, 1)), sc(std::max(n, 1));  // tiles of each instance
+    long long most = 1;
+    for (int i = 0; i < n; ++i) {
+        Instance &in = *inst_[i];
+        fill_dev(in, table[i]);
+        table[i].error = d_error_;
+        table[i].status = d_status_ + i;
+        // state kernels: chunks of the active-segment list
+        const long long nt = std::max(1ll, (in.geo.n_active + CS - 1) / CS);
+        // reducing step: kTileSegs fluid warps per tile (the list is padded to whole tiles)
+        const long long ns = std::max(1ll, (in.geo.n_fwarps + kTileSegs - 1) / kTileSegs);
+        if (nt > in.partial_capacity || ns > in.partial_capacity) return fail(LBM_ERR_STATE, "partials too small");
+        if (nt > INT32_MAX || ns > INT32_MAX) return fail(LBM_ERR_ARG, "too many tiles");
+        tc[i] = (int)nt;
+        sc[i] = (int)ns;
+        most = std::max(most, nt);
+    }
+    cudaFree(d_table_);
+    cudaFree(d_tile_count_);
+    cudaFree(d_stile_count_);
+    d_table_ = nullptr;
+    d_tile_count_ = d_stile_count_ = nullptr;
+    CK(dev_alloc(&d_table_, sizeof(InstanceDev) * table.size()));
+    CK(cudaMemcpy(d_table_, table.data(), sizeof(InstanceDev) * table.size(), cudaMemcpyHostToDevice));
+    CK(dev_alloc(&d_tile_count_, sizeof(int) * tc.size()));
+    CK(cudaMemcpy(d_tile_count_, tc.data(), sizeof(int) * tc.size(), cudaMemcpyHostToDevice));
+    CK(dev_alloc(&d_stile_count_, sizeof(int) * sc.size()));
+    CK(cudaMemcpy(d_stile_count_, sc.data(), sizeof(int) * sc.size(), cudaMemcpyHostToDevice));
+    aux_grid_ = (int)std::max(1ll, std::min((long long)sms * 8, (most + 7) / 8));
+    lbm_status st = build_groups(table);
     if (st != LBM_OK) return st;
-    lookup_shape();
+    st = setup_tma();
+    if (st != LBM_OK) return st;
+    for (auto &g : groups_) lookup_shape(*g);
     dirty_ = false;
+    return LBM_OK;
+}
+
+// Which instances step together.  The launches of a group step all of its members before the
+// next group's are queued, for all the steps of a call, so the state that a step touches is the
+// group's, not the batch's.  An instance whose fluid cells fill the GPU by themselves is a
+// group of its own: its parameters go by value, and a state of up to L2's size stays there
+// from step to step.  The others share groups of at most kGroupBytes of populations, evenly.
+// Per step of the whole batch, one launch for all -> in groups: the first 16 sweep points, FP16
+// A-B, 425 -> 366 us; 12 points, FP16 AA, 315 -> 255; 10 points, FP32 AA, 181 -> 145; 4 cells of
+// 128^3, FP32 AA, 144 -> 112; 64 cells of 48^3, FP32 AA, 150 -> 125 (two groups).  kAlone: 6
+// cells of 80^3 (290,000 fluid cells) are faster together (FP32 AA 46 us, alone 53), of 96^3
+// (560,000) alone (79, together 108).
+lbm_status Batch::build_groups(const std::vector<InstanceDev> &table)
+{
+    constexpr long long kAlone = 400000;
+    constexpr long long kGroupBytes = 64ll << 20;
+    groups_.clear();
+    std::vector<int> small;
+    long long small_cells = 0;
+    auto open = [&](std::vector<int> members) {
+        groups_.emplace_back(new StepGroup());
+        groups_.back()->members = std::move(members);
+    };
+    for (int i = 0; i < size(); ++i) {
+        const long long f = inst_[i]->geo.n_fluid;
+        if (size() == 1 || f >= kAlone) {
+            open({i});
+        } else {
+            small.push_back(i);
+            small_cells += f;
+        }
+    }
+    const long long cell_bytes = Q * (long long)storage_bytes(storage_) * (layout_ == LBM_LAYOUT_AB ? 2 : 1);
+    const long long parts = std::max(1ll, (small_cells * cell_bytes + kGroupBytes - 1) / kGroupBytes);
+    std::vector<std::vector<int>> shared((size_t)parts);
+    long long before = 0;
+    for (int i : small) {
+        shared[(size_t)(small_cells ? std::min(parts - 1, before * parts / small_cells) : 0)].push_back(i);
+        before += inst_[i]->geo.n_fluid;
+    }
+    for (auto &m : shared)
+        if (!m.empty()) open(std::move(m));
+    for (auto &gp : groups_) {
+        StepGroup &g = *gp;
+        const int n = (int)g.members.size();
+        std::vector<TileDev> tiles[kShapeWarpsN];
+        long long total[kShapeWarpsN] = {};
+        for (int r = 0; r < n; ++r) {
+            const Instance &in = *inst_[g.members[r]];
+            g.h_table.push_back(table[g.members[r]]);
+            g.fluid += in.geo.n_fluid;
+            for (int w = 0; w < kShapeWarpsN; ++w) {
+                const int W = kShapeWarps[w];
+                // at least one tile (an instance without fluid has one of padding)
+                const long long nw = std::max(1ll, (in.geo.n_fwarps + W - 1) / W);
+                if (nw * W > in.geo.n_fwarps_padded) return fail(LBM_ERR_STATE, "fluid work list too short");
+                if (total[w] + nw > INT32_MAX) return fail(LBM_ERR_ARG, "too many tiles");
+                if (n >= 2 && n <= kBatchMapMax) {
+                    g.maps[w].tile_start[r] = (int)total[w];
+                    g.maps[w].flane[r] = in.geo.flane;
+                    g.maps[w].fwarp[r] = in.geo.fwarp;
+                } else if (n > kBatchMapMax) {
+                    for (long long t = 0; t < nw; ++t)
+                        tiles[w].push_back(TileDev{r, (int)t, t * W, in.geo.flane, in.geo.fwarp});
+                }
+                total[w] += nw;
+            }
+        }
+        for (int w = 0; w < kShapeWarpsN; ++w) {
+            g.ntiles[w] = (int)total[w];
+            g.maps[w].n = n >= 2 && n <= kBatchMapMax ? n : 0;
+            if (g.maps[w].n) g.maps[w].tile_start[n] = (int)total[w];
+            if (tiles[w].empty()) continue;
+            CK(dev_alloc(&g.d_tiles[w], sizeof(TileDev) * tiles[w].size()));
+            CK(cudaMemcpy(g.d_tiles[w], tiles[w].data(), sizeof(TileDev) * tiles[w].size(), cudaMemcpyHostToDevice));
+        }
+        if (n > 1) {
+            CK(dev_alloc(&g.d_table, sizeof(InstanceDev) * n));
+            CK(cudaMemcpy(g.d_table, g.h_table.data(), sizeof(InstanceDev) * n, cudaMemcpyHostToDevice));
+        }
+    }
     return LBM_OK;
 }
 
@@ -684,34 +720,23 @@ lbm_status Batch::init_equilibrium(int i)
 struct StepQueue {
     const FormatOps *ops;
     Launch L;                // the reducing step (kStepWarps-warp tiles, one block each)
-    Launch Ln[2];            // the non-reducing steps (the tuned shape), by AA kind (A-B: [0])
+    Launch Ln;               // the non-reducing steps (the tuned shape)
     int warps;               // warps per block of Ln
-    const InstanceDev *one;  // single instance: its parameters by value; else NULL
+    const InstanceDev *one;  // a lone instance: its parameters by value; else NULL
     int wx;                  // some instance uses an interpolated wall rule
     bool to_and_fro;         // every other step takes the tiles from the last to the first
     const TmaLaunch *tma;    // non-reducing steps on the TMA brick kernel; else NULL
     int collision, layout;
-    unsigned *status;
-    int n_status;
-    const int *tile_count;
-    double *sums;
-    int n_inst;
-    double *fscratch;
-    unsigned *fcount;
 };
 
-// Queue n steps on stream s starting from (flip, aa); returns launches queued.
-static cudaError_t queue_steps(const StepQueue &q, cudaStream_t s, long long n, bool reduce_last, int &flip,
-                               int &aa, long long &launches)
+// Queue n steps of a group on stream s starting from (flip, aa), the last one reducing where
+// asked.
+static cudaError_t queue_steps(const StepQueue &q, cudaStream_t s, long long n, bool reduce_last, int flip, int aa)
 {
-    Launch L = q.L;
-    L.stream = s;
+    Launch L = q.L, Ln = q.Ln;
+    L.stream = Ln.stream = s;
     for (long long i = 0; i < n; ++i) {
         const bool red = reduce_last && i == n - 1;
-        if (red) {
-            cudaError_t e = cudaMemsetAsync(q.status, 0, sizeof(unsigned) * q.n_status, s);
-            if (e != cudaSuccess) return e;
-        }
         const int kind = q.layout == LBM_LAYOUT_AB ? KIND_AB : (aa == 0 ? KIND_AA_PULL : KIND_AA_LOCAL);
         const int order = q.to_and_fro && ((q.layout == LBM_LAYOUT_AB ? flip : aa) & 1) ? kStepBackwards : 0;
         cudaError_t e;
@@ -720,33 +745,23 @@ static cudaError_t queue_steps(const StepQueue &q, cudaStream_t s, long long n, 
             T.stream = s;
             e = q.ops->step_tma(q.collision, q.wx, T, *q.one, flip);
         } else if (red || q.wx) {  // the reducing and interpolated-wall steps: kStepWarps tiles
-            e = q.ops->step(q.collision, kind, L, flip | order, red ? 1 : 0, q.status, q.one, q.wx, kStepWarps);
+            e = q.ops->step(q.collision, kind, L, flip | order, red ? 1 : 0, q.one, q.wx, kStepWarps);
         } else {
-            Launch Ls = q.Ln[kind == KIND_AA_LOCAL ? 1 : 0];
-            Ls.stream = s;
-            e = q.ops->step(q.collision, kind, Ls, flip | order, 0, q.status, q.one, 0, q.warps);
+            e = q.ops->step(q.collision, kind, Ln, flip | order, 0, q.one, 0, q.warps);
         }
         if (e != cudaSuccess) return e;
-        ++launches;
         if (q.layout == LBM_LAYOUT_AB) flip ^= 1;
         else aa ^= 1;
-    }
-    if (reduce_last && n > 0) {
-        cudaError_t e = launch_final_reduce(q.L.table, q.tile_count, q.n_inst, q.sums, q.fscratch, q.fcount, s);
-        if (e != cudaSuccess) return e;
-        ++launches;
     }
     return cudaSuccess;
 }
 
-// Launch of the non-reducing step of AA kind (or A-B) `kind` in block shape sh.
-Launch Batch::shaped_launch(const StepShape &sh, int kind) const
+// Launch of a step of a group in blocks of `warps` warps.
+Launch Batch::shaped_launch(const StepGroup &g, int warps) const
 {
     int w = 0;
-    while (w < kShapeWarpsN && kShapeWarps[w] != sh.warps) ++w;
-    (void)kind;
-    const int nt = nwtiles_[w];
-    return Launch{d_table_, d_wtiles_[w], nt, sh.warps, std::max(1, nt), sh.warps * 32, stream_, sms_, &maps_[w]};
+    while (kShapeWarps[w] != warps) ++w;
+    return Launch{g.d_table, g.d_tiles[w], g.ntiles[w], warps, g.ntiles[w], warps * 32, stream_, sms_, &g.maps[w]};
 }
 
 // Every other step takes its tiles from the last to the first, so that it begins with the
@@ -758,53 +773,55 @@ Launch Batch::shaped_launch(const StepShape &sh, int kind) const
 // 56.8 -> 52.1.  Below 32 MiB of fluid populations (FP32 AA 80^3 and 96^3, BF16 AA 112^3) both
 // orders take the same time, and a cell of one tile per multiprocessor is 3 % slower to and
 // fro (FP64 20^3 17.1 -> 17.7 us), so those keep one direction.
-bool Batch::to_and_fro() const
+bool Batch::to_and_fro(const StepGroup &g) const
 {
-    const long long bytes = fluid_cells() * Q * (long long)storage_bytes(storage_);
+    const long long bytes = g.fluid * Q * (long long)storage_bytes(storage_);
     return bytes * (layout_ == LBM_LAYOUT_AB ? 2 : 1) >= (32ll << 20);
 }
 
-// The graph of m steps (+ the reduction when red) from (flip_, aa_phase_) in shape sh,
-// instantiated on first use and kept in a small least-recently-used cache.
-lbm_status Batch::graph_for(long long m, bool red, const StepShape &sh, int wx, cudaGraphExec_t *out)
+// The graph of m steps of a group from (flip, aa) in shape sh, the last one reducing when red,
+// instantiated on first use and kept in a small least-recently-used cache.  The only group of a
+// batch has the reduction's set-up and the final sums in its graph, too.
+lbm_status Batch::graph_for(StepGroup &g, long long m, bool red, int flip, int aa, const StepShape &sh, int wx,
+                            cudaGraphExec_t *out)
 {
-    const GraphKey key{m * 2 + (red ? 1 : 0), flip_, aa_phase_, sh.warps};
-    auto it = graphs_.find(key);
-    if (it != graphs_.end()) {
-        it->second.used = ++graph_clock_;
+    const GraphKey key{m * 2 + (red ? 1 : 0), flip, aa, sh.warps};
+    auto it = g.graphs.find(key);
+    if (it != g.graphs.end()) {
+        it->second.used = ++g.graph_clock;
         *out = it->second.exec;
         return LBM_OK;
     }
-    if (graphs_.size() >= kGraphCache) {  // evict the least recently used graph
-        auto lru = graphs_.begin();
-        for (auto g = graphs_.begin(); g != graphs_.end(); ++g)
-            if (g->second.used < lru->second.used) lru = g;
+    if (g.graphs.size() >= kGraphCache) {  // evict the least recently used graph
+        auto lru = g.graphs.begin();
+        for (auto c = g.graphs.begin(); c != g.graphs.end(); ++c)
+            if (c->second.used < lru->second.used) lru = c;
         cudaGraphExecDestroy(lru->second.exec);
-        graphs_.erase(lru);
+        g.graphs.erase(lru);
     }
-    StepQueue q{&ops(),
-                Launch{d_table_, d_stiles_, nstiles_, kTileSegs, grid_, kStepWarps * 32, stream_, sms_, &maps_[0]},
-                {shaped_launch(sh, layout_ == LBM_LAYOUT_AB ? KIND_AB : KIND_AA_PULL),
-                 shaped_launch(sh, KIND_AA_LOCAL)},
-                sh.warps,
-                size() == 1 ? &h_table_[0] : nullptr,
-                wx,
-                to_and_fro(),
-                tma_ ? &tma_launch_ : nullptr,
-                collision_,
-                layout_,
-                d_status_,
-                size(),
-                d_stile_count_,
-                d_sums_,
-                size(),
-                d_fscratch_,
-                d_fcount_};
-    int f = flip_, a = aa_phase_;
-    long long dummy = 0;
+    const StepQueue q{&ops(),
+                      shaped_launch(g, kStepWarps),
+                      shaped_launch(g, sh.warps),
+                      sh.warps,
+                      g.members.size() == 1 ? &g.h_table[0] : nullptr,
+                      wx,
+                      to_and_fro(g),
+                      tma_ ? &tma_launch_ : nullptr,
+                      collision_,
+                      layout_};
+    const bool sums = red && groups_.size() == 1;
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = queue_steps(q, cap_, m, red, f, a, dummy);
+    cudaError_t e = queue_steps(q, cap_, red ? m - 1 : m, false, flip, aa);
+    if (e == cudaSuccess && red) {
+        const int odd = (int)((m - 1) & 1);
+        if (sums) e = cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), cap_);
+        if (e == cudaSuccess)
+            e = queue_steps(q, cap_, 1, true, layout_ == LBM_LAYOUT_AB ? flip ^ odd : flip,
+                            layout_ == LBM_LAYOUT_AB ? aa : aa ^ odd);
+        if (e == cudaSuccess && sums)
+            e = launch_final_reduce(d_table_, d_stile_count_, size(), d_sums_, d_fscratch_, d_fcount_, cap_);
+    }
     cudaError_t e2 = cudaStreamEndCapture(cap_, &graph);
     if (e != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
@@ -815,14 +832,14 @@ lbm_status Batch::graph_for(long long m, bool red, const StepShape &sh, int wx, 
     e = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
-    graphs_[key] = CachedGraph{exec, ++graph_clock_};
+    g.graphs[key] = CachedGraph{exec, ++g.graph_clock};
     *out = exec;
     return LBM_OK;
 }
 
 // Block shapes of the non-reducing step, tuned online: every shape gives the same state bit
 // for bit (the cells' arithmetic does not depend on how the tiles are grouped), so the first
-// steps of a batch time each candidate on the live state.  The choice is cached per
+// steps of a group time each candidate on the live state.  The choice is cached per
 // (storage, collision, layout, instance count, total fluid cells, multiprocessor count) for
 // the process.
 namespace {
@@ -841,35 +858,34 @@ const StepShape kShapeCandidates[] = {{kShapeWarps[0]}, {kShapeWarps[1]}, {kShap
 constexpr int kTuneSteps = 16;  // steps timed per candidate (even: flip and AA phase return)
 }  // namespace
 
-void Batch::lookup_shape()
+void Batch::lookup_shape(StepGroup &g)
 {
-    tune_shape_ = false;
-    if (tma_ || size() == 0) return;
+    if (tma_) return;
     for (auto &p : inst_)
         if (p->desc.wall >= LBM_LIBB) return;  // the interpolated-wall step has one shape
     std::lock_guard<std::mutex> lk(g_shape_mu);
-    auto it = g_shapes.find(ShapeKey{storage_, collision_, layout_, size(), sms_, fluid_cells()});
+    auto it = g_shapes.find(ShapeKey{storage_, collision_, layout_, (int)g.members.size(), sms_, g.fluid});
     if (it != g_shapes.end()) {
-        shape_ = it->second;
-        shape_src_ = 2;
+        g.shape = it->second;
+        g.shape_src = 2;
     } else {
-        tune_shape_ = true;
+        g.tune = true;
     }
 }
 
-lbm_status Batch::tune_shape(int wx)
+lbm_status Batch::tune_shape(StepGroup &g, int wx)
 {
     const int nc = (int)(sizeof(kShapeCandidates) / sizeof(kShapeCandidates[0]));
     cudaEvent_t ev[2];
     CK(cudaEventCreate(&ev[0]));
     CK(cudaEventCreate(&ev[1]));
     double best = 0.0;
-    StepShape pick = shape_;
+    StepShape pick = g.shape;
     lbm_status st = LBM_OK;
     for (int c = 0; c < nc && st == LBM_OK; ++c) {
         const StepShape &sh = kShapeCandidates[c];
         cudaGraphExec_t exec = nullptr;
-        if ((st = graph_for(kTuneSteps, false, sh, wx, &exec)) != LBM_OK) break;
+        if ((st = graph_for(g, kTuneSteps, false, flip_, aa_phase_, sh, wx, &exec)) != LBM_OK) break;
         cudaError_t e = cudaEventRecord(ev[0], stream_);
         if (e == cudaSuccess) e = cudaGraphLaunch(exec, stream_);
         if (e == cudaSuccess) e = cudaEventRecord(ev[1], stream_);
@@ -881,7 +897,7 @@ lbm_status Batch::tune_shape(int wx)
             break;
         }
         launches_ += kTuneSteps;
-        shape_ms_[c] = ms / kTuneSteps;
+        g.shape_ms[c] = ms / kTuneSteps;
         if (c == 0 || ms < best) {
             best = ms;
             pick = sh;
@@ -890,11 +906,11 @@ lbm_status Batch::tune_shape(int wx)
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
     if (st != LBM_OK) return st;
-    shape_ = pick;
-    shape_src_ = 1;
-    tune_shape_ = false;
+    g.shape = pick;
+    g.shape_src = 1;
+    g.tune = false;
     std::lock_guard<std::mutex> lk(g_shape_mu);
-    g_shapes[ShapeKey{storage_, collision_, layout_, size(), sms_, fluid_cells()}] = pick;
+    g_shapes[ShapeKey{storage_, collision_, layout_, (int)g.members.size(), sms_, g.fluid}] = pick;
     return LBM_OK;
 }
 
@@ -910,24 +926,37 @@ lbm_status Batch::step(long long n)
     int wx = 0;
     for (auto &p : inst_) wx |= p->desc.wall >= LBM_LIBB;
     const int nc = (int)(sizeof(kShapeCandidates) / sizeof(kShapeCandidates[0]));
-    long long left = n;
-    if (tune_shape_ && n > (long long)nc * kTuneSteps) {  // the first steps time the shapes
-        lbm_status st = tune_shape(wx);
-        if (st != LBM_OK) return st;
-        left -= (long long)nc * kTuneSteps;
+    const bool several = groups_.size() > 1;
+    if (several) CK(cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), stream_));
+    int flip = flip_, aa = aa_phase_;
+    for (auto &g : groups_) {  // each group takes all the steps
+        long long left = n;
+        if (g->tune && n > (long long)nc * kTuneSteps) {  // the first steps time the shapes
+            lbm_status st = tune_shape(*g, wx);
+            if (st != LBM_OK) return st;
+            left -= (long long)nc * kTuneSteps;
+        }
+        flip = flip_;
+        aa = aa_phase_;
+        const long long kChunk = 1000;
+        while (left > 0) {
+            const long long m = left > 2 * kChunk ? kChunk : left;
+            const bool red = (m == left);
+            cudaGraphExec_t exec = nullptr;
+            lbm_status st = graph_for(*g, m, red, flip, aa, g->shape, wx, &exec);
+            if (st != LBM_OK) return st;
+            CK(cudaGraphLaunch(exec, stream_));
+            launches_ += m + (red && !several ? 1 : 0);
+            if (layout_ == LBM_LAYOUT_AB) flip ^= (int)(m & 1);
+            else aa ^= (int)(m & 1);
+            left -= m;
+        }
     }
-    const long long kChunk = 1000;
-    while (left > 0) {
-        const long long m = left > 2 * kChunk ? kChunk : left;
-        const bool red = (m == left);
-        cudaGraphExec_t exec = nullptr;
-        lbm_status st = graph_for(m, red, shape_, wx, &exec);
-        if (st != LBM_OK) return st;
-        CK(cudaGraphLaunch(exec, stream_));
-        launches_ += m + (red ? 1 : 0);
-        if (layout_ == LBM_LAYOUT_AB) flip_ ^= (int)(m & 1);
-        else aa_phase_ ^= (int)(m & 1);
-        left -= m;
+    flip_ = flip;
+    aa_phase_ = aa;
+    if (several) {
+        CK(launch_final_reduce(d_table_, d_stile_count_, size(), d_sums_, d_fscratch_, d_fcount_, stream_));
+        ++launches_;
     }
     for (auto &p : inst_) {
         p->steps += n;
@@ -968,18 +997,10 @@ lbm_status Batch::moment_sums_now(int i, double *sums)
         if (st != LBM_OK) return st;
     }
     Instance &in = *inst_[i];
-    std::vector<int> tb(size());
-    {
-        int acc = 0;
-        for (int j = 0; j < size(); ++j) {
-            tb[j] = acc;
-            acc += (int)std::max(1ll, (inst_[j]->geo.n_active + block_ / 32 - 1) / (block_ / 32));
-        }
-    }
     const int nt = (int)std::max(1ll, (in.geo.n_active + block_ / 32 - 1) / (block_ / 32));
-    Launch L{d_table_, d_tiles_ + tb[i], nt, block_ / 32, std::max(1, std::min(aux_grid_, (nt + 7) / 8)), 256,
+    Launch L{d_table_, nullptr, nt, block_ / 32, std::max(1, std::min(aux_grid_, (nt + 7) / 8)), 256,
              stream_};
-    CK(ops().moments(L, layout_, cur_of(in), aa_phase_, 1, 0, nullptr));
+    CK(ops().moments(L, i, layout_, cur_of(in), aa_phase_, 1, 0, nullptr));
     double *ds = d_sums_ + (size_t)kRedSlots * i;
     double *hs = h_sums_ + (size_t)kRedSlots * i;
     CK(launch_final_reduce(d_table_ + i, d_tile_count_ + i, 1, ds, d_fscratch_ + (size_t)i * kFinalSlices * (RED_F + 3),
@@ -1206,19 +1227,13 @@ lbm_status Batch::get_velocity(int i, double *host)
     Instance &in = *inst_[i];
     const long long n = in.geo.ncells;
     CK(ensure_stage(&d_stage_, &stage_cells_, n));
-    std::vector<int> tb(size());
-    int acc = 0;
-    for (int j = 0; j < size(); ++j) {
-        tb[j] = acc;
-        acc += (int)std::max(1ll, (inst_[j]->geo.n_active + block_ / 32 - 1) / (block_ / 32));
-    }
     const int nt = (int)std::max(1ll, (in.geo.n_active + block_ / 32 - 1) / (block_ / 32));
-    Launch L{d_table_, d_tiles_ + tb[i], nt, block_ / 32, std::max(1, std::min(aux_grid_, (nt + 7) / 8)), 256,
+    Launch L{d_table_, nullptr, nt, block_ / 32, std::max(1, std::min(aux_grid_, (nt + 7) / 8)), 256,
              stream_};
     for (int c = 0; c < 3; ++c) {
         // all-solid segments are not in the work list: clear the whole field first
         CK(cudaMemsetAsync(d_stage_, 0, sizeof(double) * n, stream_));
-        CK(ops().moments(L, layout_, cur_of(in), aa_phase_, 0, c, d_stage_));
+        CK(ops().moments(L, i, layout_, cur_of(in), aa_phase_, 0, c, d_stage_));
         ++launches_;
         CK(cudaMemcpyAsync(host + (long long)c * n, d_stage_, sizeof(double) * n, cudaMemcpyDeviceToHost, stream_));
     }
@@ -1281,9 +1296,14 @@ void Batch::fill_info(int i, lbm_info *out) const
     out->autotune = tune_src_;
     out->tune_ms_tiles = tune_ms_[0];
     out->tune_ms_bricks = tune_ms_[1];
-    out->step_warps = tma_ ? 0 : shape_.warps;
-    out->shape_source = shape_src_;
-    for (int c = 0; c < kShapeWarpsN; ++c) out->shape_ms[c] = shape_ms_[c];
+    out->step_warps = tma_ ? 0 : kStepWarps;
+    for (auto &g : groups_) {  // the instance's group's, the first group's for a whole batch
+        if (i >= 0 && std::find(g->members.begin(), g->members.end(), i) == g->members.end()) continue;
+        if (!tma_) out->step_warps = g->shape.warps;
+        out->shape_source = g->shape_src;
+        for (int c = 0; c < kShapeWarpsN; ++c) out->shape_ms[c] = g->shape_ms[c];
+        break;
+    }
 }
 
 // ------------------------------------------------------------------------------------

@@ -49,6 +49,44 @@ constexpr int kShapeWarps[] = {4, 2, 8};  // the candidates, in the order they a
 static_assert(kShapeWarps[0] == kStepWarps, "shape 0 is the reducing step's (its tile map serves both)");
 constexpr int kShapeWarpsN = 3;
 
+struct GraphKey {
+    long long steps_red;
+    int flip, aa, shape;
+    bool operator<(const GraphKey &o) const
+    {
+        return std::tie(steps_red, flip, aa, shape) < std::tie(o.steps_red, o.flip, o.aa, o.shape);
+    }
+};
+struct CachedGraph {
+    cudaGraphExec_t exec;
+    long long used;
+};
+
+// Instances of a batch that one launch per time step advances together.  A group takes all the
+// steps of a call before the next group's, so that its state stays in L2 from step to step.
+struct StepGroup {
+    std::vector<int> members;            // instance indices, increasing
+    std::vector<InstanceDev> h_table;    // their parameters (a lone one's go by value)
+    InstanceDev *d_table = nullptr;
+    // step tiles: their number by block shape (kShapeWarps; [0] is the reducing step's too),
+    // and where they are: maps for 2 .. kBatchMapMax members, records beyond
+    int ntiles[kShapeWarpsN] = {};
+    BatchMap maps[kShapeWarpsN] = {};
+    TileDev *d_tiles[kShapeWarpsN] = {};
+    long long fluid = 0;
+    StepShape shape;
+    int shape_src = 0;                   // 0 default, 1 measured by this group, 2 from the cache
+    double shape_ms[kShapeWarpsN] = {};
+    bool tune = false;
+    std::map<GraphKey, CachedGraph> graphs;
+    long long graph_clock = 0;
+
+    StepGroup() = default;
+    StepGroup(const StepGroup &) = delete;
+    StepGroup &operator=(const StepGroup &) = delete;
+    ~StepGroup();
+};
+
 class Batch {
 public:
     ~Batch();
@@ -99,24 +137,14 @@ public:
     lbm_status prepare();              // upload tables and choose the step kernel now if pending
 
 private:
-    struct GraphKey {
-        long long steps_red;
-        int flip, aa, shape;
-        bool operator<(const GraphKey &o) const
-        {
-            return std::tie(steps_red, flip, aa, shape) < std::tie(o.steps_red, o.flip, o.aa, o.shape);
-        }
-    };
-    struct CachedGraph {
-        cudaGraphExec_t exec;
-        long long used;
-    };
-    static constexpr size_t kGraphCache = 16;  // instantiated step graphs kept per batch
-    bool to_and_fro() const;            // the order of the step tiles alternates
-    Launch shaped_launch(const StepShape &sh, int kind) const;
-    lbm_status graph_for(long long m, bool red, const StepShape &sh, int wx, cudaGraphExec_t *out);
-    void lookup_shape();                // the cached shape of this batch, or tuning pending
-    lbm_status tune_shape(int wx);      // time every candidate shape on the live state
+    static constexpr size_t kGraphCache = 16;  // instantiated step graphs kept per group
+    Launch shaped_launch(const StepGroup &g, int warps) const;
+    bool to_and_fro(const StepGroup &g) const;  // the order of the step tiles alternates
+    lbm_status graph_for(StepGroup &g, long long m, bool red, int flip, int aa, const StepShape &sh, int wx,
+                         cudaGraphExec_t *out);
+    void lookup_shape(StepGroup &g);              // the cached shape of this group, or tuning pending
+    lbm_status tune_shape(StepGroup &g, int wx);  // time every candidate shape on the live state
+    lbm_status build_groups(const std::vector<InstanceDev> &table);
     lbm_status rebuild();          // upload table and tiles, drop graphs
     lbm_status aa_restart(int i);  // instance i (i < 0: all) set from outside: AA arrangement of step 0
     int cur_of(const Instance &in) const { return in.phase ^ flip_; }
@@ -129,18 +157,14 @@ private:
     cudaStream_t stream_ = nullptr;   // user stream (launches)
     cudaStream_t cap_ = nullptr;      // private stream for graph capture
     InstanceDev *d_table_ = nullptr;
-    std::vector<InstanceDev> h_table_;  // host copy (the single-instance launch passes it by value)
-    TileDev *d_tiles_ = nullptr;      // tiles of the active-segment lists (state kernels)
-    int *d_tile_count_ = nullptr;
-    TileDev *d_stiles_ = nullptr;     // tiles of the fluid-warp lists (step kernels)
-    int *d_stile_count_ = nullptr;
-    int nstiles_ = 0;
+    int *d_tile_count_ = nullptr;     // chunks of the active-segment lists (state kernels), per instance
+    int *d_stile_count_ = nullptr;    // tiles of the fluid-warp lists (step kernels), per instance
+    std::vector<std::unique_ptr<StepGroup>> groups_;
     double *d_sums_ = nullptr;        // [n][kRedSlots]
     unsigned *d_status_ = nullptr;    // [n]
     double *h_sums_ = nullptr;        // pinned [n][kRedSlots]
     unsigned *h_status_ = nullptr;    // pinned [n]
     int capacity_ = 0;
-    int ntiles_ = 0;
     int block_ = 32 * kStepWarps;      // cells per chunk of the state kernels
     int step_mode_ = 0;               // 0 (default) and 1: tiles of fluid cells; 2: TMA bricks
     // TMA brick kernel (single instance, A-B layout, box a multiple of the brick)
@@ -149,23 +173,11 @@ private:
     uint32_t *d_bricks_ = nullptr;
     unsigned *d_error_ = nullptr;
     lbm_status setup_tma();           // decides tma_ and builds maps and brick list
-    int grid_ = 0;                    // step-kernel blocks (one per step tile)
     int aux_grid_ = 1;
     int flip_ = 0;
     int aa_phase_ = 0;
     bool dirty_ = true;
     long long launches_ = 0;
-    std::map<GraphKey, CachedGraph> graphs_;
-    long long graph_clock_ = 0;
-    // tiles of every block shape of the non-reducing step
-    TileDev *d_wtiles_[kShapeWarpsN] = {nullptr, nullptr, nullptr};
-    int nwtiles_[kShapeWarpsN] = {0, 0, 0};
-    // the same tiles as kernel-parameter maps (batches of 2 .. kBatchMapMax instances)
-    BatchMap maps_[kShapeWarpsN] = {};
-    StepShape shape_;
-    int shape_src_ = 0;                // 0 default, 1 measured by this batch, 2 from the cache
-    double shape_ms_[kShapeWarpsN] = {0, 0, 0};
-    bool tune_shape_ = false;
     int sms_ = 0;
     double *d_stage_ = nullptr;       // FP64 staging for import/export (one direction)
     long long stage_cells_ = 0;

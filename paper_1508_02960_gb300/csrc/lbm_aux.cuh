@@ -273,14 +273,14 @@ __global__ void state_scatter_kernel(const InstanceDev *__restrict__ table, int 
     }
 }
 
-// Moments of the stored post-collision state of every fluid cell, one warp per work
-// chunk.  mode 0: write the velocity component `comp` to out[cell] of fluid cells (the
+// Moments of the stored post-collision state of every fluid cell of an instance, one warp per
+// chunk of chunk_segs active segments.  mode 0: write the velocity component `comp` to out[cell] of fluid cells (the
 // caller clears out first).  mode 1: chunk partial sums (drho, u_x, u_y, u_z) into
 // I.partials, in FP64 in a fixed order; the force slots, which only a step defines, are
 // written as 0.
 template <int STORE>
 __global__ void __launch_bounds__(256) moments_kernel(const InstanceDev *__restrict__ table,
-                                                      const TileDev *__restrict__ chunks, int nchunks, int chunk_segs,
+                                                      int inst, int nchunks, int chunk_segs,
                                                       int layout, int cur, int aa_phase, int mode, int comp,
                                                       double *__restrict__ out)
 {
@@ -290,22 +290,22 @@ __global__ void __launch_bounds__(256) moments_kernel(const InstanceDev *__restr
     const int gw = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     const int nw = (int)((gridDim.x * (long long)blockDim.x) >> 5);
     for (int c = gw; c < nchunks; c += nw) {
-        const TileDev chunk = chunks[c];
-        const InstanceDev &I = table[chunk.inst];
-        const int n_e = min(chunk_segs, (int)(I.n_active - (uint32_t)chunk.seg0));
+        const InstanceDev &I = table[inst];
+        const long long seg0 = (long long)c * chunk_segs;  // chunk c of the active segments
+        const int n_e = min(chunk_segs, (int)((long long)I.n_active - seg0));
         double a[4] = {0.0, 0.0, 0.0, 0.0};
         for (int i = 0; i < n_e; ++i) {
-            const uint4 meta = I.aseg[chunk.seg0 + i];
+            const uint4 meta = I.aseg[seg0 + i];
             const long long cell = (long long)meta.w * 32 + lane;
             if ((meta.x >> lane) & 1u) continue;
-            CellGeom c;
-            cell_geom(I, cell, meta, lane, c);
+            CellGeom cg;
+            cell_geom(I, cell, meta, lane, cg);
             double drho = 0.0, j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
             for (int k = 0; k < Q; ++k) {
                 int buf;
                 const long long idx =
-                    canonical_index<STORE>(I, layout, aa_phase, cur, cell, k, c.wm, c.X, c.Y, c.Z, buf);
+                    canonical_index<STORE>(I, layout, aa_phase, cur, cell, k, cg.wm, cg.X, cg.Y, cg.Z, buf);
                 const T *f = reinterpret_cast<const T *>(buf ? I.f1 : I.f0);
                 const double g = (double)S::load(f + idx, I.inv_scale);
                 drho += g;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256) moments_kernel(const InstanceDev *__restr
 #pragma unroll
             for (int d = 0; d < 4; ++d) a[d] = warp_sum(a[d]);
             if (lane == 0)
-                for (int d = 0; d < kRedSlots; ++d) I.partials[(long long)chunk.local * kRedSlots + d] = d < 4 ? a[d] : 0.0;
+                for (int d = 0; d < kRedSlots; ++d) I.partials[(long long)c * kRedSlots + d] = d < 4 ? a[d] : 0.0;
         }
     }
 }

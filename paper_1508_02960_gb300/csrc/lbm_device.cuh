@@ -372,6 +372,7 @@ struct alignas(16) InstanceDev {
     // (STATUS_BOUNDS, STATUS_TIMEOUT), which the host reads with the reductions
     uint32_t n_fwarps_padded, n_boundary, n_links;
     unsigned *error;
+    unsigned *status;        // the instance's status word (STATUS_DIVERGED, reducing steps)
 };
 
 #ifdef LBM_CHECKED

@@ -36,7 +36,7 @@ cudaError_t launch_step(void (*kernel)(P...), const Launch &L, bool overlap, A &
 template <int STORE> constexpr int kSrt = STORE == ST_F64 ? (int)COLL_TRT : (int)COLL_SRT;
 
 template <int STORE, int COLL, int KIND, bool RED, bool WX, int WARPS>
-cudaError_t step_red(const Launch &L, int flip, unsigned *status, const InstanceDev *one)
+cudaError_t step_red(const Launch &L, int flip, const InstanceDev *one)
 {
     cudaError_t e;
     // A grid that the multiprocessors hold at once starts after the previous step has ended:
@@ -49,12 +49,12 @@ cudaError_t step_red(const Launch &L, int flip, unsigned *status, const Instance
     const bool overlap = (long long)L.grid * WARPS > (long long)L.sms * resident;
     if (one) {  // a single instance: parameters travel in the constant bank
         e = launch_step(step_kernel<COLL, STORE, KIND, false, RED, WX, WARPS>, L, overlap, L.table, *one, NoBatchMap{}, L.tiles,
-                        L.ntiles, flip, status);
+                        L.ntiles, flip);
     } else {  // a batch: parameters from the device table, the tiles' instances from the map
         static const InstanceDev unused{};
         static const BatchMap no_map{};  // n = 0: tile records
         e = launch_step(step_kernel<COLL, STORE, KIND, true, RED, WX, WARPS>, L, overlap, L.table, unused,
-                        L.map ? *L.map : no_map, L.tiles, L.ntiles, flip, status);
+                        L.map ? *L.map : no_map, L.tiles, L.ntiles, flip);
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -64,44 +64,44 @@ cudaError_t step_red(const Launch &L, int flip, unsigned *status, const Instance
 // warps: warps per block of a non-reducing SBB/CLI step (2, 4 or 8); the reducing and the
 // interpolated-wall steps run kStepWarps.
 template <int STORE, int COLL, int KIND>
-cudaError_t step_one(const Launch &L, int flip, int reduce, unsigned *status, const InstanceDev *one, int wx,
+cudaError_t step_one(const Launch &L, int flip, int reduce, const InstanceDev *one, int wx,
                      int warps)
 {
     if constexpr (KIND == KIND_AB) {
         if (wx)
-            return reduce ? step_red<STORE, COLL, KIND, true, true, kStepWarps>(L, flip, status, one)
-                          : step_red<STORE, COLL, KIND, false, true, kStepWarps>(L, flip, status, one);
+            return reduce ? step_red<STORE, COLL, KIND, true, true, kStepWarps>(L, flip, one)
+                          : step_red<STORE, COLL, KIND, false, true, kStepWarps>(L, flip, one);
     } else {
         if (wx) return cudaErrorInvalidValue;
     }
-    if (reduce) return step_red<STORE, COLL, KIND, true, false, kStepWarps>(L, flip, status, one);
+    if (reduce) return step_red<STORE, COLL, KIND, true, false, kStepWarps>(L, flip, one);
     switch (warps) {
-    case 2: return step_red<STORE, COLL, KIND, false, false, 2>(L, flip, status, one);
-    case 8: return step_red<STORE, COLL, KIND, false, false, 8>(L, flip, status, one);
-    default: return step_red<STORE, COLL, KIND, false, false, kStepWarps>(L, flip, status, one);
+    case 2: return step_red<STORE, COLL, KIND, false, false, 2>(L, flip, one);
+    case 8: return step_red<STORE, COLL, KIND, false, false, 8>(L, flip, one);
+    default: return step_red<STORE, COLL, KIND, false, false, kStepWarps>(L, flip, one);
     }
 }
 
 template <int STORE>
-cudaError_t step(int coll, int kind, const Launch &L, int flip, int reduce, unsigned *status, const InstanceDev *one,
+cudaError_t step(int coll, int kind, const Launch &L, int flip, int reduce, const InstanceDev *one,
                  int wx, int warps)
 {
     switch (coll * 3 + kind) {
-    case COLL_SRT * 3 + KIND_AB: return step_one<STORE, kSrt<STORE>, KIND_AB>(L, flip, reduce, status, one, wx, warps);
+    case COLL_SRT * 3 + KIND_AB: return step_one<STORE, kSrt<STORE>, KIND_AB>(L, flip, reduce, one, wx, warps);
     case COLL_SRT * 3 + KIND_AA_PULL:
-        return step_one<STORE, kSrt<STORE>, KIND_AA_PULL>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, kSrt<STORE>, KIND_AA_PULL>(L, flip, reduce, one, wx, warps);
     case COLL_SRT * 3 + KIND_AA_LOCAL:
-        return step_one<STORE, kSrt<STORE>, KIND_AA_LOCAL>(L, flip, reduce, status, one, wx, warps);
-    case COLL_TRT * 3 + KIND_AB: return step_one<STORE, COLL_TRT, KIND_AB>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, kSrt<STORE>, KIND_AA_LOCAL>(L, flip, reduce, one, wx, warps);
+    case COLL_TRT * 3 + KIND_AB: return step_one<STORE, COLL_TRT, KIND_AB>(L, flip, reduce, one, wx, warps);
     case COLL_TRT * 3 + KIND_AA_PULL:
-        return step_one<STORE, COLL_TRT, KIND_AA_PULL>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, COLL_TRT, KIND_AA_PULL>(L, flip, reduce, one, wx, warps);
     case COLL_TRT * 3 + KIND_AA_LOCAL:
-        return step_one<STORE, COLL_TRT, KIND_AA_LOCAL>(L, flip, reduce, status, one, wx, warps);
-    case COLL_MRT * 3 + KIND_AB: return step_one<STORE, COLL_MRT, KIND_AB>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, COLL_TRT, KIND_AA_LOCAL>(L, flip, reduce, one, wx, warps);
+    case COLL_MRT * 3 + KIND_AB: return step_one<STORE, COLL_MRT, KIND_AB>(L, flip, reduce, one, wx, warps);
     case COLL_MRT * 3 + KIND_AA_PULL:
-        return step_one<STORE, COLL_MRT, KIND_AA_PULL>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, COLL_MRT, KIND_AA_PULL>(L, flip, reduce, one, wx, warps);
     case COLL_MRT * 3 + KIND_AA_LOCAL:
-        return step_one<STORE, COLL_MRT, KIND_AA_LOCAL>(L, flip, reduce, status, one, wx, warps);
+        return step_one<STORE, COLL_MRT, KIND_AA_LOCAL>(L, flip, reduce, one, wx, warps);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -214,9 +214,9 @@ cudaError_t state_dir(const InstanceDev *table, int inst, long long nf, int layo
 }
 
 template <int STORE>
-cudaError_t moments(const Launch &L, int layout, int cur, int aa_phase, int mode, int comp, double *out)
+cudaError_t moments(const Launch &L, int inst, int layout, int cur, int aa_phase, int mode, int comp, double *out)
 {
-    moments_kernel<STORE><<<L.grid, L.block, 0, L.stream>>>(L.table, L.tiles, L.ntiles, L.chunk_segs, layout, cur,
+    moments_kernel<STORE><<<L.grid, L.block, 0, L.stream>>>(L.table, inst, L.ntiles, L.chunk_segs, layout, cur,
                                                             aa_phase, mode, comp, out);
     return cudaGetLastError();
 }

@@ -27,11 +27,11 @@ struct TraceRange {
     ~TraceRange();
 };
 
-// Arguments of one launch over a tile list (each tile: up to chunk_segs consecutive
-// entries of one instance's active-segment list).
+// Arguments of one launch: ntiles step tiles (of the instances of a group, table its
+// parameters), or ntiles chunks of chunk_segs active segments of one instance (state kernels).
 struct Launch {
     const InstanceDev *table;
-    const TileDev *tiles;
+    const TileDev *tiles;           // step tiles of a batch too large for a map; else NULL
     int ntiles;
     int chunk_segs;
     int grid, block;
@@ -58,8 +58,8 @@ struct FormatOps {
     // wx: some instance uses LIBB, QIBB, IEBB or MR (A-B layout)
     // warps: warps per block of a non-reducing SBB/CLI step (2, 4 or 8; the reducing and the
     // interpolated-wall steps run kStepWarps); L.block must be warps * 32
-    cudaError_t (*step)(int coll, int kind, const Launch &L, int flip, int reduce, unsigned *status,
-                        const InstanceDev *one, int wx, int warps);
+    cudaError_t (*step)(int coll, int kind, const Launch &L, int flip, int reduce, const InstanceDev *one, int wx,
+                        int warps);
     cudaError_t (*init)(const InstanceDev *table, int inst, long long ncells, int layout, int cur,
                         double amp, unsigned long long seed, cudaStream_t s);
     cudaError_t (*import_dir)(const InstanceDev *table, int inst, long long ncells, int layout, int cur,
@@ -70,7 +70,7 @@ struct FormatOps {
     // gathers them into buf [nk][n_fluid], 0 scatters them from buf (the step-0 arrangement)
     cudaError_t (*state_dir)(const InstanceDev *table, int inst, long long n_fluid, int layout, int cur,
                              int aa_phase, int k, int nk, void *buf, int to_host, cudaStream_t s);
-    cudaError_t (*moments)(const Launch &L, int layout, int cur, int aa_phase, int mode, int comp,
+    cudaError_t (*moments)(const Launch &L, int inst, int layout, int cur, int aa_phase, int mode, int comp,
                            double *out);
     // TMA brick step (non-reducing, single instance, A-B); one: the instance's parameters
     cudaError_t (*step_tma)(int coll, int wx, const TmaLaunch &T, const InstanceDev &one, int flip);

@@ -869,23 +869,31 @@ __device__ __forceinline__ void walls_out(const InstanceDev &I, const Par<R> &P,
     }
 }
 
-// Locate one work item: this lane's cell, its x-face flags and wall mask, whether every lane
-// is away from the y and z faces, and the item's links (number and first), all precomputed in
-// tables that no step writes (no dependent load and no division).
-template <typename R>
-__device__ __forceinline__ void locate_item(const InstanceDev &I, const Par<R> &P, const uint2 *flane,
-                                            const uint2 *fwarp, uint32_t w, int lane, WarpItem &it, uint2 &links)
+// Work item w of a work list (flane, fwarp): this lane's entry and the item's links (number and
+// first), precomputed in tables that no step writes (no dependent load and no division).
+struct ItemEntry {
+    uint2 cell, links;
+};
+__device__ __forceinline__ ItemEntry load_entry(const uint2 *flane, const uint2 *fwarp, uint32_t w, int lane, bool ok)
 {
     const uint64_t keep = l2_keep_policy();
-    const bool w_ok = checked(I, w, I.n_fwarps_padded);
-    links = w_ok ? ld_keep(fwarp + w, keep) : make_uint2(0u, 0u);
-    const uint2 e = w_ok ? ld_keep(flane + (w * 32u + (uint32_t)lane), keep) : make_uint2(0xFFFFFFFFu, 0u);
-    const bool live = e.x != 0xFFFFFFFFu;
-    it.cell = live ? (e.x & 0x0FFFFFFFu) : 0xFFFFFFFFu;
+    ItemEntry e;
+    e.links = ok ? ld_keep(fwarp + w, keep) : make_uint2(0u, 0u);
+    e.cell = ok ? ld_keep(flane + (w * 32u + (uint32_t)lane), keep) : make_uint2(0xFFFFFFFFu, 0u);
+    return e;
+}
+// This lane's cell, its x-face flags and wall mask, and whether every lane is away from the y
+// and z faces.
+__device__ __forceinline__ WarpItem locate_item(const InstanceDev &I, const ItemEntry &e)
+{
+    WarpItem it;
+    const bool live = e.cell.x != 0xFFFFFFFFu;
+    it.cell = live ? (e.cell.x & 0x0FFFFFFFu) : 0xFFFFFFFFu;
     if (live && !checked(I, it.cell, I.n32)) it.cell = 0xFFFFFFFFu;
-    it.xf = live ? (e.x >> 28) & 3u : 0u;
-    it.inner = ((e.x >> 30) & 1u) != 0u;  // the same in all live lanes of the item
-    it.wm = e.y;
+    it.xf = live ? (e.cell.x >> 28) & 3u : 0u;
+    it.inner = ((e.cell.x >> 30) & 1u) != 0u;  // the same in all live lanes of the item
+    it.wm = e.cell.y;
+    return it;
 }
 
 // Issue the 19 pulls of a located work item into raw[] (storage type, converted in
@@ -939,7 +947,7 @@ __device__ __forceinline__ void finish_item(const InstanceDev &I, const Par<R> &
                                             const typename Store<STORE>::T (&raw)[Q], const WarpItem &it,
                                             const LinkOfLane<R> &L, const WallStage<R> &st, int lane,
                                             const typename Store<STORE>::T *fs, typename Store<STORE>::T *fd,
-                                            unsigned *status, RedAcc<R> &acc)
+                                            RedAcc<R> &acc)
 {
     using S = Store<STORE>;
     const bool live = it.cell != 0xFFFFFFFFu;
@@ -955,7 +963,7 @@ __device__ __forceinline__ void finish_item(const InstanceDev &I, const Par<R> &
         const R unit = STORE == ST_F16 ? R(P.isc) : R(1);  // FP16: from the stored units
         if (live) {
             const R uu = ux * ux + uy * uy + uz * uz;
-            if (!(uu < R(1)) || !(drho == drho)) atomicOr(status, STATUS_DIVERGED);
+            if (!(uu < R(1)) || !(drho == drho)) atomicOr(I.status, STATUS_DIVERGED);
             acc.v[RED_DRHO] += drho * unit;
             acc.v[RED_U + 0] += ux;
             acc.v[RED_U + 1] += uy;
@@ -1030,11 +1038,43 @@ __device__ __forceinline__ void reduce_tile(const RedAcc<R> &acc, double *partia
 __device__ __forceinline__ void allow_next_step() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <bool BATCH>
-__device__ __forceinline__ const InstanceDev &instance_of(const InstanceDev *copied, const InstanceDev &one)
+// The tile t of a launch.  A single instance's tiles are consecutive: tile t holds work items
+// WARPS t ... (no load precedes the work list's).
+template <bool BATCH, int WARPS>
+__device__ __forceinline__ TileDev tile_of(const MapArg<BATCH> &map, const TileDev *tiles, int t)
 {
-    if constexpr (BATCH) return *copied;
-    else return one;
+    if constexpr (BATCH) {
+        if (map.n == 0) return tiles[t];
+        int lo = 0, hi = map.n - 1;  // the instance whose tiles hold t: the last i with tile_start[i] <= t
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (map.tile_start[mid] <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        const int local = t - map.tile_start[lo];
+        return TileDev{lo, local, (long long)local * WARPS, map.flane[lo], map.fwarp[lo]};
+    } else {
+        return TileDev{0, t, (long long)t * WARPS, nullptr, nullptr};
+    }
+}
+
+// The parameters of a block's instance: a single instance's in the constant bank; a batch's
+// block copies its instance's to shared memory (params), where they are read in the same way,
+// at their use, not held in registers.
+template <bool BATCH> constexpr int kParamWords = BATCH ? (int)(sizeof(InstanceDev) / sizeof(uint4)) : 1;
+static_assert(sizeof(InstanceDev) % sizeof(uint4) == 0, "copied in 16-byte pieces");
+template <bool BATCH, int WARPS>
+__device__ __forceinline__ const InstanceDev &instance_of(const InstanceDev *table, const InstanceDev &one, int inst,
+                                                          uint4 *params)
+{
+    if constexpr (BATCH) {
+        for (int i = threadIdx.x; i < kParamWords<BATCH>; i += WARPS * 32)
+            params[i] = __ldg(reinterpret_cast<const uint4 *>(table + inst) + i);
+        __syncthreads();
+        return *reinterpret_cast<const InstanceDev *>(params);
+    } else {
+        return one;
+    }
 }
 
 // The fused step.  One block of WARPS warps per tile of WARPS work items (32 fluid cells
@@ -1045,13 +1085,12 @@ __device__ __forceinline__ const InstanceDev &instance_of(const InstanceDev *cop
 // and the order of the tiles (bit kStepBackwards).  The RED variant (the step that ends a
 // chunk) also makes every tile write its FP64 partial sums (the kRedSlots slots: drho, u_x,
 // u_y, u_z and the momentum exchanged with the solid) and flags diverged cells in
-// status[instance]; the other steps carry none of that code.  The WX variant (A-B only)
+// the instance's status word; the other steps carry none of that code.  The WX variant (A-B only)
 // also runs the interpolated wall rules LIBB, QIBB, IEBB and MR.
 template <int COLL, int STORE, int KIND, bool BATCH, bool RED, bool WX, int WARPS = kStepWarps>
 __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, WX, WARPS, KIND, BATCH>())
     step_kernel(const InstanceDev *__restrict__ table, const __grid_constant__ InstanceDev one,
-                const __grid_constant__ MapArg<BATCH> map, const TileDev *__restrict__ tiles, int ntiles, int flip,
-                unsigned *__restrict__ status)
+                const __grid_constant__ MapArg<BATCH> map, const TileDev *__restrict__ tiles, int ntiles, int flip)
 {
     static_assert(!RED || WARPS == kStepWarps, "the reducing step runs kStepWarps-warp tiles");
     using S = Store<STORE>;
@@ -1063,33 +1102,17 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
     const int t = (flip & kStepBackwards) ? ntiles - 1 - (int)blockIdx.x : (int)blockIdx.x;
     // a single instance's tiles are consecutive: tile t holds work items WARPS t ... (its
     // table entry holds the same, so that no load precedes the work list's)
-    TileDev tile;
-    if constexpr (BATCH) {
-        if (map.n > 0) {  // the instance whose tiles hold t: the last i with tile_start[i] <= t
-            int lo = 0, hi = map.n - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (map.tile_start[mid] <= t) lo = mid;
-                else hi = mid - 1;
-            }
-            const int local = t - map.tile_start[lo];
-            tile = TileDev{lo, local, (long long)local * WARPS, map.flane[lo], map.fwarp[lo]};
-        } else {
-            tile = tiles[t];
-        }
-    } else {
-        tile = TileDev{0, t, (long long)t * WARPS, nullptr, nullptr};
-    }
-    // a batch's block copies its instance's parameters to shared memory, where they are read as
-    // a single instance's are in the constant bank: at their use, not held in registers
-    __shared__ uint4 params[BATCH ? sizeof(InstanceDev) / sizeof(uint4) : 1];
-    static_assert(sizeof(InstanceDev) % sizeof(uint4) == 0, "copied in 16-byte pieces");
-    if constexpr (BATCH) {
-        for (int i = threadIdx.x; i < (int)(sizeof(InstanceDev) / sizeof(uint4)); i += WARPS * 32)
-            params[i] = __ldg(reinterpret_cast<const uint4 *>(table + tile.inst) + i);
-        __syncthreads();
-    }
-    const InstanceDev &I = instance_of<BATCH>(reinterpret_cast<const InstanceDev *>(params), one);
+    const TileDev tile = tile_of<BATCH, WARPS>(map, tiles, t);
+    const uint32_t w = (uint32_t)tile.seg0 + (uint32_t)warp;
+    ItemEntry entry;
+    // a batch's entries are loaded beside its parameters, not after them (the checked build needs
+    // their number first)
+    if constexpr (BATCH && !kChecked) entry = load_entry(tile.flane, tile.fwarp, w, lane, true);
+    __shared__ uint4 params[kParamWords<BATCH>];
+    const InstanceDev &I = instance_of<BATCH, WARPS>(table, one, tile.inst, params);
+    if constexpr (!BATCH || kChecked)
+        entry = load_entry(BATCH ? tile.flane : I.flane, BATCH ? tile.fwarp : I.fwarp, w, lane,
+                           checked(I, w, I.n_fwarps_padded));
     const Par<R> P = load_par<R>(I);
     const T *fs;  // state read this step
     T *fd;        // state written this step
@@ -1103,17 +1126,14 @@ __global__ void __launch_bounds__(WARPS * 32, step_min_blocks<STORE, COLL, RED, 
     }
     __shared__ R stage[WARPS * kWallStage<R, WX>];
     const WallStage<R> st{stage + warp * kWallStage<R, WX>};
-    WarpItem it;
-    uint2 links;
-    locate_item<R>(I, P, BATCH ? tile.flane : I.flane, BATCH ? tile.fwarp : I.fwarp,
-                   (uint32_t)tile.seg0 + (uint32_t)warp, lane, it, links);
+    const WarpItem it = locate_item(I, entry);
     wait_previous_step();
     T raw[Q];
     pull_item<STORE, KIND, R>(I, P, fs, it, raw);
     // issued behind the pulls (before them its registers cost FP32 AA 256^3 2 %)
-    const LinkOfLane<R> L = first_links<WX, false, R>(I, P, links.x, links.y, lane);
+    const LinkOfLane<R> L = first_links<WX, false, R>(I, P, entry.links.x, entry.links.y, lane);
     RedAcc<R> acc{};
-    finish_item<COLL, STORE, KIND, RED, WX, false, R>(I, P, raw, it, L, st, lane, fs, fd, status + tile.inst, acc);
+    finish_item<COLL, STORE, KIND, RED, WX, false, R>(I, P, raw, it, L, st, lane, fs, fd, acc);
     if constexpr (RED) reduce_tile(acc, I.partials, tile.local);
 }
 

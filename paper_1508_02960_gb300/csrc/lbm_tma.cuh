@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kBrickCells, tma_min_blocks<STORE>())
         const LinkOfLane<R> now_link = link;
         if (brick + (int)gridDim.x < nbricks) locate(brick + (int)gridDim.x, meta, link, meta_yz);
         RedAcc<R> acc{};
-        finish_item<COLL, STORE, KIND_AB, false, WX, true, R>(I, P, raw, now, now_link, wst, cx, fs, fd, nullptr, acc);
+        finish_item<COLL, STORE, KIND_AB, false, WX, true, R>(I, P, raw, now, now_link, wst, cx, fs, fd, acc);
     }
 }
 
