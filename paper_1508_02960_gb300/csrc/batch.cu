@@ -725,6 +725,7 @@ struct StepQueue {
     const InstanceDev *one;  // a lone instance: its parameters by value; else NULL
     int wx;                  // some instance uses an interpolated wall rule
     bool to_and_fro;         // every other step takes the tiles from the last to the first
+    bool early;              // work-list entries asked for at once
     const TmaLaunch *tma;    // non-reducing steps on the TMA brick kernel; else NULL
     int collision, layout;
 };
@@ -738,7 +739,8 @@ static cudaError_t queue_steps(const StepQueue &q, cudaStream_t s, long long n, 
     for (long long i = 0; i < n; ++i) {
         const bool red = reduce_last && i == n - 1;
         const int kind = q.layout == LBM_LAYOUT_AB ? KIND_AB : (aa == 0 ? KIND_AA_PULL : KIND_AA_LOCAL);
-        const int order = q.to_and_fro && ((q.layout == LBM_LAYOUT_AB ? flip : aa) & 1) ? kStepBackwards : 0;
+        const int order = (q.to_and_fro && ((q.layout == LBM_LAYOUT_AB ? flip : aa) & 1) ? kStepBackwards : 0) |
+                          (q.early ? kStepEarly : 0);
         cudaError_t e;
         if (!red && q.tma) {  // the reducing step always runs the tile kernel
             TmaLaunch T = *q.tma;
@@ -773,11 +775,19 @@ Launch Batch::shaped_launch(const StepGroup &g, int warps) const
 // 56.8 -> 52.1.  Below 32 MiB of fluid populations (FP32 AA 80^3 and 96^3, BF16 AA 112^3) both
 // orders take the same time, and a cell of one tile per multiprocessor is 3 % slower to and
 // fro (FP64 20^3 17.1 -> 17.7 us), so those keep one direction.
-bool Batch::to_and_fro(const StepGroup &g) const
+bool Batch::to_and_fro(const StepGroup &g) const { return state_bytes(g) >= (32ll << 20); }
+
+long long Batch::state_bytes(const StepGroup &g) const
 {
-    const long long bytes = g.fluid * Q * (long long)storage_bytes(storage_);
-    return bytes * (layout_ == LBM_LAYOUT_AB ? 2 : 1) >= (32ll << 20);
+    return g.fluid * Q * (long long)storage_bytes(storage_) * (layout_ == LBM_LAYOUT_AB ? 2 : 1);
 }
+
+// A state inside L2 leaves its steps waiting for latencies, not bytes: they ask for every
+// item's work-list entries at once, where larger ones read those of a run not at all.  Both
+// ways, early / not: BF16 AA 96^3 (19 MB) 12.4 / 12.6 us, 128^3 (45 MB) 23.75 / 23.9; FP32 AA
+// 128^3 (91 MB) 27.8 / 27.5, 256^3 258 / 252; FP16 A-B 128^3 (91 MB) 32.0 / 31.6; BF16 AA 384^3
+// 681 / 655.
+bool Batch::early(const StepGroup &g) const { return state_bytes(g) <= (64ll << 20); }
 
 // The graph of m steps of a group from (flip, aa) in shape sh, the last one reducing when red,
 // instantiated on first use and kept in a small least-recently-used cache.  The only group of a
@@ -806,6 +816,7 @@ lbm_status Batch::graph_for(StepGroup &g, long long m, bool red, int flip, int a
                       g.members.size() == 1 ? &g.h_table[0] : nullptr,
                       wx,
                       to_and_fro(g),
+                      early(g),
                       tma_ ? &tma_launch_ : nullptr,
                       collision_,
                       layout_};

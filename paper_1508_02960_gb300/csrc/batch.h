@@ -139,7 +139,9 @@ public:
 private:
     static constexpr size_t kGraphCache = 16;  // instantiated step graphs kept per group
     Launch shaped_launch(const StepGroup &g, int warps) const;
+    long long state_bytes(const StepGroup &g) const;  // fluid populations, both buffers
     bool to_and_fro(const StepGroup &g) const;  // the order of the step tiles alternates
+    bool early(const StepGroup &g) const;       // work-list entries asked for at once
     lbm_status graph_for(StepGroup &g, long long m, bool red, int flip, int aa, const StepShape &sh, int wx,
                          cudaGraphExec_t *out);
     void lookup_shape(StepGroup &g);              // the cached shape of this group, or tuning pending

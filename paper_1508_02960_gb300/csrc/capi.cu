@@ -139,7 +139,11 @@ lbm_status lbm_debug_corrupt_worklist(lbm_ctx *ctx)
     if (!in.geo.flane || in.geo.n_fwarps < 1) return fail(LBM_ERR_STATE, "no fluid cells");
     const uint32_t bad = (uint32_t)in.geo.ncells;  // one past the last cell
     // the cell of the step kernels' first work-list entry (flane[0].x)
-    cudaError_t e = cudaMemcpyAsync(in.geo.flane, &bad, sizeof(bad), cudaMemcpyHostToDevice, ctx->b.stream());
+    const uint4 own_entries = make_uint4(0u, 0u, 0u, 0u);  // (the first item no run, so that the step reads it)
+    cudaError_t e = cudaMemcpyAsync(in.geo.fwarp, &own_entries, sizeof(own_entries), cudaMemcpyHostToDevice,
+                                    ctx->b.stream());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(in.geo.flane, &bad, sizeof(bad), cudaMemcpyHostToDevice, ctx->b.stream());
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->b.stream());
     return e == cudaSuccess ? LBM_OK : cuda_fail(e, "cudaMemcpyAsync");
 }

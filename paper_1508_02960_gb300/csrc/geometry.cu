@@ -156,11 +156,15 @@ __global__ void fluid_scatter_kernel(long long n, const uint4 *__restrict__ seg,
 //      x = 0, bit 29 x = nx - 1 (the pulls and pushes that cross the x faces), bit 30 every
 //      cell of the item away from the y and z faces (the same in all its lanes);
 //      0xFFFFFFFF for a padding lane;
-//   y: the wall mask (bit k: x - e_k solid).
-// count[w] = number of cut links of the item's cells.
+//   y: the wall mask (bit k: x - e_k solid);
+// and fwarp[w] = {x: the item's links (item_links_kernel: y the first of them), z, w}: an item
+// that is a run, 32 consecutive cells without walls in rows of at least 32, is described by
+// z = bit 31 | its first cell | bit 30 as above and w = the lane of the cell at x = 0 (32: the
+// cell after the last; 63: none), and a step does not read its entries in flane; other items
+// have z = 0.  count[w] = x.
 __global__ void flane_kernel(long long nw, int nx, int ny, int nz, const uint32_t *__restrict__ icell,
                              const uint4 *__restrict__ seg, const uint32_t *__restrict__ bmask,
-                             uint2 *__restrict__ flane, unsigned long long *__restrict__ count)
+                             uint2 *__restrict__ flane, uint4 *__restrict__ fwarp, unsigned long long *__restrict__ count)
 {
     const int lane = threadIdx.x & 31;
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -172,29 +176,39 @@ __global__ void flane_kernel(long long nw, int nx, int ny, int nz, const uint32_
         if (live && ((m.y >> (c & 31u)) & 1u))  // the boundary table lists boundary cells in cell order
             wm = bmask[m.z + __popc(m.y & ((1u << (c & 31u)) - 1u))];
         const unsigned links = __reduce_add_sync(0xffffffffu, (unsigned)__popc(wm));
-        uint32_t ce = 0xFFFFFFFFu;
+        uint32_t ce = 0xFFFFFFFFu, x = 1u;
         bool in_yz = true;
         if (live) {
-            const uint32_t x = c % (uint32_t)nx, yz = c / (uint32_t)nx;
-            const uint32_t y = yz % (uint32_t)ny, z = yz / (uint32_t)ny;
+            x = c % (uint32_t)nx;
+            const uint32_t yz = c / (uint32_t)nx, y = yz % (uint32_t)ny, z = yz / (uint32_t)ny;
             ce = c | (x == 0 ? 1u << 28 : 0u) | (x == (uint32_t)nx - 1u ? 1u << 29 : 0u);
             in_yz = y >= 1 && y + 2 <= (uint32_t)ny && z >= 1 && z + 2 <= (uint32_t)nz;
         }
-        if (__all_sync(0xffffffffu, in_yz) && live) ce |= 1u << 30;
+        const bool inner = __all_sync(0xffffffffu, in_yz);
+        if (inner && live) ce |= 1u << 30;
         flane[w * 32 + lane] = make_uint2(ce, wm);
-        if (lane == 0) count[w] = links;
+        const uint32_t c0 = __shfl_sync(0xffffffffu, c, 0);
+        const bool run = __all_sync(0xffffffffu, live && c == c0 + (uint32_t)lane) && links == 0 && nx >= 32;
+        const unsigned at0 = __ballot_sync(0xffffffffu, live && x == 0u);
+        const bool end = __shfl_sync(0xffffffffu, x, 31) == (uint32_t)nx - 1u;
+        if (lane == 0) {
+            count[w] = links;
+            fwarp[w] = run ? make_uint4(0u, 0u, c0 | 1u << 31 | (inner ? 1u << 30 : 0u),
+                                        at0 ? (uint32_t)__ffs(at0) - 1u : end ? 32u : 63u)
+                           : make_uint4(links, 0u, 0u, 0u);
+        }
     }
 }
 
 // The links of the work items, item by item (an item's cells may have other items' between
-// them): fwarp[w] = {the item's links, the first of them}, and for link i of this order
+// them): fwarp[w].y = the first of the item's links, and for link i of this order
 // ilinkr[i] = k | lane << 8, ilinkc[i] its CLI coefficient and, where
 // given, ilink[i] its index in cell order (linkw's).
 template <typename R>
 __global__ void item_links_kernel(long long nw, const uint2 *__restrict__ flane,
                                   const uint4 *__restrict__ seg, const uint32_t *__restrict__ boff,
                                   const unsigned long long *__restrict__ base, const R *__restrict__ linkc,
-                                  uint2 *__restrict__ fwarp, uint16_t *__restrict__ ilinkr, R *__restrict__ ilinkc,
+                                  uint4 *__restrict__ fwarp, uint16_t *__restrict__ ilinkr, R *__restrict__ ilinkc,
                                   uint32_t *__restrict__ ilink)
 {
     const int lane = threadIdx.x & 31;
@@ -207,8 +221,8 @@ __global__ void item_links_kernel(long long nw, const uint2 *__restrict__ flane,
             const uint32_t v = __shfl_up_sync(0xffffffffu, at, o);
             if (lane >= o) at += v;
         }
-        const uint32_t first = (uint32_t)base[w], total = __shfl_sync(0xffffffffu, at, 31);
-        if (lane == 0) fwarp[w] = make_uint2(total, first);
+        const uint32_t first = (uint32_t)base[w];
+        if (lane == 0) fwarp[w].y = first;
         if (n == 0) continue;
         at += first - n;
         const uint32_t c = e.x & 0x0FFFFFFFu;
@@ -673,7 +687,7 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
                                       s));
         GEO_CHECK(cudaStreamSynchronize(s));  // before items goes out of scope
     }
-    GEO_CHECK(dev_alloc(&g->fwarp, sizeof(uint2) * g->n_fwarps_padded));
+    GEO_CHECK(dev_alloc(&g->fwarp, sizeof(uint4) * g->n_fwarps_padded));
 
     if (g->n_boundary > 0) {
         const long long nb = g->n_boundary;
@@ -727,7 +741,7 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
     GEO_CHECK(dev_alloc(&d_icnt, sizeof(unsigned long long) * g->n_fwarps_padded));
     GEO_CHECK(dev_alloc(&d_ibase, sizeof(unsigned long long) * g->n_fwarps_padded));
     flane_kernel<<<grid_for(g->n_fwarps_padded * 32, 256), 256, 0, s>>>(g->n_fwarps_padded, nx, ny, nz, d_icell,
-                                                                          g->seg, g->bmask, g->flane, d_icnt);
+                                                                          g->seg, g->bmask, g->flane, g->fwarp, d_icnt);
     GEO_CHECK(cudaGetLastError());
     GEO_CHECK(exclusive_scan(d_icnt, d_ibase, g->n_fwarps_padded, s));
     if (c_double)
@@ -744,7 +758,7 @@ cudaError_t build_geometry(int nx, int ny, int nz, const double *spheres, int n_
     g->n_fluid = (long long)h_ctr[0];
     g->n_links_cli = (long long)h_ctr[1];
     g->bytes = n + sizeof(uint4) * (g->nseg_padded + g->n_active_padded) + sizeof(uint32_t) * g->n_fcell_padded +
-               (sizeof(uint2) * 32 + sizeof(uint2)) * g->n_fwarps_padded +
+               (sizeof(uint2) * 32 + sizeof(uint4)) * g->n_fwarps_padded +
                (sizeof(uint32_t) * 2 + sizeof(long long)) * g->n_boundary +
                (sizeof(double) + 2 * sizeof(uint16_t) + (wall >= 2 ? sizeof(uint32_t) : 0) +
                 (c_double ? 8 : 4) * (wall >= 2 ? 2 + kLinkW : 2)) * g->n_links;

@@ -292,9 +292,10 @@ enum { STATUS_DIVERGED = 1u, STATUS_TIMEOUT = 2u, STATUS_BOUNDS = 4u };
 // 0-27) with bit 28 x = 0, bit 29 x = nx - 1, bit 30 all the item's cells away from the y and
 // z faces (0xFFFFFFFF: padding lane); y the wall mask (as bmask below, 0 for other cells).
 // The cut links again in item order (an item's cells may have other items' between them):
-// fwarp[w] = {the item's links, the first of them}, ilinkr[i] = k | lane << 8, ilinkc[i] = its
-// linkc, ilink[i] = its index in cell order.  So a step needs no
-// dependent load and no division to find a cell's walls and its periodic fix-ups.
+// fwarp[w] = {the item's links, the first of them, z, w}, ilinkr[i] = k | lane << 8, ilinkc[i] =
+// its linkc, ilink[i] = its index in cell order.  An item that is a run (32 consecutive cells
+// without walls, rows of at least 32) is described by z and w (geometry.cu, flane_kernel)
+// without its entries in flane.  So a step needs no division to find a cell's walls and its periodic fix-ups.
 // Boundary cell b: bmask[b] bit k set when x - e_k is solid (the pull of direction k hits
 // the wall), boff[b] the index of its first link; its links are ordered by k.  Link l:
 // linkc[l] = CLI coefficient (1-2q)/(1+2q) (0 where CLI falls back to SBB), linkr[l] = k | the
@@ -341,7 +342,7 @@ struct alignas(16) InstanceDev {
     const uint4 *aseg;       // [n_active_padded]: seg entries of segments holding fluid, .w = segment
     const uint32_t *fcell;   // [n_fluid] (padded)
     const uint2 *flane;      // [32 n_fwarps_padded]
-    const uint2 *fwarp;      // [n_fwarps_padded]
+    const uint4 *fwarp;      // [n_fwarps_padded]
     const uint32_t *bmask;   // [n_boundary]
     const uint32_t *boff;    // [n_boundary]
     const void *linkc;       // [n_links], type R
@@ -417,12 +418,14 @@ struct TileDev {
     int local;           // tile index within its instance (partials slot)
     long long seg0;      // first entry of the work list
     const uint2 *flane;  // step tiles: the instance's flane and fwarp; else NULL
-    const uint2 *fwarp;
+    const uint4 *fwarp;
 };
 
 enum { KIND_AB = 0, KIND_AA_PULL = 1, KIND_AA_LOCAL = 2 };
 // Bit of the step kernel's flip argument: this step takes its tiles from the last to the first.
 constexpr int kStepBackwards = 2;
+// Bit: it reads its work-list entries without waiting to see which it needs.
+constexpr int kStepEarly = 4;
 
 // The tiles of a batched step launch, as a kernel parameter (constant bank) for batches of up
 // to kBatchMapMax instances: instance i owns tiles tile_start[i] .. tile_start[i + 1] - 1 of
@@ -434,7 +437,7 @@ struct BatchMap {
     int n;
     int tile_start[kBatchMapMax + 1];
     const uint2 *flane[kBatchMapMax];
-    const uint2 *fwarp[kBatchMapMax];
+    const uint4 *fwarp[kBatchMapMax];
 };
 struct NoBatchMap {};
 template <bool BATCH> struct MapArgT { using type = NoBatchMap; };

@@ -99,7 +99,7 @@ struct GeometryDev {
     long long n_fcell = 0, n_fcell_padded = 0;
     uint2 *flane = nullptr;        // [32 n_fwarps_padded] the step work items' cells with their
                                    // wall masks and face flags (lbm_device.cuh)
-    uint2 *fwarp = nullptr;        // [n_fwarps_padded] per work item: links, first link
+    uint4 *fwarp = nullptr;        // [n_fwarps_padded] per work item: links, first link, run
     long long n_fwarps = 0, n_fwarps_padded = 0;
     uint32_t *bmask = nullptr;     // [n_boundary]
     uint32_t *boff = nullptr;      // [n_boundary]
