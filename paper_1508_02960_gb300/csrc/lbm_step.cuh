@@ -153,23 +153,20 @@ __device__ __forceinline__ uint2 ld_keep(const uint2 *a, uint64_t pol)
     return v;
 }
 
-// Blocks per multiprocessor the register allocation is sized for.  The plain SRT and TRT
-// step of the 32- and 16-bit formats: 36 warps (56 registers a thread; measured 1-6 %
-// faster than 32 warps at 64 registers, and 40 warps spill).  MRT, the reducing and
-// interpolated-wall variants and the in-place 16-bit steps keep 32 warps (64 registers),
-// where 56 would spill (MRT at 56 spills 136 bytes and ran 3 % slower).  FP64: 8 warps.
+// Blocks per multiprocessor the register allocation is sized for: 36 warps (56 registers a
+// thread) for the single-instance steps that do not reduce (against 32 at 64 registers: FP32
+// 1-6 % faster, 16-bit AA 1-3 % from 128^3 on and 1 % slower below, FP32 MRT 1-2 %; 40 warps
+// spill and are 2-6 % slower); 32 for the reducing and interpolated-wall variants and the
+// 16-bit MRT, which would spill at 56, and for batches (36: 2-5 % slower).  FP64: 8 warps.
 #ifndef LBM_STEP_WARPS_PER_SM
 #define LBM_STEP_WARPS_PER_SM 36
 #endif
 template <int STORE, int COLL, bool RED, bool WX, int WARPS = kStepWarps, int KIND = KIND_AB, bool BATCH = false>
 constexpr int step_min_blocks()
 {
-    // the in-place steps of the 16-bit formats (stochastic rounding) spill at 56 registers: 32
-    // warps, measured 0.3-3 % faster than 36; so do a batch's steps, whose parameters come
-    // from the instance table instead of the constant bank
-    constexpr bool wide = RED || WX || COLL == COLL_MRT || BATCH ||
-                          ((STORE == ST_F16 || STORE == ST_BF16) && KIND != KIND_AB);
-    return (STORE == ST_F64 ? 8 : wide ? 32 : LBM_STEP_WARPS_PER_SM) / WARPS;
+    if (STORE == ST_F64) return 8 / WARPS;
+    constexpr bool wide = RED || WX || BATCH || (COLL == COLL_MRT && kStochastic<STORE>);
+    return (wide ? 32 : LBM_STEP_WARPS_PER_SM) / WARPS;
 }
 
 // Two values of the compute type side by side.  FP32: a register pair and Blackwell's packed
