@@ -240,6 +240,9 @@ Batch::~Batch()
     if (h_status_) cudaFreeHost(h_status_);
     if (cap_) cudaStreamDestroy(cap_);
     if (copy_) cudaStreamSynchronize(copy_);  // no copy still reads a caller's buffer
+    if (fields_) cudaStreamSynchronize(fields_);
+    cudaFree(d_field_[0]);
+    cudaFree(d_field_[1]);
     cudaFree(d_sstage_[0]);
     cudaFree(d_sstage_[1]);
     cudaFree(d_pstage_[0]);
@@ -251,6 +254,7 @@ Batch::~Batch()
     cudaFree(d_fscratch_);
     cudaFree(d_fcount_);
     if (copy_) cudaStreamDestroy(copy_);
+    if (fields_) cudaStreamDestroy(fields_);
     for (cudaEvent_t e : ev_)
         if (e) cudaEventDestroy(e);
 }
@@ -1011,7 +1015,7 @@ lbm_status Batch::moment_sums_now(int i, double *sums)
     const int nt = (int)std::max(1ll, (in.geo.n_active + block_ / 32 - 1) / (block_ / 32));
     Launch L{d_table_, nullptr, nt, block_ / 32, std::max(1, std::min(aux_grid_, (nt + 7) / 8)), 256,
              stream_};
-    CK(ops().moments(L, i, layout_, cur_of(in), aa_phase_, 1, 0, nullptr));
+    CK(ops().moments(L, i, layout_, cur_of(in), aa_phase_));
     double *ds = d_sums_ + (size_t)kRedSlots * i;
     double *hs = h_sums_ + (size_t)kRedSlots * i;
     CK(launch_final_reduce(d_table_ + i, d_tile_count_ + i, 1, ds, d_fscratch_ + (size_t)i * kFinalSlices * (RED_F + 3),
@@ -1034,6 +1038,88 @@ static cudaError_t ensure_stage(double **buf, long long *cap, long long n)
     return e;
 }
 
+// How rows of n FP64 values (directions or components) pass through staging buffers of
+// kFieldStage doubles: nk rows of nc values a pass.  Several rows of a small box, a part of
+// one of a large box; at least `together` rows, which one kernel writes.  8 MB a copy: the
+// link's 190-210 GB/s are reached (19 copies of 4 MB took 445 us where one of 84 MB took 406),
+// and the first and last pass, which overlap nothing, stay short.
+constexpr long long kFieldStage = 1ll << 20;
+struct FieldPlan {
+    long long n;
+    int rows, nk;
+    long long nc, parts, passes;
+    FieldPlan(long long n_, int rows_, int together) : n(n_), rows(rows_)
+    {
+        nk = (int)std::min<long long>(rows, std::max<long long>(together, kFieldStage / n));
+        parts = nk * n <= kFieldStage ? 1 : (nk * n + kFieldStage - 1) / kFieldStage;
+        nc = parts == 1 ? n : ((n + parts - 1) / parts + 31) / 32 * 32;
+        parts = (n + nc - 1) / nc;
+        passes = (rows + nk - 1) / nk * parts;
+    }
+    struct Pass {
+        int k0, nk;
+        long long c0, nc;
+    };
+    Pass pass(long long p) const
+    {
+        const int k0 = (int)(p / parts) * nk;
+        const long long c0 = p % parts * nc;
+        return {k0, std::min(nk, rows - k0), c0, std::min(nc, n - c0)};
+    }
+};
+
+lbm_status Batch::ensure_field_stage(long long elems)
+{
+    lbm_status st = ensure_copy_stream();
+    if (st != LBM_OK) return st;
+    // a stream of their own: a staged state's copy may be under way on the other
+    if (!fields_) CK(cudaStreamCreateWithFlags(&fields_, cudaStreamNonBlocking));
+    if (field_elems_ >= elems) return LBM_OK;
+    for (double *&b : d_field_) {
+        cudaFree(b);
+        b = nullptr;
+    }
+    field_elems_ = 0;
+    CK(dev_alloc(&d_field_[0], sizeof(double) * elems));
+    CK(dev_alloc(&d_field_[1], sizeof(double) * elems));
+    field_elems_ = elems;
+    return LBM_OK;
+}
+
+// fill(pass, buffer) launches the kernel that writes a pass; its copy runs beside the next
+// pass's kernel, which is launched first (a copy to pageable memory holds the host).
+// 96 x 80 x 72 FP64 cells, populations: 1100 us with a kernel and a copy in turn, the
+// copies alone 445.
+template <typename Fill> lbm_status Batch::fields_to_host(double *host, const FieldPlan &plan, Fill fill)
+{
+    lbm_status st = ensure_field_stage(plan.nk * plan.nc);
+    if (st != LBM_OK) return st;
+    auto produce = [&](long long p) -> lbm_status {
+        const int b = (int)(p & 1);
+        if (p >= 2) CK(cudaStreamWaitEvent(stream_, ev_[2 + b], 0));
+        CK(fill(plan.pass(p), d_field_[b]));
+        ++launches_;
+        CK(cudaEventRecord(ev_[b], stream_));
+        return LBM_OK;
+    };
+    st = produce(0);
+    if (st != LBM_OK) return st;
+    for (long long p = 0; p < plan.passes; ++p) {
+        if (p + 1 < plan.passes && (st = produce(p + 1)) != LBM_OK) return st;
+        const int b = (int)(p & 1);
+        const FieldPlan::Pass q = plan.pass(p);
+        CK(cudaStreamWaitEvent(fields_, ev_[b], 0));
+        const int blocks = q.nc == plan.n ? 1 : q.nk;  // whole rows are contiguous
+        const long long len = q.nk * q.nc / blocks;
+        for (int r = 0; r < blocks; ++r)
+            CK(cudaMemcpyAsync(host + (q.k0 + r) * plan.n + q.c0, d_field_[b] + r * q.nc, sizeof(double) * len,
+                               cudaMemcpyDeviceToHost, fields_));
+        CK(cudaEventRecord(ev_[2 + b], fields_));
+    }
+    CK(cudaStreamSynchronize(fields_));
+    return LBM_OK;
+}
+
 lbm_status Batch::get_f64(int i, double *host)
 {
     if (i < 0 || i >= size() || !host) return fail(LBM_ERR_ARG, "bad instance index or NULL buffer");
@@ -1042,15 +1128,9 @@ lbm_status Batch::get_f64(int i, double *host)
         if (st != LBM_OK) return st;
     }
     Instance &in = *inst_[i];
-    const long long n = in.geo.ncells;
-    CK(ensure_stage(&d_stage_, &stage_cells_, n));
-    for (int k = 0; k < Q; ++k) {
-        CK(ops().export_dir(d_table_, i, n, layout_, cur_of(in), aa_phase_, k, d_stage_, stream_));
-        ++launches_;
-        CK(cudaMemcpyAsync(host + (long long)k * n, d_stage_, sizeof(double) * n, cudaMemcpyDeviceToHost, stream_));
-    }
-    CK(cudaStreamSynchronize(stream_));
-    return LBM_OK;
+    return fields_to_host(host, FieldPlan(in.geo.ncells, Q, 1), [&](const FieldPlan::Pass &q, double *buf) {
+        return ops().export_f64(d_table_, i, layout_, cur_of(in), aa_phase_, q.k0, q.nk, q.c0, q.nc, buf, stream_);
+    });
 }
 
 lbm_status Batch::set_f64(int i, const double *host)
@@ -1065,11 +1145,24 @@ lbm_status Batch::set_f64(int i, const double *host)
         if (st != LBM_OK) return st;
     }
     Instance &in = *inst_[i];
-    const long long n = in.geo.ncells;
-    CK(ensure_stage(&d_stage_, &stage_cells_, n));
-    for (int k = 0; k < Q; ++k) {
-        CK(cudaMemcpyAsync(d_stage_, host + (long long)k * n, sizeof(double) * n, cudaMemcpyHostToDevice, stream_));
-        CK(ops().import_dir(d_table_, i, n, layout_, cur_of(in), k, d_stage_, stream_));
+    const FieldPlan plan(in.geo.ncells, Q, 1);
+    {
+        lbm_status st = ensure_field_stage(plan.nk * plan.nc);
+        if (st != LBM_OK) return st;
+    }
+    // what the caller's stream still does to the host buffer comes first
+    CK(cudaEventRecord(ev_[0], stream_));
+    CK(cudaStreamWaitEvent(fields_, ev_[0], 0));
+    for (long long p = 0; p < plan.passes; ++p) {
+        const int b = (int)(p & 1);
+        const FieldPlan::Pass q = plan.pass(p);
+        if (p >= 2) CK(cudaStreamWaitEvent(fields_, ev_[2 + b], 0));
+        CK(cudaMemcpyAsync(d_field_[b], host + q.k0 * plan.n + q.c0, sizeof(double) * q.nk * q.nc,
+                           cudaMemcpyHostToDevice, fields_));
+        CK(cudaEventRecord(ev_[b], fields_));
+        CK(cudaStreamWaitEvent(stream_, ev_[b], 0));
+        CK(ops().import_f64(d_table_, i, layout_, cur_of(in), q.k0, q.nk, q.c0, q.nc, d_field_[b], stream_));
+        CK(cudaEventRecord(ev_[2 + b], stream_));
         ++launches_;
     }
     if (in.geo.n_boundary > 0) {
@@ -1236,20 +1329,9 @@ lbm_status Batch::get_velocity(int i, double *host)
         if (st != LBM_OK) return st;
     }
     Instance &in = *inst_[i];
-    const long long n = in.geo.ncells;
-    CK(ensure_stage(&d_stage_, &stage_cells_, n));
-    const int nt = (int)std::max(1ll, (in.geo.n_active + block_ / 32 - 1) / (block_ / 32));
-    Launch L{d_table_, nullptr, nt, block_ / 32, std::max(1, std::min(aux_grid_, (nt + 7) / 8)), 256,
-             stream_};
-    for (int c = 0; c < 3; ++c) {
-        // all-solid segments are not in the work list: clear the whole field first
-        CK(cudaMemsetAsync(d_stage_, 0, sizeof(double) * n, stream_));
-        CK(ops().moments(L, i, layout_, cur_of(in), aa_phase_, 0, c, d_stage_));
-        ++launches_;
-        CK(cudaMemcpyAsync(host + (long long)c * n, d_stage_, sizeof(double) * n, cudaMemcpyDeviceToHost, stream_));
-    }
-    CK(cudaStreamSynchronize(stream_));
-    return LBM_OK;
+    return fields_to_host(host, FieldPlan(in.geo.ncells, 3, 3), [&](const FieldPlan::Pass &q, double *buf) {
+        return ops().velocity(d_table_, i, layout_, cur_of(in), aa_phase_, q.c0, q.nc, buf, stream_);
+    });
 }
 
 lbm_status Batch::get_flags(int i, uint8_t *host)

@@ -87,6 +87,8 @@ struct StepGroup {
     ~StepGroup();
 };
 
+struct FieldPlan;  // the passes of an FP64 field transfer (batch.cu)
+
 class Batch {
 public:
     ~Batch();
@@ -181,8 +183,14 @@ private:
     bool dirty_ = true;
     long long launches_ = 0;
     int sms_ = 0;
-    double *d_stage_ = nullptr;       // FP64 staging for import/export (one direction)
+    double *d_stage_ = nullptr;       // FP64 staging of the wall distances (one direction)
     long long stage_cells_ = 0;
+    // FP64 fields: two staging buffers of up to kFieldStage doubles and a stream of their copies
+    double *d_field_[2] = {nullptr, nullptr};
+    long long field_elems_ = 0;
+    cudaStream_t fields_ = nullptr;
+    lbm_status ensure_field_stage(long long elems);
+    template <typename Fill> lbm_status fields_to_host(double *host, const FieldPlan &plan, Fill fill);
     // state transfers: two staging buffers of one direction each, a copy stream, and
     // events: ev_[b] buffer b filled, ev_[2 + b] buffer b free again
     void *d_sstage_[2] = {nullptr, nullptr};

@@ -1,7 +1,8 @@
 // lbm_aux.cuh -- kernels around the time step: initial state, import/export of the
 // populations as FP64, velocity field and moment sums of the stored state.  All of
-// them see the state through canonical(): the post-collision population g~_k(x) in
-// either layout.
+// them see the state through stored_slot(): the post-collision population g~_k(x) in
+// either layout.  Slots are 32-bit numbers: a box whose 19 directions hold 2^32 or more is
+// refused at creation.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -9,58 +10,102 @@
 
 namespace lbm {
 
-// Where g~_k(x) of a fluid cell lives.  A-B: slot k of the current buffer.  AA after a
-// LOCAL step (or import): own slot kbar.  AA after a PULL step: slot k of x + e_k (a
+// Where g~_k(x) of a fluid cell lives.  A-B: slot k of the cell in the current buffer.  AA
+// after a LOCAL step (or import): own slot kbar.  AA after a PULL step: slot k of x + e_k (a
 // solid cell's slot when x + e_k is solid: the link's own slot there).
-template <int STORE>
-__device__ __forceinline__ long long canonical_index(const InstanceDev &I, int layout, int aa_phase,
-                                                     int cur, long long cell, int k, uint32_t wm,
-                                                     const long long (&X)[3], const long long (&Y)[3],
-                                                     const long long (&Z)[3], int &buf)
+enum Arrangement { ARR_OWN = 0, ARR_OPPOSITE = 1, ARR_NEIGHBOUR = 2 };
+__device__ __forceinline__ Arrangement arrangement(int layout, int aa_phase)
 {
-    const long long N = I.ks;
-    if (layout == 0) {
-        buf = cur;
-        return (long long)k * N + cell;
-    }
-    buf = 0;
-    (void)wm;
-    if (aa_phase == 0) return (long long)opp(k) * N + cell;
-    return (long long)k * N + X[1 + ex(k)] + Y[1 + ey(k)] + Z[1 + ez(k)];
+    return layout == 0 ? ARR_OWN : aa_phase == 0 ? ARR_OPPOSITE : ARR_NEIGHBOUR;
 }
 
-struct CellGeom {
-    long long cell;
-    int x, y, z;
-    long long X[3], Y[3], Z[3];
-    uint32_t wm, off;
-};
-
-__device__ __forceinline__ void cell_geom(const InstanceDev &I, long long cell, uint4 meta, int lane,
-                                          CellGeom &c)
+template <int STORE>
+__device__ __forceinline__ typename Store<STORE>::T *state_buffer(const InstanceDev &I, int layout, int cur)
 {
-    const int nx = I.nx, ny = I.ny, nz = I.nz;
-    c.cell = cell;
-    c.x = (int)(cell % nx);
-    const long long yz = cell / nx;
-    c.y = (int)(yz % ny);
-    c.z = (int)(yz / ny);
-    const long long nxy = (long long)nx * ny;
-    c.X[0] = c.x == 0 ? nx - 1 : c.x - 1;
-    c.X[1] = c.x;
-    c.X[2] = c.x == nx - 1 ? 0 : c.x + 1;
-    c.Y[0] = (long long)(c.y == 0 ? ny - 1 : c.y - 1) * nx;
-    c.Y[1] = (long long)c.y * nx;
-    c.Y[2] = (long long)(c.y == ny - 1 ? 0 : c.y + 1) * nx;
-    c.Z[0] = (long long)(c.z == 0 ? nz - 1 : c.z - 1) * nxy;
-    c.Z[1] = (long long)c.z * nxy;
-    c.Z[2] = (long long)(c.z == nz - 1 ? 0 : c.z + 1) * nxy;
-    c.wm = 0u;
-    c.off = 0u;
-    if ((meta.y >> lane) & 1u) {
-        const uint32_t b = meta.z + __popc(meta.y & ((1u << lane) - 1u));
-        c.wm = I.bmask[b];
-        c.off = I.boff[b];
+    return reinterpret_cast<typename Store<STORE>::T *>(layout == 0 && cur ? I.f1 : I.f0);
+}
+
+// The periodic neighbours of a cell: X[1 + a] + Y[1 + b] + Z[1 + c] is the cell at (a, b, c).
+struct Around {
+    uint32_t X[3], Y[3], Z[3];
+};
+__device__ __forceinline__ Around around(const InstanceDev &I, uint32_t cell)
+{
+    const uint32_t nx = I.nx, ny = I.ny, nz = I.nz, nxy = nx * ny;
+    const uint32_t yz = cell / nx, x = cell - yz * nx, z = yz / ny, y = yz - z * ny;
+    Around a;
+    a.X[0] = x == 0 ? nx - 1 : x - 1;
+    a.X[1] = x;
+    a.X[2] = x == nx - 1 ? 0 : x + 1;
+    a.Y[0] = (y == 0 ? ny - 1 : y - 1) * nx;
+    a.Y[1] = y * nx;
+    a.Y[2] = (y == ny - 1 ? 0 : y + 1) * nx;
+    a.Z[0] = (z == 0 ? nz - 1 : z - 1) * nxy;
+    a.Z[1] = z * nxy;
+    a.Z[2] = (z == nz - 1 ? 0 : z + 1) * nxy;
+    return a;
+}
+__device__ __forceinline__ uint32_t slot_towards(const InstanceDev &I, const Around &a, int k)
+{
+    return (uint32_t)k * (uint32_t)I.ks + a.X[1 + ex(k)] + a.Y[1 + ey(k)] + a.Z[1 + ez(k)];
+}
+// One direction's slot (the neighbours, with their divisions, only where they are needed).
+__device__ __forceinline__ uint32_t stored_slot(const InstanceDev &I, Arrangement arr, uint32_t cell, int k)
+{
+    if (arr == ARR_NEIGHBOUR) return slot_towards(I, around(I, cell), k);
+    return (uint32_t)(arr == ARR_OWN ? k : opp(k)) * (uint32_t)I.ks + cell;
+}
+// All 19.
+template <int STORE>
+__device__ __forceinline__ void load_stored(const InstanceDev &I, const typename Store<STORE>::T *f, Arrangement arr,
+                                            uint32_t cell, typename Store<STORE>::R (&g)[Q])
+{
+    using S = Store<STORE>;
+    if (arr == ARR_NEIGHBOUR) {
+        const Around a = around(I, cell);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) g[k] = S::load(f + slot_towards(I, a, k), I.inv_scale);
+    } else {
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+            g[k] = S::load(f + ((uint32_t)(arr == ARR_OWN ? k : opp(k)) * (uint32_t)I.ks + cell), I.inv_scale);
+    }
+}
+
+// Momentum sum_k e_k g_k in FP64.  GB300 runs an FP64 warp instruction per 19 cycles of a
+// multiprocessor, so the terms that are no part of a component are left out: 21 operations
+// from the differences of opposite directions, where multiplying all 19 populations by the
+// components of e_k takes 57 (the velocity field of 96 x 80 x 72 cells in one pass instead of
+// three of those: see velocity_kernel).  A population that is infinite or NaN takes the long
+// form, whose 0 * g makes every component of the cell show it.
+template <typename R> __device__ __forceinline__ void momentum(const R (&g)[Q], double (&j)[3])
+{
+    uint32_t top = 0;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        if constexpr (sizeof(R) == 8) top = max(top, (uint32_t)__double2hiint(g[k]) & 0x7fffffffu);
+        else top = max(top, __float_as_uint(g[k]) & 0x7fffffffu);
+    }
+    j[0] = j[1] = j[2] = 0.0;
+    if (top >= (sizeof(R) == 8 ? 0x7ff00000u : 0x7f800000u)) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            j[0] += ex(k) * (double)g[k];
+            j[1] += ey(k) * (double)g[k];
+            j[2] += ez(k) * (double)g[k];
+        }
+        return;
+    }
+#pragma unroll
+    for (int k = 1; k < Q; ++k) {
+        if (opp(k) < k) continue;
+        const double d = (double)g[k] - (double)g[opp(k)];
+        const int e[3] = {ex(k), ey(k), ez(k)};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (e[a] > 0) j[a] += d;
+            if (e[a] < 0) j[a] -= d;
+        }
     }
 }
 
@@ -94,15 +139,15 @@ __global__ void init_kernel(const InstanceDev *__restrict__ table, int inst, int
     for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < N;
          cell += (long long)gridDim.x * blockDim.x) {
         const uint4 meta = I.seg[cell >> 5];
-        T *f = reinterpret_cast<T *>(layout == 0 ? (cur ? I.f1 : I.f0) : I.f0);
-        if ((meta.x >> lane) & 1u) {
+        T *f = state_buffer<STORE>(I, layout, cur);
+        // at rest every g is 0, without the FP64 arithmetic (512^3: 24 ms with it)
+        if (amp == 0.0 || ((meta.x >> lane) & 1u)) {
 #pragma unroll
             for (int k = 0; k < Q; ++k) f[(long long)k * I.ks + cell] = S::pack(0.0f);
             continue;
         }
-        double u[3] = {0.0, 0.0, 0.0};
-        if (amp != 0.0)
-            for (int a = 0; a < 3; ++a) u[a] = amp * hash_uniform_pm1(seed, cell, a);
+        double u[3];
+        for (int a = 0; a < 3; ++a) u[a] = amp * hash_uniform_pm1(seed, cell, a);
         const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
 #pragma unroll
         for (int k = 0; k < Q; ++k) {
@@ -128,14 +173,14 @@ __global__ void wall_prepare_kernel(const InstanceDev *__restrict__ table, int i
     using T = typename S::T;
     using R = typename S::R;
     const InstanceDev &I = table[inst];
-    T *f = reinterpret_cast<T *>(layout == 0 && cur ? I.f1 : I.f0);
+    T *f = state_buffer<STORE>(I, layout, cur);
     const R *linkc = reinterpret_cast<const R *>(I.linkc);
-    const long long ks = I.ks, nx = I.nx, ny = I.ny, nz = I.nz;
+    const long long ks = I.ks;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nb;
          b += (long long)gridDim.x * blockDim.x) {
         const long long cell = bcell[b];
         const uint32_t wm = I.bmask[b], off = I.boff[b];
-        const long long x = cell % nx, yz = cell / nx, y = yz % ny, z = yz / ny;
+        const Around at = around(I, (uint32_t)cell);
         const RoundKey key = round_key<STORE>((uint32_t)cell, I.cf.hash_off);
         // the cell's moments at t (for IEBB): the post-collision state conserves them
         R drho = R(0), u[3] = {R(0), R(0), R(0)};
@@ -173,60 +218,51 @@ __global__ void wall_prepare_kernel(const InstanceDev *__restrict__ table, int i
                 const R cq = I.wall == 1 ? linkc[l] : R(0);
                 sv = wall_own_part(I.wall, cq, C, B);
             }
-            const long long src = (x - ex(k) + nx) % nx + nx * ((y - ey(k) + ny) % ny + ny * ((z - ez(k) + nz) % nz));
+            const uint32_t src = at.X[1 - ex(k)] + at.Y[1 - ey(k)] + at.Z[1 - ez(k)];
             put1<STORE>(f + (long long)(layout == 0 ? k : kb) * ks + src, sv * R(I.scale), key, k);
         }
     }
 }
 
-// Import direction k from FP64 f (cells of one direction): g = f - w rho0.
+// Import of FP64 f into directions k0 + blockIdx.y, cells c0 ... c0 + nc - 1, from
+// fk[blockIdx.y * nc + cell - c0]: g = f - w rho0.  These transfers run at the speed of the
+// host link (190-210 GB/s); the kernels only have to stay ahead of it, a pass in one staging
+// buffer while the other is being copied.
 template <int STORE>
-__global__ void import_kernel(const InstanceDev *__restrict__ table, int inst, int layout, int cur, int k,
-                              const double *__restrict__ fk)
+__global__ void import_kernel(const InstanceDev *__restrict__ table, int inst, int layout, int cur, int k0,
+                              long long c0, long long nc, const double *__restrict__ fk)
 {
     using S = Store<STORE>;
-    using T = typename S::T;
     const InstanceDev &I = table[inst];
-    const long long N = I.ncells;
-    const int lane = threadIdx.x & 31;
+    const int k = k0 + (int)blockIdx.y;
     const double wr = weight(k) * I.rho0;
-    for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < N;
-         cell += (long long)gridDim.x * blockDim.x) {
-        const uint4 meta = I.seg[cell >> 5];
-        T *f = reinterpret_cast<T *>(layout == 0 ? (cur ? I.f1 : I.f0) : I.f0);
-        const long long slot = (long long)(layout == 0 ? k : opp(k)) * I.ks + cell;
-        if ((meta.x >> lane) & 1u) {
-            f[slot] = S::pack(0.0f);
-            continue;
-        }
-        f[slot] = S::pack((typename S::R)(fk[cell] - wr) * I.scale);
+    auto *f = state_buffer<STORE>(I, layout, cur) + (long long)(layout == 0 ? k : opp(k)) * I.ks;
+    fk += (long long)blockIdx.y * nc;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long cell = c0 + i;
+        const bool solid = (I.seg[cell >> 5].x >> (cell & 31)) & 1u;
+        f[cell] = solid ? S::pack(0.0f) : S::pack((typename S::R)(fk[i] - wr) * I.scale);
     }
 }
 
-// Export direction k as FP64 f = w rho0 + g~ (0 in solid cells).
+// Export as FP64 f = w rho0 + g~ (0 in solid cells), arguments as import_kernel's.
 template <int STORE>
 __global__ void export_kernel(const InstanceDev *__restrict__ table, int inst, int layout, int cur,
-                              int aa_phase, int k, double *__restrict__ fk)
+                              int aa_phase, int k0, long long c0, long long nc, double *__restrict__ fk)
 {
     using S = Store<STORE>;
-    using T = typename S::T;
     const InstanceDev &I = table[inst];
-    const long long N = I.ncells;
-    const int lane = threadIdx.x & 31;
+    const int k = k0 + (int)blockIdx.y;
     const double wr = weight(k) * I.rho0;
-    for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < N;
-         cell += (long long)gridDim.x * blockDim.x) {
-        const uint4 meta = I.seg[cell >> 5];
-        if ((meta.x >> lane) & 1u) {
-            fk[cell] = 0.0;
-            continue;
-        }
-        CellGeom c;
-        cell_geom(I, cell, meta, lane, c);
-        int buf;
-        const long long idx = canonical_index<STORE>(I, layout, aa_phase, cur, cell, k, c.wm, c.X, c.Y, c.Z, buf);
-        const T *f = reinterpret_cast<const T *>(buf ? I.f1 : I.f0);
-        fk[cell] = wr + (double)S::load(f + idx, I.inv_scale);
+    const Arrangement arr = arrangement(layout, aa_phase);
+    const auto *f = state_buffer<STORE>(I, layout, cur);
+    fk += (long long)blockIdx.y * nc;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long cell = c0 + i;
+        const bool solid = (I.seg[cell >> 5].x >> (cell & 31)) & 1u;
+        fk[i] = solid ? 0.0 : wr + (double)S::load(f + stored_slot(I, arr, (uint32_t)cell, k), I.inv_scale);
     }
 }
 
@@ -240,16 +276,12 @@ __global__ void state_gather_kernel(const InstanceDev *__restrict__ table, int i
     using T = typename Store<STORE>::T;
     const InstanceDev &I = table[inst];
     const int k = k0 + (int)blockIdx.y;
+    const Arrangement arr = arrangement(layout, aa_phase);
+    const T *f = state_buffer<STORE>(I, layout, cur);
     out += (long long)blockIdx.y * nf;
     for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < nf;
          j += (long long)gridDim.x * blockDim.x) {
-        const long long cell = I.fcell[j];
-        const int lane = (int)(cell & 31);
-        CellGeom c;
-        cell_geom(I, cell, I.seg[cell >> 5], lane, c);
-        int buf;
-        const long long idx = canonical_index<STORE>(I, layout, aa_phase, cur, cell, k, c.wm, c.X, c.Y, c.Z, buf);
-        out[j] = reinterpret_cast<const T *>(buf ? I.f1 : I.f0)[idx];
+        out[j] = f[stored_slot(I, arr, I.fcell[j], k)];
     }
 }
 
@@ -265,7 +297,7 @@ __global__ void state_scatter_kernel(const InstanceDev *__restrict__ table, int 
     const InstanceDev &I = table[inst];
     const int k = k0 + (int)blockIdx.y;
     in += (long long)blockIdx.y * nf;
-    T *f = reinterpret_cast<T *>(layout == 0 ? (cur ? I.f1 : I.f0) : I.f0);
+    T *f = state_buffer<STORE>(I, layout, cur);
     for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < nf;
          j += (long long)gridDim.x * blockDim.x) {
         const long long cell = I.fcell[j];
@@ -273,59 +305,67 @@ __global__ void state_scatter_kernel(const InstanceDev *__restrict__ table, int 
     }
 }
 
-// Moments of the stored post-collision state of every fluid cell of an instance, one warp per
-// chunk of chunk_segs active segments.  mode 0: write the velocity component `comp` to out[cell] of fluid cells (the
-// caller clears out first).  mode 1: chunk partial sums (drho, u_x, u_y, u_z) into
+// Velocity of cells c0 ... c0 + nc - 1 from the stored post-collision state (0 in solid
+// cells): out[a * nc + cell - c0] = component a.
+template <int STORE>
+__global__ void __launch_bounds__(128) velocity_kernel(const InstanceDev *__restrict__ table, int inst, int layout,
+                                                       int cur, int aa_phase, long long c0, long long nc,
+                                                       double *__restrict__ out)
+{
+    const InstanceDev &I = table[inst];
+    const Arrangement arr = arrangement(layout, aa_phase);
+    const auto *f = state_buffer<STORE>(I, layout, cur);
+    const double rho0 = I.rho0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long cell = c0 + i;
+        double j[3] = {0.0, 0.0, 0.0};
+        if (!((I.seg[cell >> 5].x >> (cell & 31)) & 1u)) {
+            typename Store<STORE>::R g[Q];
+            load_stored<STORE>(I, f, arr, (uint32_t)cell, g);
+            momentum(g, j);
+            if (rho0 != 1.0)  // an FP64 division is 10 FP64 instructions
+                for (int a = 0; a < 3; ++a) j[a] /= rho0;
+        }
+        for (int a = 0; a < 3; ++a) out[a * nc + i] = j[a];
+    }
+}
+
+// Moment sums of the stored post-collision state of every fluid cell of an instance, one
+// warp per chunk of chunk_segs active segments: chunk partial sums (drho, u_x, u_y, u_z) into
 // I.partials, in FP64 in a fixed order; the force slots, which only a step defines, are
 // written as 0.
 template <int STORE>
 __global__ void __launch_bounds__(256) moments_kernel(const InstanceDev *__restrict__ table,
                                                       int inst, int nchunks, int chunk_segs,
-                                                      int layout, int cur, int aa_phase, int mode, int comp,
-                                                      double *__restrict__ out)
+                                                      int layout, int cur, int aa_phase)
 {
-    using S = Store<STORE>;
-    using T = typename S::T;
+    const InstanceDev &I = table[inst];
+    const Arrangement arr = arrangement(layout, aa_phase);
+    const auto *f = state_buffer<STORE>(I, layout, cur);
     const int lane = threadIdx.x & 31;
     const int gw = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     const int nw = (int)((gridDim.x * (long long)blockDim.x) >> 5);
     for (int c = gw; c < nchunks; c += nw) {
-        const InstanceDev &I = table[inst];
         const long long seg0 = (long long)c * chunk_segs;  // chunk c of the active segments
         const int n_e = min(chunk_segs, (int)((long long)I.n_active - seg0));
         double a[4] = {0.0, 0.0, 0.0, 0.0};
         for (int i = 0; i < n_e; ++i) {
             const uint4 meta = I.aseg[seg0 + i];
-            const long long cell = (long long)meta.w * 32 + lane;
             if ((meta.x >> lane) & 1u) continue;
-            CellGeom cg;
-            cell_geom(I, cell, meta, lane, cg);
-            double drho = 0.0, j[3] = {0.0, 0.0, 0.0};
+            typename Store<STORE>::R g[Q];
+            load_stored<STORE>(I, f, arr, meta.w * 32u + (uint32_t)lane, g);
+            double j[3];
+            momentum(g, j);
 #pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                int buf;
-                const long long idx =
-                    canonical_index<STORE>(I, layout, aa_phase, cur, cell, k, cg.wm, cg.X, cg.Y, cg.Z, buf);
-                const T *f = reinterpret_cast<const T *>(buf ? I.f1 : I.f0);
-                const double g = (double)S::load(f + idx, I.inv_scale);
-                drho += g;
-                j[0] += ex(k) * g;
-                j[1] += ey(k) * g;
-                j[2] += ez(k) * g;
-            }
-            if (mode == 0) {
-                out[cell] = j[comp] / I.rho0;
-            } else {
-                a[0] += drho;
-                for (int d = 0; d < 3; ++d) a[1 + d] += j[d] / I.rho0;
-            }
+            for (int k = 0; k < Q; ++k) a[0] += (double)g[k];
+            for (int d = 0; d < 3; ++d) a[1 + d] += j[d];
         }
-        if (mode == 1) {
 #pragma unroll
-            for (int d = 0; d < 4; ++d) a[d] = warp_sum(a[d]);
-            if (lane == 0)
-                for (int d = 0; d < kRedSlots; ++d) I.partials[(long long)c * kRedSlots + d] = d < 4 ? a[d] : 0.0;
-        }
+        for (int d = 0; d < 4; ++d) a[d] = warp_sum(a[d]);
+        if (lane == 0)
+            for (int d = 0; d < kRedSlots; ++d)
+                I.partials[(long long)c * kRedSlots + d] = d == 0 ? a[0] : d < 4 ? a[d] / I.rho0 : 0.0;
     }
 }
 

@@ -183,18 +183,20 @@ cudaError_t init(const InstanceDev *table, int inst, long long n, int layout, in
 }
 
 template <int STORE>
-cudaError_t import_dir(const InstanceDev *table, int inst, long long n, int layout, int cur, int k,
-                       const double *fk, cudaStream_t s)
+cudaError_t import_f64(const InstanceDev *table, int inst, int layout, int cur, int k, int nk, long long c0,
+                       long long nc, const double *fk, cudaStream_t s)
 {
-    import_kernel<STORE><<<flat_grid(n, 256), 256, 0, s>>>(table, inst, layout, cur, k, fk);
+    const dim3 grid((unsigned)flat_grid(nc, 256), (unsigned)nk);
+    import_kernel<STORE><<<grid, 256, 0, s>>>(table, inst, layout, cur, k, c0, nc, fk);
     return cudaGetLastError();
 }
 
 template <int STORE>
-cudaError_t export_dir(const InstanceDev *table, int inst, long long n, int layout, int cur, int aa_phase,
-                       int k, double *fk, cudaStream_t s)
+cudaError_t export_f64(const InstanceDev *table, int inst, int layout, int cur, int aa_phase, int k, int nk,
+                       long long c0, long long nc, double *fk, cudaStream_t s)
 {
-    export_kernel<STORE><<<flat_grid(n, 256), 256, 0, s>>>(table, inst, layout, cur, aa_phase, k, fk);
+    const dim3 grid((unsigned)flat_grid(nc, 256), (unsigned)nk);
+    export_kernel<STORE><<<grid, 256, 0, s>>>(table, inst, layout, cur, aa_phase, k, c0, nc, fk);
     return cudaGetLastError();
 }
 
@@ -214,10 +216,19 @@ cudaError_t state_dir(const InstanceDev *table, int inst, long long nf, int layo
 }
 
 template <int STORE>
-cudaError_t moments(const Launch &L, int inst, int layout, int cur, int aa_phase, int mode, int comp, double *out)
+cudaError_t velocity(const InstanceDev *table, int inst, int layout, int cur, int aa_phase, long long c0, long long nc,
+                     double *out, cudaStream_t s)
+{
+    velocity_kernel<STORE>
+        <<<flat_grid(nc, 128), 128, 0, s>>>(table, inst, layout, cur, aa_phase, c0, nc, out);
+    return cudaGetLastError();
+}
+
+template <int STORE>
+cudaError_t moments(const Launch &L, int inst, int layout, int cur, int aa_phase)
 {
     moments_kernel<STORE><<<L.grid, L.block, 0, L.stream>>>(L.table, inst, L.ntiles, L.chunk_segs, layout, cur,
-                                                            aa_phase, mode, comp, out);
+                                                            aa_phase);
     return cudaGetLastError();
 }
 
@@ -236,9 +247,10 @@ FormatOps make_ops()
     FormatOps o;
     o.step = &step<STORE>;
     o.init = &init<STORE>;
-    o.import_dir = &import_dir<STORE>;
-    o.export_dir = &export_dir<STORE>;
+    o.import_f64 = &import_f64<STORE>;
+    o.export_f64 = &export_f64<STORE>;
     o.state_dir = &state_dir<STORE>;
+    o.velocity = &velocity<STORE>;
     o.moments = &moments<STORE>;
     o.wall_prepare = &wall_prepare<STORE>;
     o.step_tma = &step_tma<STORE>;

@@ -62,16 +62,19 @@ struct FormatOps {
                         int warps);
     cudaError_t (*init)(const InstanceDev *table, int inst, long long ncells, int layout, int cur,
                         double amp, unsigned long long seed, cudaStream_t s);
-    cudaError_t (*import_dir)(const InstanceDev *table, int inst, long long ncells, int layout, int cur,
-                              int k, const double *fk, cudaStream_t s);
-    cudaError_t (*export_dir)(const InstanceDev *table, int inst, long long ncells, int layout, int cur,
-                              int aa_phase, int k, double *fk, cudaStream_t s);
+    // FP64 f of directions k .. k + nk - 1 and cells c0 .. c0 + nc - 1, as [nk][nc]
+    cudaError_t (*import_f64)(const InstanceDev *table, int inst, int layout, int cur, int k, int nk, long long c0,
+                              long long nc, const double *fk, cudaStream_t s);
+    cudaError_t (*export_f64)(const InstanceDev *table, int inst, int layout, int cur, int aa_phase, int k, int nk,
+                              long long c0, long long nc, double *fk, cudaStream_t s);
     // fluid-cell state of directions k .. k + nk - 1 in the storage type: to_host = 1
     // gathers them into buf [nk][n_fluid], 0 scatters them from buf (the step-0 arrangement)
     cudaError_t (*state_dir)(const InstanceDev *table, int inst, long long n_fluid, int layout, int cur,
                              int aa_phase, int k, int nk, void *buf, int to_host, cudaStream_t s);
-    cudaError_t (*moments)(const Launch &L, int inst, int layout, int cur, int aa_phase, int mode, int comp,
-                           double *out);
+    // velocity of cells c0 .. c0 + nc - 1, as [3][nc]
+    cudaError_t (*velocity)(const InstanceDev *table, int inst, int layout, int cur, int aa_phase, long long c0,
+                            long long nc, double *out, cudaStream_t s);
+    cudaError_t (*moments)(const Launch &L, int inst, int layout, int cur, int aa_phase);
     // TMA brick step (non-reducing, single instance, A-B); one: the instance's parameters
     cudaError_t (*step_tma)(int coll, int wx, const TmaLaunch &T, const InstanceDev &one, int flip);
     // once per kernel, before any launch or capture: opt in to its shared memory; returns
