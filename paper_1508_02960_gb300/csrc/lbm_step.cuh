@@ -17,7 +17,7 @@
 //   collide   SRT, TRT or MRT relaxation towards Eq. equilibrium;
 //   store     A-B: to the other buffer; AA: in place (see below).
 // The 19 pulls are issued unconditionally: a solid source slot holds the own-cell part
-// of the wall rule (A-B layout, see finish_cell) or is replaced by the wall rule (AA), so
+// of the wall rule, left by the previous step (see WallStage), so
 // no pull waits on the boundary table; the wall code runs only for boundary cells.
 //
 // AA layout (in-place, one buffer).  PULL steps read g~_k(x - e_k) from slot kbar of
@@ -46,9 +46,12 @@ __device__ __forceinline__ double warp_sum(double v)
 }
 
 // Loads of population values.  An A-B step reads a buffer that no thread of the step
-// writes, through the read-only (non-coherent) path.  The AA steps update their buffer, and
-// the CLI link buffer, in place: a non-coherent load there is not allowed (the compiler may
-// then order it after a store of the same thread), so they load plainly.
+// writes, through the read-only (non-coherent) path.  The AA steps update their buffer in
+// place: a non-coherent load there is not allowed (the compiler may then order it after a
+// store of the same thread), so they load plainly.  Both with the ordinary L2 policy: loads
+// marked evict-first take A-B 128^3 from 42.4 to 45 us a step and 256^3 from 280 to 330
+// (neighbouring items share sectors); the first 20 MB of the tiles marked evict-last, loads
+// and stores, gain 2 % there and lose 1-2 % in the AA layout.
 template <int KIND, typename T> __device__ __forceinline__ T ld_pop(const T *p)
 {
     if constexpr (KIND == KIND_AB) return __ldg(p);
