@@ -159,9 +159,8 @@ __global__ void fluid_scatter_kernel(long long n, const uint4 *__restrict__ seg,
 //   y: the wall mask (bit k: x - e_k solid);
 // and fwarp[w] = {x: the item's links (item_links_kernel: y the first of them), z, w}: an item
 // that is a run, 32 consecutive cells without walls in rows of at least 32, is described by
-// z = bit 31 | its first cell | bit 30 as above and w = the lane of the cell at x = 0 (32: the
-// cell after the last; 63: none), and a step does not read its entries in flane; other items
-// have z = 0.  count[w] = x.
+// z and w (lbm_device.cuh, run_entry), and a step may make its entries instead of reading them in
+// flane; other items have z = 0.  count[w] = x.
 __global__ void flane_kernel(long long nw, int nx, int ny, int nz, const uint32_t *__restrict__ icell,
                              const uint4 *__restrict__ seg, const uint32_t *__restrict__ bmask,
                              uint2 *__restrict__ flane, uint4 *__restrict__ fwarp, unsigned long long *__restrict__ count)
@@ -189,12 +188,9 @@ __global__ void flane_kernel(long long nw, int nx, int ny, int nz, const uint32_
         flane[w * 32 + lane] = make_uint2(ce, wm);
         const uint32_t c0 = __shfl_sync(0xffffffffu, c, 0);
         const bool run = __all_sync(0xffffffffu, live && c == c0 + (uint32_t)lane) && links == 0 && nx >= 32;
-        const unsigned at0 = __ballot_sync(0xffffffffu, live && x == 0u);
-        const bool end = __shfl_sync(0xffffffffu, x, 31) == (uint32_t)nx - 1u;
         if (lane == 0) {
             count[w] = links;
-            fwarp[w] = run ? make_uint4(0u, 0u, c0 | 1u << 31 | (inner ? 1u << 30 : 0u),
-                                        at0 ? (uint32_t)__ffs(at0) - 1u : end ? 32u : 63u)
+            fwarp[w] = run ? make_uint4(0u, 0u, c0 | 1u << 31 | (inner ? 1u << 30 : 0u), run_faces(x, (uint32_t)nx))
                            : make_uint4(links, 0u, 0u, 0u);
         }
     }

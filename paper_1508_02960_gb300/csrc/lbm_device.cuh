@@ -294,8 +294,8 @@ enum { STATUS_DIVERGED = 1u, STATUS_TIMEOUT = 2u, STATUS_BOUNDS = 4u };
 // The cut links again in item order (an item's cells may have other items' between them):
 // fwarp[w] = {the item's links, the first of them, z, w}, ilinkr[i] = k | lane << 8, ilinkc[i] =
 // its linkc, ilink[i] = its index in cell order.  An item that is a run (32 consecutive cells
-// without walls, rows of at least 32) is described by z and w (geometry.cu, flane_kernel)
-// without its entries in flane.  So a step needs no division to find a cell's walls and its periodic fix-ups.
+// without walls, rows of at least 32) is described by z and w (run_entry) without its entries
+// in flane.  So a step needs no division to find a cell's walls and its periodic fix-ups.
 // Boundary cell b: bmask[b] bit k set when x - e_k is solid (the pull of direction k hits
 // the wall), boff[b] the index of its first link; its links are ordered by k.  Link l:
 // linkc[l] = CLI coefficient (1-2q)/(1+2q) (0 where CLI falls back to SBB), linkr[l] = k | the
@@ -420,6 +420,27 @@ struct TileDev {
     const uint2 *flane;  // step tiles: the instance's flane and fwarp; else NULL
     const uint4 *fwarp;
 };
+
+// The entry of a work item that is a run (fwarp's z and w): z = bit 31 | bit 30 (every cell away
+// from the y and z faces) | its first cell; w = run_faces.  A run lies in rows of at least 32 cells, so
+// that at most one of its cells is at x = 0 and at most one at x = nx - 1: adjacent ones, or, when
+// the run is a whole row of 32, the first and the last.
+constexpr uint32_t kNoLane = 0xFFu;
+// The lanes of the cells at x = 0 (bits 0-7) and at x = nx - 1 (bits 8-15) of a run that begins at
+// x0; kNoLane: none.
+__host__ __device__ inline uint32_t run_faces(uint32_t x0, uint32_t nx)
+{
+    const uint32_t first = x0 == 0u ? 0u : nx - x0, last = nx - 1u - x0;
+    return (first < 32u ? first : kNoLane) | (last < 32u ? last : kNoLane) << 8;
+}
+// What flane holds for a lane of it.
+__host__ __device__ inline uint32_t run_entry(uint32_t z, uint32_t w, uint32_t lane)
+{
+    uint32_t e = (z & 0x4FFFFFFFu) + lane;
+    if (lane == (w & 0xFFu)) e |= 1u << 28;
+    if (lane == w >> 8) e |= 1u << 29;
+    return e;
+}
 
 enum { KIND_AB = 0, KIND_AA_PULL = 1, KIND_AA_LOCAL = 2 };
 // Bit of the step kernel's flip argument: this step takes its tiles from the last to the first.

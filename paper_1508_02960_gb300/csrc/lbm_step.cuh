@@ -899,9 +899,7 @@ __device__ __forceinline__ ItemEntry load_entry(const uint2 *flane, const uint4 
     e.links = make_uint2(h.x, h.y);
     if (!early) {
         if (h.z >> 31) {
-            e.cell.x = (h.z & 0x4FFFFFFFu) + (uint32_t)lane;
-            if ((uint32_t)lane == h.w) e.cell.x |= 1u << 28;
-            if ((uint32_t)lane + 1u == h.w) e.cell.x |= 1u << 29;
+            e.cell.x = run_entry(h.z, h.w, (uint32_t)lane);
         } else if (ok) {
             e.cell = ld_keep(flane + (w * 32u + (uint32_t)lane), keep);
         }
