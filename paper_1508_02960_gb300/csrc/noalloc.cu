@@ -20,6 +20,7 @@
 #include <mutex>
 
 #include "batch.h"
+#include "fixed_sum.cuh"
 
 namespace lbm {
 namespace {
@@ -45,21 +46,6 @@ __host__ __device__ inline long long noalloc_cells_per_block(long long n)
 // nothing (equilibrium populations span 2^4).  Smaller ones are truncated below 2^-57 of it,
 // where an FP64 sum of the cell would round at 2^-53.
 constexpr int kFixedTop = 57;
-
-struct FixedSum {           // sum = hi 2^32 + lo, as the sums of the halves of the terms
-    long long hi;
-    unsigned long long lo;
-    __device__ __forceinline__ void add(long long x)
-    {
-        lo += (unsigned long long)(unsigned)x;
-        hi += x >> 32;
-    }
-};
-
-__device__ __forceinline__ double to_double(__int128 t)
-{
-    return (double)(long long)(t >> 64) * 18446744073709551616.0 + (double)(unsigned long long)t;
-}
 
 // Sums of m cells held in units of exponent field E, as FP64: .v[0] = sum rho - m rho0,
 // .v[1..3] = sum j.  Out of line: rare in a warp's loop, once at the end of a block.
