@@ -352,7 +352,8 @@ LBM_API lbm_status lbm_synchronize(lbm_ctx *ctx);
  *             direction order above; entries of solid cells are ignored
  *   solid_dev device, n_cells flags (1 = solid), or NULL when every cell is fluid
  *   sums_dev  device, 4 doubles out: sums over fluid cells of (rho - rho0, u_x, u_y, u_z),
- *             u = rho0^-1 sum e_k f_k, reduced in a fixed order
+ *             u = rho0^-1 sum e_k f_k, reduced in a fixed order.  A cell's sums are exact or
+ *             rounded as FP64 sums of its values
  *   cuda_stream  stream the two kernels are queued on (NULL = legacy default stream)
  * Calls no cudaMalloc or cudaFree: block sums go to a fixed 256 KiB scratch array inside
  * the library, held by every GPU that loads it.  n_cells is limited to 268,435,456

@@ -31,21 +31,21 @@ constexpr long long kNoAllocMaxCells = (long long)kNoAllocMaxBlocks * 32768;
 
 static __device__ __align__(256) double g_noalloc_partials[kNoAllocMaxBlocks * 4];
 
-// Blocks of a call: 8 to a multiprocessor (its full complement of threads), each over one
-// contiguous range of whole rounds of its threads; small fields take a round a block.  Fixed
-// by the cell count alone, so that the order of the sums is.
+// Blocks of a call: 8 for each multiprocessor, which holds two at a time (128 registers a thread),
+// each over one contiguous range of whole rounds of its threads; small fields take a round a
+// block.  Fixed by the cell count alone, so that the order of the sums is.
 constexpr long long kNoAllocBlocks = 152 * 8;
 __host__ __device__ inline long long noalloc_cells_per_block(long long n)
 {
     return ((n + kNoAllocBlocks - 1) / kNoAllocBlocks + kNoAllocThreads - 1) / kNoAllocThreads * kNoAllocThreads;
 }
 
-// Fixed-point sums.  A cell's 19 values, the largest of which has the exponent field E, are
-// taken as integers in units of 2^(E - 1080): 1.52-bit mantissas at bit 57 and
-// below, so that 19 of them fit 63 bits and values down to 2^-5 of the largest power lose
-// nothing (equilibrium populations span 2^4).  Smaller ones are truncated below 2^-57 of it,
-// where an FP64 sum of the cell would round at 2^-53.
-constexpr int kFixedTop = 57;
+// Fixed-point sums.  Values whose exponent field is at most E are integers in units of
+// 2^(E - 1080): 1.52-bit mantissas at bit 57 and below, so that 19 of them fit 63 bits, and those
+// with exponent fields from E - kFixedSpan on (5: equilibrium populations span 4) lose nothing.  A cell
+// is summed in integers only if all of its values are such, so that its sums are exact where an FP64
+// sum would round; the unit is kept from cell to cell while they are.
+constexpr int kFixedTop = 57, kFixedSpan = kFixedTop - 52;
 
 // Sums of m cells held in units of exponent field E, as FP64: .v[0] = sum rho - m rho0,
 // .v[1..3] = sum j.  Out of line: rare in a warp's loop, once at the end of a block.
@@ -72,13 +72,16 @@ __device__ __noinline__ Sums4 to_sums(FixedSum s0, FixedSum s1, FixedSum s2, Fix
     return a;
 }
 
-// Block b sums its range of the fluid cells; partial -> partials[b].  Bound: one read of the
-// field.  The sums are integer sums because FP64 arithmetic is slow on GB300 (a warp
-// instruction per 19 cycles a multiprocessor): the 49 FP64 additions of a cell would take four
-// times as long as its loads, the 340 integer instructions they become take 0.8 of it.
-// 160^3 cells, 43 % of them solid at random: 1044 us with FP64 sums in 125 blocks of fixed
-// size -> 160 us.  Values out of the integers' reach (infinities, NaN, a cell's
-// largest value below 2^-959) are summed in FP64.
+// Block b sums its range of the fluid cells; partial -> partials[b].  The sums are integer sums
+// because FP64 arithmetic is slow on GB300 (a warp instruction per 19 cycles a multiprocessor):
+// the 49 FP64 additions of a cell would take four times as long as its loads.  The 360 integer
+// instructions they become, by 16 warps a multiprocessor (a cell's 19 values are held until
+// their exponents are known), leave it at 1.75 times the sectors it reads: 160^3 cells, 43 % of
+// them solid at random, 1044 us with FP64 sums in 125 blocks of fixed size -> 165 us,
+// and 255 when the largest population crosses a power of two from cell to cell (rho0 = 0.75, 1.5,
+// 3: lanes change their unit).  Cells that are not exact in integers (values of very different
+// sizes, infinities, NaN, a largest value below 2^-959) are summed in FP64: 770 us for a field
+// with such cells among the others of every warp.
 __global__ void __launch_bounds__(kNoAllocThreads, 2) noalloc_partials_kernel(const double *__restrict__ f,
                                                                           const uint8_t *__restrict__ solid,
                                                                           long long n, double rho0,
@@ -102,26 +105,38 @@ __global__ void __launch_bounds__(kNoAllocThreads, 2) noalloc_partials_kernel(co
 #pragma unroll
         for (int k = 0; k < Q; ++k)
             v[k] = live ? __ldg(reinterpret_cast<const unsigned long long *>(f) + ((long long)k * n + c)) : 0ull;
-        unsigned top = 0u;
+        unsigned top = 0u, low = 0xffffffffu;
 #pragma unroll
-        for (int k = 0; k < Q; ++k) top = max(top, (unsigned)(v[k] >> 32) & 0x7ff00000u);
-        const int E = (int)(top >> 20);
-        if (E >= 64 && E < 0x7ff) {
-            if (E != Ecur) {
-                const Sums4 w = to_sums(s[0], s[1], s[2], s[3], Ecur, m, rho0);
-                for (int d = 0; d < 4; ++d) a[d] += w.v[d];
-                for (int d = 0; d < 4; ++d) s[d] = FixedSum{0, 0ull};
-                m = 0;
-                Ecur = E;
-            }
+        for (int k = 0; k < Q; ++k) {
+            const unsigned x = (unsigned)(v[k] >> 32) & 0x7ff00000u;
+            top = max(top, x);
+            low = min(low, x);
+        }
+        if (live && low == 0u) {  // zeros are exact in any unit
+            low = 0xffffffffu;
+#pragma unroll
+            for (int k = 0; k < Q; ++k)
+                if (v[k] << 1) low = min(low, (unsigned)(v[k] >> 32) & 0x7ff00000u);
+        }
+        const int E = (int)(top >> 20), Elow = (int)(low >> 20);
+        bool exact = E >= 64 && E <= Ecur && Elow >= Ecur - kFixedSpan;
+        if (!exact && E >= 64 && E < 0x7ff && Elow >= E - kFixedSpan) {
+            const Sums4 w = to_sums(s[0], s[1], s[2], s[3], Ecur, m, rho0);
+            for (int d = 0; d < 4; ++d) a[d] += w.v[d];
+            for (int d = 0; d < 4; ++d) s[d] = FixedSum{0, 0ull};
+            m = 0;
+            Ecur = E;
+            exact = true;
+        }
+        if (exact) {
             long long x[4] = {0, 0, 0, 0};
 #pragma unroll
             for (int k = 0; k < Q; ++k) {
                 const unsigned hi = (unsigned)(v[k] >> 32), lo = (unsigned)v[k];
-                const unsigned sh = (unsigned)(E + 62 - kFixedTop) - ((hi >> 20) & 0x7ffu);
+                const unsigned sh = (unsigned)(Ecur + 62 - kFixedTop) - ((hi >> 20) & 0x7ffu);
                 const unsigned mh = (__funnelshift_l(lo, hi, 10) & 0x3fffffffu) | 0x40000000u;
                 unsigned long long t = (unsigned long long)mh << 32 | (unsigned long long)(lo << 10);
-                asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(t), "r"(sh));  // 0 from 64 on
+                asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(t), "r"(sh));  // (a zero: sh > 63, t = 0)
                 const long long sg = (long long)v[k] >> 63;
                 const long long q = ((long long)t ^ sg) - sg;
                 x[0] += q;
