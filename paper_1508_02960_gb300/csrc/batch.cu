@@ -30,6 +30,7 @@ lbm_status fail(lbm_status st, const std::string &msg)
 lbm_status cuda_fail(cudaError_t e, const char *what)
 {
     set_error(std::string(what) + ": " + cudaGetErrorString(e));
+    cudaGetLastError();  // reported here: not again by the next launch's check
     return e == cudaErrorMemoryAllocation ? LBM_ERR_NO_MEMORY : LBM_ERR_CUDA;
 }
 
