@@ -552,15 +552,17 @@ lbm_status Batch::rebuild()
         d_status_ = nullptr;
         h_sums_ = nullptr;
         h_status_ = nullptr;
-        capacity_ = std::max(n, 2 * capacity_);
-        CK(dev_alloc(&d_sums_, sizeof(double) * kRedSlots * capacity_));
-        CK(dev_alloc(&d_status_, sizeof(unsigned) * capacity_));
-        CK(cudaMemset(d_status_, 0, sizeof(unsigned) * capacity_));
-        CK(dev_alloc(&d_fscratch_, sizeof(double) * (RED_F + 3) * kFinalSlices * capacity_));
-        CK(dev_alloc(&d_fcount_, sizeof(unsigned) * capacity_));
-        CK(cudaMemset(d_fcount_, 0, sizeof(unsigned) * capacity_));
-        CK(cudaMallocHost(&h_sums_, sizeof(double) * kRedSlots * capacity_));
-        CK(cudaMallocHost(&h_status_, sizeof(unsigned) * capacity_));
+        const int room = std::max(n, 2 * capacity_);
+        capacity_ = 0;  // until all of them are there: after a failure the next call tries again
+        CK(dev_alloc(&d_sums_, sizeof(double) * kRedSlots * room));
+        CK(dev_alloc(&d_status_, sizeof(unsigned) * room));
+        CK(cudaMemset(d_status_, 0, sizeof(unsigned) * room));
+        CK(dev_alloc(&d_fscratch_, sizeof(double) * (RED_F + 3) * kFinalSlices * room));
+        CK(dev_alloc(&d_fcount_, sizeof(unsigned) * room));
+        CK(cudaMemset(d_fcount_, 0, sizeof(unsigned) * room));
+        CK(cudaMallocHost(&h_sums_, sizeof(double) * kRedSlots * room));
+        CK(cudaMallocHost(&h_status_, sizeof(unsigned) * room));
+        capacity_ = room;
     }
     std::vector<InstanceDev> table(std::max(n, 1));
     std::vector<int> tc(std::max(n, 1)), sc(std::max(n, 1));  // tiles of each instance
