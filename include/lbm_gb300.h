@@ -418,7 +418,8 @@ LBM_API lbm_status lbm_server_create(const lbm_server_opts *opts, lbm_server **o
 LBM_API lbm_status lbm_server_submit(lbm_server *s, const lbm_desc *desc, double tol,
                              int64_t max_steps, int64_t *req_id);
 /* LBM_ERR_STATE while the request is queued or running; LBM_OK with the result once it
- * converged; LBM_ERR_NOT_CONVERGED / LBM_ERR_DIVERGED with the last result otherwise.
+ * converged; LBM_ERR_NOT_CONVERGED / LBM_ERR_DIVERGED with the last result otherwise; the
+ * status of a step that failed (LBM_ERR_NO_MEMORY, LBM_ERR_CUDA), with the result before it.
  * latency_s (may be NULL): submit-to-finish wall time. */
 LBM_API lbm_status lbm_server_poll(lbm_server *s, int64_t req_id, lbm_obs *out, double *latency_s);
 /* Block until every submitted request has finished (bounded by timeout_s; <= 0: none). */

@@ -186,14 +186,15 @@ void lbm_server::run()
         TraceRange trace("lbm.server.chunk");
         const auto t0 = Clock::now();
         double updates = 0.0;
+        std::map<GroupKey, lbm_status> stepped;  // a group whose step failed has no new sums to judge by
         for (auto &kv : groups) {
             Batch &b = *kv.second;
             if (b.size() == 0) continue;
-            if (b.step(opts.check_interval) != LBM_OK) continue;
-            updates += (double)b.fluid_cells() * opts.check_interval;
+            stepped[kv.first] = b.step(opts.check_interval);
+            if (stepped[kv.first] == LBM_OK) updates += (double)b.fluid_cells() * opts.check_interval;
         }
         for (auto &kv : groups)
-            if (kv.second->size()) kv.second->fetch_sums();
+            if (kv.second->size() && stepped[kv.first] == LBM_OK) stepped[kv.first] = kv.second->fetch_sums();
         const double dt = std::chrono::duration<double>(Clock::now() - t0).count();
         lk.lock();
         stats.fluid_updates += updates;
@@ -206,7 +207,9 @@ void lbm_server::run()
                 Instance &in = b.at(i);
                 const double U = in.sums[1] / (double)in.geo.ncells;
                 lbm_status st = LBM_ERR_STATE;
+                const lbm_status failed = stepped[kv.first];
                 if (r.cancel) st = LBM_ERR_CANCELLED;
+                else if (failed != LBM_OK) st = failed == LBM_ERR_STATE ? LBM_ERR_CUDA : failed;
                 else if (in.status & STATUS_DIVERGED) st = LBM_ERR_DIVERGED;
                 else if (r.have_U && std::fabs(U - r.U_old) < r.tol * std::fabs(U)) st = LBM_OK;
                 else if (in.steps >= r.max_steps) st = LBM_ERR_NOT_CONVERGED;

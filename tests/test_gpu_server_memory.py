@@ -82,3 +82,21 @@ def test_batch_is_usable_after_a_failed_join(capi):
         if not failed:
             break                          # n allocations suffice: every failure was met
     assert 10 < n < 99
+
+
+def test_resident_point_is_not_judged_by_a_failed_step(capi):
+    """A resident point whose steps fail for want of memory is reported so (or steps on), never as
+    converged on the numbers of the step before."""
+    met = 0
+    for n in range(100):
+        srv = capi.Server(hbm_budget_bytes=1 << 30, check_interval=50, max_resident=4)
+        try:
+            r1, failed = _join_without_memory(capi, srv, n)
+            got = srv.poll(r1)
+            assert got is None or got[0] == capi.ERR_NO_MEMORY, (n, got and got[0])
+            met += got is not None
+        finally:
+            srv.close()
+        if not failed:
+            break
+    assert met > 0
