@@ -265,7 +265,8 @@ LBM_API lbm_status lbm_observables(lbm_ctx *ctx, double K_darcy, lbm_obs *out);
 /* Host-side fault injection for tests (there is no device-side fault injection): after
  * the next n device allocations made by the library succeed, the following ones fail as if
  * the device were out of memory (cudaErrorMemoryAllocation), so that every out-of-memory
- * path can be exercised without touching the GPU's state.  n < 0 (the default) disables it.
+ * path can be exercised without touching the GPU's state.  The recording of a graph of
+ * steps, for which the driver allocates, counts as one.  n < 0 (the default) disables it.
  * Process-wide; not for production use. */
 LBM_API void lbm_debug_fail_alloc_after(int64_t n);
 

@@ -291,6 +291,7 @@ lbm_status Batch::remove(int i)
     CK(cudaStreamSynchronize(stream_));
     inst_.erase(inst_.begin() + i);  // the instance frees its device memory
     dirty_ = true;
+    if (inst_.empty()) split_ = false;
     return LBM_OK;
 }
 
@@ -528,6 +529,7 @@ lbm_status Batch::setup_tma()
 
 lbm_status Batch::rebuild()
 {
+    if (split_) return fail(LBM_ERR_STATE, "a step failed between two groups of the batch's instances: they stand at different steps");
     CK(cudaStreamSynchronize(stream_));
     const int n = size();
     const int CS = block_ / 32;  // segments per work chunk
@@ -796,26 +798,12 @@ long long Batch::state_bytes(const StepGroup &g) const
 // 681 / 655.
 bool Batch::early(const StepGroup &g) const { return state_bytes(g) <= (64ll << 20); }
 
-// The graph of m steps of a group from (flip, aa) in shape sh, the last one reducing when red,
-// instantiated on first use and kept in a small least-recently-used cache.  The only group of a
-// batch has the reduction's set-up and the final sums in its graph, too.
-lbm_status Batch::graph_for(StepGroup &g, long long m, bool red, int flip, int aa, const StepShape &sh, int wx,
-                            cudaGraphExec_t *out)
+// Queue m steps of a group on stream s from (flip, aa) in shape sh, the last one reducing when
+// red.  With the first group of a batch goes the reduction's set-up, with the last one the final
+// sums, for all instances.
+cudaError_t Batch::queue_group(const StepGroup &g, cudaStream_t s, long long m, bool red, int flip, int aa,
+                               const StepShape &sh, int wx)
 {
-    const GraphKey key{m * 2 + (red ? 1 : 0), flip, aa, sh.warps};
-    auto it = g.graphs.find(key);
-    if (it != g.graphs.end()) {
-        it->second.used = ++g.graph_clock;
-        *out = it->second.exec;
-        return LBM_OK;
-    }
-    if (g.graphs.size() >= kGraphCache) {  // evict the least recently used graph
-        auto lru = g.graphs.begin();
-        for (auto c = g.graphs.begin(); c != g.graphs.end(); ++c)
-            if (c->second.used < lru->second.used) lru = c;
-        cudaGraphExecDestroy(lru->second.exec);
-        g.graphs.erase(lru);
-    }
     const StepQueue q{&ops(),
                       shaped_launch(g, kStepWarps),
                       shaped_launch(g, sh.warps),
@@ -827,19 +815,41 @@ lbm_status Batch::graph_for(StepGroup &g, long long m, bool red, int flip, int a
                       tma_ ? &tma_launch_ : nullptr,
                       collision_,
                       layout_};
-    const bool sums = red && groups_.size() == 1;
+    cudaError_t e = queue_steps(q, s, red ? m - 1 : m, false, flip, aa);
+    if (e != cudaSuccess || !red) return e;
+    const int odd = (int)((m - 1) & 1);
+    if (&g == groups_.front().get()) e = cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), s);
+    if (e == cudaSuccess)
+        e = queue_steps(q, s, 1, true, layout_ == LBM_LAYOUT_AB ? flip ^ odd : flip,
+                        layout_ == LBM_LAYOUT_AB ? aa : aa ^ odd);
+    if (e == cudaSuccess && &g == groups_.back().get())
+        e = launch_final_reduce(d_table_, d_stile_count_, size(), d_sums_, d_fscratch_, d_fcount_, s);
+    return e;
+}
+
+// The graph of these steps, instantiated on first use and kept in a small least-recently-used
+// cache.
+lbm_status Batch::graph_for(StepGroup &g, long long m, bool red, int flip, int aa, const StepShape &sh, int wx,
+                            cudaGraphExec_t *out)
+{
+    const GraphKey key{m * 2 + (red ? 1 : 0), flip, aa, sh.warps};
+    auto it = g.graphs.find(key);
+    if (it != g.graphs.end()) {
+        it->second.used = ++g.graph_clock;
+        *out = it->second.exec;
+        return LBM_OK;
+    }
+    if (!may_allocate()) return cuda_fail(cudaErrorMemoryAllocation, "recording of step kernels");
+    if (g.graphs.size() >= kGraphCache) {  // evict the least recently used graph
+        auto lru = g.graphs.begin();
+        for (auto c = g.graphs.begin(); c != g.graphs.end(); ++c)
+            if (c->second.used < lru->second.used) lru = c;
+        cudaGraphExecDestroy(lru->second.exec);
+        g.graphs.erase(lru);
+    }
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = queue_steps(q, cap_, red ? m - 1 : m, false, flip, aa);
-    if (e == cudaSuccess && red) {
-        const int odd = (int)((m - 1) & 1);
-        if (sums) e = cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), cap_);
-        if (e == cudaSuccess)
-            e = queue_steps(q, cap_, 1, true, layout_ == LBM_LAYOUT_AB ? flip ^ odd : flip,
-                            layout_ == LBM_LAYOUT_AB ? aa : aa ^ odd);
-        if (e == cudaSuccess && sums)
-            e = launch_final_reduce(d_table_, d_stile_count_, size(), d_sums_, d_fscratch_, d_fcount_, cap_);
-    }
+    cudaError_t e = queue_group(g, cap_, m, red, flip, aa, sh, wx);
     cudaError_t e2 = cudaStreamEndCapture(cap_, &graph);
     if (e != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
@@ -872,7 +882,7 @@ struct ShapeKey {
 };
 std::mutex g_shape_mu;
 std::map<ShapeKey, StepShape> g_shapes;
-const StepShape kShapeCandidates[] = {{kShapeWarps[0]}, {kShapeWarps[1]}, {kShapeWarps[2]}};
+const StepShape kShapeCandidates[kShapeWarpsN] = {{kShapeWarps[0]}, {kShapeWarps[1]}, {kShapeWarps[2]}};
 constexpr int kTuneSteps = 16;  // steps timed per candidate (even: flip and AA phase return)
 }  // namespace
 
@@ -891,39 +901,36 @@ void Batch::lookup_shape(StepGroup &g)
     }
 }
 
+// Take kTuneSteps steps of a group in each shape, and then the fastest for good.  Nothing is
+// launched unless the steps of all the shapes can be.
 lbm_status Batch::tune_shape(StepGroup &g, int wx)
 {
-    const int nc = (int)(sizeof(kShapeCandidates) / sizeof(kShapeCandidates[0]));
-    cudaEvent_t ev[2];
-    CK(cudaEventCreate(&ev[0]));
-    CK(cudaEventCreate(&ev[1]));
-    double best = 0.0;
+    cudaGraphExec_t exec[kShapeWarpsN] = {};
+    for (int c = 0; c < kShapeWarpsN; ++c) {
+        lbm_status st = graph_for(g, kTuneSteps, false, flip_, aa_phase_, kShapeCandidates[c], wx, &exec[c]);
+        if (st != LBM_OK) return st;
+    }
+    cudaEvent_t ev[2] = {};
+    cudaError_t e = cudaEventCreate(&ev[0]);
+    if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
+    float best = 0.0f;
     StepShape pick = g.shape;
-    lbm_status st = LBM_OK;
-    for (int c = 0; c < nc && st == LBM_OK; ++c) {
-        const StepShape &sh = kShapeCandidates[c];
-        cudaGraphExec_t exec = nullptr;
-        if ((st = graph_for(g, kTuneSteps, false, flip_, aa_phase_, sh, wx, &exec)) != LBM_OK) break;
-        cudaError_t e = cudaEventRecord(ev[0], stream_);
-        if (e == cudaSuccess) e = cudaGraphLaunch(exec, stream_);
+    for (int c = 0; c < kShapeWarpsN && e == cudaSuccess; ++c) {
+        float ms = 0.0f;
+        e = cudaEventRecord(ev[0], stream_);
+        if (e == cudaSuccess && (e = cudaGraphLaunch(exec[c], stream_)) == cudaSuccess) advance(g, kTuneSteps);
         if (e == cudaSuccess) e = cudaEventRecord(ev[1], stream_);
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
-        float ms = 0.0f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
-        if (e != cudaSuccess) {
-            st = cuda_fail(e, "timing of a step shape");
-            break;
-        }
-        launches_ += kTuneSteps;
         g.shape_ms[c] = ms / kTuneSteps;
         if (c == 0 || ms < best) {
             best = ms;
-            pick = sh;
+            pick = kShapeCandidates[c];
         }
     }
-    cudaEventDestroy(ev[0]);
-    cudaEventDestroy(ev[1]);
-    if (st != LBM_OK) return st;
+    for (cudaEvent_t v : ev)
+        if (v) cudaEventDestroy(v);
+    if (e != cudaSuccess) return cuda_fail(e, "timing of a step shape");
     g.shape = pick;
     g.shape_src = 1;
     g.tune = false;
@@ -932,6 +939,50 @@ lbm_status Batch::tune_shape(StepGroup &g, int wx)
     return LBM_OK;
 }
 
+// n steps of a group are queued.
+void Batch::advance(const StepGroup &g, long long n)
+{
+    launches_ += n;
+    for (int i : g.members) {
+        Instance &in = *inst_[i];
+        in.steps += n;
+        in.have_sums = in.have_force = in.sums_pending = false;
+    }
+}
+
+// n steps of a group.  begun: others of the call are queued already, after which a lack of memory
+// for graphs is no reason to fail: the shapes are timed another time and the steps queued one by
+// one.
+lbm_status Batch::step_group(StepGroup &g, long long n, int wx, bool begun)
+{
+    constexpr long long kChunk = 1000;                         // (even)
+    constexpr long long tuning = kShapeWarpsN * kTuneSteps;    // (even)
+    long long left = n;
+    if (g.tune && n > tuning) {  // the first steps time the shapes
+        const long long at = launches_;
+        lbm_status st = tune_shape(g, wx);
+        if (st != LBM_OK && (st != LBM_ERR_NO_MEMORY || !begun)) return st;
+        left -= launches_ - at;
+        begun |= left < n;
+    }
+    while (left > 0) {
+        const long long m = left > 2 * kChunk ? kChunk : left;
+        cudaGraphExec_t exec = nullptr;
+        lbm_status st = graph_for(g, m, m == left, flip_, aa_phase_, g.shape, wx, &exec);
+        if (st == LBM_OK) CK(cudaGraphLaunch(exec, stream_));
+        else if (st != LBM_ERR_NO_MEMORY || !begun) return st;
+        else CK(queue_group(g, stream_, m, m == left, flip_, aa_phase_, g.shape, wx));
+        advance(g, m);
+        begun = true;
+        left -= m;
+    }
+    return LBM_OK;
+}
+
+// Each group takes all the steps before the next; its graphs are recorded while the one before
+// steps.  The instances share one phase (flip_, aa_phase_), so a call is refused before its first
+// launch or goes through (step_group); if a launch itself fails behind another group's of an odd
+// number of steps (split_), further calls are refused.
 lbm_status Batch::step(long long n)
 {
     TraceRange trace("lbm.step");
@@ -943,45 +994,17 @@ lbm_status Batch::step(long long n)
     }
     int wx = 0;
     for (auto &p : inst_) wx |= p->desc.wall >= LBM_LIBB;
-    const int nc = (int)(sizeof(kShapeCandidates) / sizeof(kShapeCandidates[0]));
-    const bool several = groups_.size() > 1;
-    if (several) CK(cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), stream_));
-    int flip = flip_, aa = aa_phase_;
-    for (auto &g : groups_) {  // each group takes all the steps
-        long long left = n;
-        if (g->tune && n > (long long)nc * kTuneSteps) {  // the first steps time the shapes
-            lbm_status st = tune_shape(*g, wx);
-            if (st != LBM_OK) return st;
-            left -= (long long)nc * kTuneSteps;
-        }
-        flip = flip_;
-        aa = aa_phase_;
-        const long long kChunk = 1000;
-        while (left > 0) {
-            const long long m = left > 2 * kChunk ? kChunk : left;
-            const bool red = (m == left);
-            cudaGraphExec_t exec = nullptr;
-            lbm_status st = graph_for(*g, m, red, flip, aa, g->shape, wx, &exec);
-            if (st != LBM_OK) return st;
-            CK(cudaGraphLaunch(exec, stream_));
-            launches_ += m + (red && !several ? 1 : 0);
-            if (layout_ == LBM_LAYOUT_AB) flip ^= (int)(m & 1);
-            else aa ^= (int)(m & 1);
-            left -= m;
+    const long long before = launches_;
+    for (auto &g : groups_) {
+        lbm_status st = step_group(*g, n, wx, launches_ != before);
+        if (st != LBM_OK) {
+            if (groups_.size() > 1 && launches_ != before && (n & 1)) split_ = dirty_ = true;
+            return st;
         }
     }
-    flip_ = flip;
-    aa_phase_ = aa;
-    if (several) {
-        CK(launch_final_reduce(d_table_, d_stile_count_, size(), d_sums_, d_fscratch_, d_fcount_, stream_));
-        ++launches_;
-    }
-    for (auto &p : inst_) {
-        p->steps += n;
-        p->have_sums = false;
-        p->have_force = false;
-        p->sums_pending = true;
-    }
+    ++launches_;  // the final sums
+    (layout_ == LBM_LAYOUT_AB ? flip_ : aa_phase_) ^= (int)(n & 1);
+    for (auto &p : inst_) p->sums_pending = true;
     return LBM_OK;
 }
 

@@ -148,6 +148,10 @@ private:
                          cudaGraphExec_t *out);
     void lookup_shape(StepGroup &g);              // the cached shape of this group, or tuning pending
     lbm_status tune_shape(StepGroup &g, int wx);  // time every candidate shape on the live state
+    lbm_status step_group(StepGroup &g, long long n, int wx, bool begun);
+    cudaError_t queue_group(const StepGroup &g, cudaStream_t s, long long m, bool red, int flip, int aa,
+                            const StepShape &sh, int wx);
+    void advance(const StepGroup &g, long long n);
     lbm_status build_groups(const std::vector<InstanceDev> &table);
     lbm_status rebuild();          // upload table and tiles, drop graphs
     lbm_status aa_restart(int i);  // instance i (i < 0: all) set from outside: AA arrangement of step 0
@@ -181,6 +185,7 @@ private:
     int flip_ = 0;
     int aa_phase_ = 0;
     bool dirty_ = true;
+    bool split_ = false;               // a launch failed between two groups
     long long launches_ = 0;
     int sms_ = 0;
     double *d_stage_ = nullptr;       // FP64 staging of the wall distances (one direction)

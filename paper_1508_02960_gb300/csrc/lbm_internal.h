@@ -14,7 +14,9 @@
 namespace lbm {
 
 // Every device buffer the library owns is allocated here, so that the fault injection of
-// lbm_debug_fail_alloc_after reaches every out-of-memory path.
+// lbm_debug_fail_alloc_after reaches every out-of-memory path; what makes the driver allocate
+// asks may_allocate first.
+bool may_allocate();
 cudaError_t dev_alloc(void **p, size_t bytes);
 template <typename T> cudaError_t dev_alloc(T **p, size_t bytes)
 {

@@ -14,15 +14,21 @@ std::atomic<long long> g_alloc_budget{-1};
 
 void set_alloc_budget(long long n) { g_alloc_budget.store(n < 0 ? -1 : n); }
 
-cudaError_t dev_alloc(void **p, size_t bytes)
+bool may_allocate()
 {
     long long b = g_alloc_budget.load();
     while (b >= 0) {
-        if (b == 0) {
-            *p = nullptr;
-            return cudaErrorMemoryAllocation;
-        }
+        if (b == 0) return false;
         if (g_alloc_budget.compare_exchange_weak(b, b - 1)) break;
+    }
+    return true;
+}
+
+cudaError_t dev_alloc(void **p, size_t bytes)
+{
+    if (!may_allocate()) {
+        *p = nullptr;
+        return cudaErrorMemoryAllocation;
     }
     return cudaMalloc(p, bytes);
 }
