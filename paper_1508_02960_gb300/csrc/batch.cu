@@ -227,6 +227,7 @@ StepGroup::~StepGroup()
 Batch::~Batch()
 {
     if (stream_ || cap_) cudaStreamSynchronize(stream_);
+    whole_.reset();
     groups_.clear();
     inst_.clear();
     cudaFree(d_table_);
@@ -613,13 +614,22 @@ lbm_status Batch::rebuild()
 // Per step of the whole batch, one launch for all -> in groups: the first 16 sweep points, FP16
 // A-B, 425 -> 366 us; 12 points, FP16 AA, 315 -> 255; 10 points, FP32 AA, 181 -> 145; 4 cells of
 // 128^3, FP32 AA, 144 -> 112; 64 cells of 48^3, FP32 AA, 150 -> 125 (two groups).  kAlone: 6
-// cells of 80^3 (290,000 fluid cells) are faster together (FP32 AA 46 us, alone 53), of 96^3
-// (560,000) alone (79, together 108).
+// cells of 80^3 (375,000 fluid cells) are faster together or equal (FP32 AA 50.5 us, alone 53.0;
+// FP16 AA 54.1 / 56.5, A-B 57.3 / 57.0; BF16 AA 51.5 / 54.4, A-B 55.4 / 55.0), of 96^3 (648,000)
+// alone (FP32 AA together 82.2, alone 77.8; FP16 AA 90.1 / 84.8, A-B 89.8 / 86.4; BF16 AA 85.7 /
+// 81.1, A-B 86.8 / 83.0).
+// A call of at most kTogether steps finds little of a group's state in L2 and pays for every
+// group's first and last step, so it steps all instances in one launch.  Per call of one step,
+// groups -> together: 64 cells of 48^3, FP32 A-B, 433 -> 291 us; 6 of 80^3, FP32 AA, 148 -> 122; 6
+// of 96^3, FP16 A-B, 250 -> 200.  Of five steps: 1118 -> 1035, 367 -> 367, 614 -> 602 (6 of 96^3,
+// FP32 AA, 596 -> 619); of six, groups are faster or equal but for FP16 and BF16 cells that share
+// groups (64 of 48^3, A-B, 1 % slower).
 lbm_status Batch::build_groups(const std::vector<InstanceDev> &table)
 {
     constexpr long long kAlone = 400000;
     constexpr long long kGroupBytes = 64ll << 20;
     groups_.clear();
+    whole_.reset();
     std::vector<int> small;
     long long small_cells = 0;
     auto open = [&](std::vector<int> members) {
@@ -645,44 +655,69 @@ lbm_status Batch::build_groups(const std::vector<InstanceDev> &table)
     }
     for (auto &m : shared)
         if (!m.empty()) open(std::move(m));
-    for (auto &gp : groups_) {
-        StepGroup &g = *gp;
-        const int n = (int)g.members.size();
-        std::vector<TileDev> tiles[kShapeWarpsN];
-        long long total[kShapeWarpsN] = {};
-        for (int r = 0; r < n; ++r) {
-            const Instance &in = *inst_[g.members[r]];
-            g.h_table.push_back(table[g.members[r]]);
-            g.fluid += in.geo.n_fluid;
-            for (int w = 0; w < kShapeWarpsN; ++w) {
-                const int W = kShapeWarps[w];
-                // at least one tile (an instance without fluid has one of padding)
-                const long long nw = std::max(1ll, (in.geo.n_fwarps + W - 1) / W);
-                if (nw * W > in.geo.n_fwarps_padded) return fail(LBM_ERR_STATE, "fluid work list too short");
-                if (total[w] + nw > INT32_MAX) return fail(LBM_ERR_ARG, "too many tiles");
-                if (n >= 2 && n <= kBatchMapMax) {
-                    g.maps[w].tile_start[r] = (int)total[w];
-                    g.maps[w].flane[r] = in.geo.flane;
-                    g.maps[w].fwarp[r] = in.geo.fwarp;
-                } else if (n > kBatchMapMax) {
-                    for (long long t = 0; t < nw; ++t)
-                        tiles[w].push_back(TileDev{r, (int)t, t * W, in.geo.flane, in.geo.fwarp});
-                }
-                total[w] += nw;
-            }
-        }
+    for (auto &g : groups_) {
+        for (int i : g->members) g->h_table.push_back(table[i]);
+        lbm_status st = fill_group(*g);
+        if (st != LBM_OK) return st;
+    }
+    return LBM_OK;
+}
+
+// All instances as one group, for the short calls of a batch of several groups.
+lbm_status Batch::whole_group(StepGroup **out)
+{
+    if (!whole_) {
+        std::unique_ptr<StepGroup> g(new StepGroup());
+        g->h_table.resize((size_t)size());
+        for (auto &p : groups_)
+            for (size_t r = 0; r < p->members.size(); ++r) g->h_table[(size_t)p->members[r]] = p->h_table[r];
+        for (int i = 0; i < size(); ++i) g->members.push_back(i);
+        lbm_status st = fill_group(*g);
+        if (st != LBM_OK) return st;
+        lookup_shape(*g);
+        whole_ = std::move(g);
+    }
+    *out = whole_.get();
+    return LBM_OK;
+}
+
+// The step tiles and the parameters of a group whose members and h_table are set.
+lbm_status Batch::fill_group(StepGroup &g)
+{
+    const int n = (int)g.members.size();
+    std::vector<TileDev> tiles[kShapeWarpsN];
+    long long total[kShapeWarpsN] = {};
+    for (int r = 0; r < n; ++r) {
+        const Instance &in = *inst_[g.members[r]];
+        g.fluid += in.geo.n_fluid;
         for (int w = 0; w < kShapeWarpsN; ++w) {
-            g.ntiles[w] = (int)total[w];
-            g.maps[w].n = n >= 2 && n <= kBatchMapMax ? n : 0;
-            if (g.maps[w].n) g.maps[w].tile_start[n] = (int)total[w];
-            if (tiles[w].empty()) continue;
-            CK(dev_alloc(&g.d_tiles[w], sizeof(TileDev) * tiles[w].size()));
-            CK(cudaMemcpy(g.d_tiles[w], tiles[w].data(), sizeof(TileDev) * tiles[w].size(), cudaMemcpyHostToDevice));
+            const int W = kShapeWarps[w];
+            // at least one tile (an instance without fluid has one of padding)
+            const long long nw = std::max(1ll, (in.geo.n_fwarps + W - 1) / W);
+            if (nw * W > in.geo.n_fwarps_padded) return fail(LBM_ERR_STATE, "fluid work list too short");
+            if (total[w] + nw > INT32_MAX) return fail(LBM_ERR_ARG, "too many tiles");
+            if (n >= 2 && n <= kBatchMapMax) {
+                g.maps[w].tile_start[r] = (int)total[w];
+                g.maps[w].flane[r] = in.geo.flane;
+                g.maps[w].fwarp[r] = in.geo.fwarp;
+            } else if (n > kBatchMapMax) {
+                for (long long t = 0; t < nw; ++t)
+                    tiles[w].push_back(TileDev{r, (int)t, t * W, in.geo.flane, in.geo.fwarp});
+            }
+            total[w] += nw;
         }
-        if (n > 1) {
-            CK(dev_alloc(&g.d_table, sizeof(InstanceDev) * n));
-            CK(cudaMemcpy(g.d_table, g.h_table.data(), sizeof(InstanceDev) * n, cudaMemcpyHostToDevice));
-        }
+    }
+    for (int w = 0; w < kShapeWarpsN; ++w) {
+        g.ntiles[w] = (int)total[w];
+        g.maps[w].n = n >= 2 && n <= kBatchMapMax ? n : 0;
+        if (g.maps[w].n) g.maps[w].tile_start[n] = (int)total[w];
+        if (tiles[w].empty()) continue;
+        CK(dev_alloc(&g.d_tiles[w], sizeof(TileDev) * tiles[w].size()));
+        CK(cudaMemcpy(g.d_tiles[w], tiles[w].data(), sizeof(TileDev) * tiles[w].size(), cudaMemcpyHostToDevice));
+    }
+    if (n > 1) {
+        CK(dev_alloc(&g.d_table, sizeof(InstanceDev) * n));
+        CK(cudaMemcpy(g.d_table, g.h_table.data(), sizeof(InstanceDev) * n, cudaMemcpyHostToDevice));
     }
     return LBM_OK;
 }
@@ -799,7 +834,7 @@ long long Batch::state_bytes(const StepGroup &g) const
 bool Batch::early(const StepGroup &g) const { return state_bytes(g) <= (64ll << 20); }
 
 // Queue m steps of a group on stream s from (flip, aa) in shape sh, the last one reducing when
-// red.  With the first group of a batch goes the reduction's set-up, with the last one the final
+// red.  With the first group of a call goes the reduction's set-up, with the last one the final
 // sums, for all instances.
 cudaError_t Batch::queue_group(const StepGroup &g, cudaStream_t s, long long m, bool red, int flip, int aa,
                                const StepShape &sh, int wx)
@@ -818,11 +853,11 @@ cudaError_t Batch::queue_group(const StepGroup &g, cudaStream_t s, long long m, 
     cudaError_t e = queue_steps(q, s, red ? m - 1 : m, false, flip, aa);
     if (e != cudaSuccess || !red) return e;
     const int odd = (int)((m - 1) & 1);
-    if (&g == groups_.front().get()) e = cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), s);
+    if (&g == whole_.get() || &g == groups_.front().get()) e = cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), s);
     if (e == cudaSuccess)
         e = queue_steps(q, s, 1, true, layout_ == LBM_LAYOUT_AB ? flip ^ odd : flip,
                         layout_ == LBM_LAYOUT_AB ? aa : aa ^ odd);
-    if (e == cudaSuccess && &g == groups_.back().get())
+    if (e == cudaSuccess && (&g == whole_.get() || &g == groups_.back().get()))
         e = launch_final_reduce(d_table_, d_stile_count_, size(), d_sums_, d_fscratch_, d_fcount_, s);
     return e;
 }
@@ -979,10 +1014,11 @@ lbm_status Batch::step_group(StepGroup &g, long long n, int wx, bool begun)
     return LBM_OK;
 }
 
-// Each group takes all the steps before the next; its graphs are recorded while the one before
-// steps.  The instances share one phase (flip_, aa_phase_), so a call is refused before its first
-// launch or goes through (step_group); if a launch itself fails behind another group's of an odd
-// number of steps (split_), further calls are refused.
+// Each group (in a short call all instances as one: build_groups) takes all the steps before the
+// next; its graphs are recorded while the one before steps.  The instances share one phase (flip_,
+// aa_phase_), so a call is refused before its first launch or goes through (step_group); if a
+// launch itself fails behind another group's of an odd number of steps (split_), further calls are
+// refused.
 lbm_status Batch::step(long long n)
 {
     TraceRange trace("lbm.step");
@@ -994,11 +1030,18 @@ lbm_status Batch::step(long long n)
     }
     int wx = 0;
     for (auto &p : inst_) wx |= p->desc.wall >= LBM_LIBB;
+    std::vector<StepGroup *> groups;
+    if (groups_.size() > 1 && n <= kTogether) {
+        lbm_status st = whole_group(&groups.emplace_back());
+        if (st != LBM_OK) return st;
+    } else {
+        for (auto &g : groups_) groups.push_back(g.get());
+    }
     const long long before = launches_;
-    for (auto &g : groups_) {
+    for (StepGroup *g : groups) {
         lbm_status st = step_group(*g, n, wx, launches_ != before);
         if (st != LBM_OK) {
-            if (groups_.size() > 1 && launches_ != before && (n & 1)) split_ = dirty_ = true;
+            if (groups.size() > 1 && launches_ != before && (n & 1)) split_ = dirty_ = true;
             return st;
         }
     }

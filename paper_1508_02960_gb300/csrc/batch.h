@@ -153,6 +153,8 @@ private:
                             const StepShape &sh, int wx);
     void advance(const StepGroup &g, long long n);
     lbm_status build_groups(const std::vector<InstanceDev> &table);
+    lbm_status fill_group(StepGroup &g);
+    lbm_status whole_group(StepGroup **out);
     lbm_status rebuild();          // upload table and tiles, drop graphs
     lbm_status aa_restart(int i);  // instance i (i < 0: all) set from outside: AA arrangement of step 0
     int cur_of(const Instance &in) const { return in.phase ^ flip_; }
@@ -167,7 +169,9 @@ private:
     InstanceDev *d_table_ = nullptr;
     int *d_tile_count_ = nullptr;     // chunks of the active-segment lists (state kernels), per instance
     int *d_stile_count_ = nullptr;    // tiles of the fluid-warp lists (step kernels), per instance
+    static constexpr long long kTogether = 5;  // steps of a call that takes no groups
     std::vector<std::unique_ptr<StepGroup>> groups_;
+    std::unique_ptr<StepGroup> whole_;  // all instances, once a short call was made (several groups)
     double *d_sums_ = nullptr;        // [n][kRedSlots]
     unsigned *d_status_ = nullptr;    // [n]
     double *h_sums_ = nullptr;        // pinned [n][kRedSlots]
