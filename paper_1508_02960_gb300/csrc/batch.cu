@@ -618,6 +618,9 @@ lbm_status Batch::rebuild()
 // FP16 AA 54.1 / 56.5, A-B 57.3 / 57.0; BF16 AA 51.5 / 54.4, A-B 55.4 / 55.0), of 96^3 (648,000)
 // alone (FP32 AA together 82.2, alone 77.8; FP16 AA 90.1 / 84.8, A-B 89.8 / 86.4; BF16 AA 85.7 /
 // 81.1, A-B 86.8 / 83.0).
+// FP64 instances stay together: their steps are bound by the FP64 pipe, not by L2, and every group
+// leaves multiprocessors idle at its end (40 steps a call, in groups -> one launch for all: 6 cells
+// of 64^3, A-B, 293 -> 268 us a step, of 80^3 561 -> 512, of 96^3 933 -> 873, in place 933 -> 873).
 // A call of at most kTogether steps finds little of a group's state in L2 and pays for every
 // group's first and last step, so it steps all instances in one launch.  Per call of one step,
 // groups -> together: 64 cells of 48^3, FP32 A-B, 433 -> 291 us; 6 of 80^3, FP32 AA, 148 -> 122; 6
@@ -628,6 +631,7 @@ lbm_status Batch::build_groups(const std::vector<InstanceDev> &table)
 {
     constexpr long long kAlone = 400000;
     constexpr long long kGroupBytes = 64ll << 20;
+    const bool fp64 = storage_ == LBM_F64;
     groups_.clear();
     whole_.reset();
     std::vector<int> small;
@@ -638,7 +642,7 @@ lbm_status Batch::build_groups(const std::vector<InstanceDev> &table)
     };
     for (int i = 0; i < size(); ++i) {
         const long long f = inst_[i]->geo.n_fluid;
-        if (size() == 1 || f >= kAlone) {
+        if (size() == 1 || (!fp64 && f >= kAlone)) {
             open({i});
         } else {
             small.push_back(i);
@@ -646,7 +650,7 @@ lbm_status Batch::build_groups(const std::vector<InstanceDev> &table)
         }
     }
     const long long cell_bytes = Q * (long long)storage_bytes(storage_) * (layout_ == LBM_LAYOUT_AB ? 2 : 1);
-    const long long parts = std::max(1ll, (small_cells * cell_bytes + kGroupBytes - 1) / kGroupBytes);
+    const long long parts = fp64 ? 1 : std::max(1ll, (small_cells * cell_bytes + kGroupBytes - 1) / kGroupBytes);
     std::vector<std::vector<int>> shared((size_t)parts);
     long long before = 0;
     for (int i : small) {

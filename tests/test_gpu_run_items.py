@@ -5,7 +5,7 @@ an x face.
 
 Against the oracle, and bit for bit against steps that read the entries: the FP64 state of
 about 290,000 fluid cells is above the limit in the A-B layout and below it in place, where the
-two layouts agree; in a batch, two such in-place instances that step together are above it."""
+two layouts agree; in a batch, in-place instances that step together are above it."""
 import numpy as np
 import pytest
 
@@ -84,8 +84,7 @@ def test_made_entries_of_a_group(capi, orc, nx):
     for i, f in enumerate(states):
         b.set_populations(i, f)
     nf = b.info()["n_fluid"]
-    # two groups for three equal instances, so that one of the groups is two of them
-    assert LIMIT < nf * 19 * 8 <= 2 * LIMIT and nf / 3 * 19 * 8 <= LIMIT < nf / 3 * 2 * 19 * 8
+    assert nf / 3 * 19 * 8 <= LIMIT < nf / 3 * 2 * 19 * 8
     for n in (5, 2):
         b.step(n)
     got = [b.get_populations(i) for i in range(3)]

@@ -42,3 +42,28 @@ def test_short_and_long_calls(layout, geoms):
             o = ctx.observables()
         for k in ("U_sup", "mass", "F_x", "F_y", "F_z", "K", "steps", "n_fluid"):
             assert o[k] == got[i][1][k], k
+
+
+def test_fp64_instances_step_together():
+    """FP64 instances, whatever their size, share every launch."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1508_02960_gb300 import capi
+    geoms = [I.centred_sphere(80, 12.0), I.centred_sphere(24, 7.0), I.centred_sphere(76, 11.0)]
+    keep = [capi.make_desc(spheres=g.spheres, shape=g.shape, tau=0.6 + 0.01 * i, delta_rho=1e-4, collision=capi.TRT,
+                           wall=capi.CLI, storage=capi.F64) for i, g in enumerate(geoms)]
+    b = capi.Batch([d for d, _ in keep])
+    b.init_equilibrium()
+    for n in (60, 7):
+        before = b.info()["kernel_launches"]
+        b.step(n)
+        assert b.info()["kernel_launches"] - before == n + 1
+    got = [b.get_populations(i) for i in range(3)]
+    b.close()
+    for (d, _), f in zip(keep, got):
+        with capi.Context(desc=d) as ctx:
+            ctx.init_equilibrium()
+            for n in (60, 7):
+                ctx.step(n)
+            assert np.array_equal(ctx.get_populations(), f)
