@@ -76,10 +76,11 @@ __device__ __noinline__ Sums4 to_sums(FixedSum s0, FixedSum s1, FixedSum s2, Fix
 // because FP64 arithmetic is slow on GB300 (a warp instruction per 19 cycles a multiprocessor):
 // the 49 FP64 additions of a cell would take four times as long as its loads.  The 360 integer
 // instructions they become, by 16 warps a multiprocessor (a cell's 19 values are held until
-// their exponents are known), leave it at 1.75 times the sectors it reads: 160^3 cells, 43 % of
-// them solid at random, 1044 us with FP64 sums in 125 blocks of fixed size -> 165 us,
-// and 255 when the largest population crosses a power of two from cell to cell (rho0 = 0.75, 1.5,
-// 3: lanes change their unit).  Cells that are not exact in integers (values of very different
+// their exponents are known), leave it at 1.7 times the sectors it reads: 160^3 cells, 43 % of
+// them solid at random, 1044 us with FP64 sums in 125 blocks of fixed size -> 155 us (164 with a
+// cell's flag loaded before its values and not a round ahead), and 250 when the largest
+// population crosses a power of two from cell to cell (rho0 = 0.75, 1.5, 3: lanes change their
+// unit).  Cells that are not exact in integers (values of very different
 // sizes, infinities, NaN, a largest value below 2^-959) are summed in FP64: 770 us for a field
 // with such cells among the others of every warp.
 __global__ void __launch_bounds__(kNoAllocThreads, 2) noalloc_partials_kernel(const double *__restrict__ f,
@@ -98,13 +99,16 @@ __global__ void __launch_bounds__(kNoAllocThreads, 2) noalloc_partials_kernel(co
     FixedSum s[4] = {};
     unsigned m = 0;
     int Ecur = 0;  // exponent field of s (0: none yet)
+    auto fluid = [&](long long c) { return c < c1 && !(solid && solid[c]); };
+    bool next = fluid(c0 + warp * 32 + lane);
     for (long long cw = c0 + warp * 32; cw < c1; cw += kNoAllocThreads) {
         const long long c = cw + lane;
-        const bool live = c < c1 && !(solid && solid[c]);
+        const bool live = next;
         unsigned long long v[Q];
 #pragma unroll
         for (int k = 0; k < Q; ++k)
             v[k] = live ? __ldg(reinterpret_cast<const unsigned long long *>(f) + ((long long)k * n + c)) : 0ull;
+        next = fluid(c + kNoAllocThreads);  // before the loads are waited for
         unsigned top = 0u, low = 0xffffffffu;
 #pragma unroll
         for (int k = 0; k < Q; ++k) {
