@@ -530,7 +530,7 @@ lbm_status Batch::setup_tma()
 
 lbm_status Batch::rebuild()
 {
-    if (split_) return fail(LBM_ERR_STATE, "a step failed between two groups of the batch's instances: they stand at different steps");
+    if (split_) return fail(LBM_ERR_STATE, "a launch failed in an earlier step: the instances stand at different steps");
     CK(cudaStreamSynchronize(stream_));
     const int n = size();
     const int CS = block_ / 32;  // segments per work chunk
@@ -857,11 +857,12 @@ cudaError_t Batch::queue_group(const StepGroup &g, cudaStream_t s, long long m, 
     cudaError_t e = queue_steps(q, s, red ? m - 1 : m, false, flip, aa);
     if (e != cudaSuccess || !red) return e;
     const int odd = (int)((m - 1) & 1);
-    if (&g == whole_.get() || &g == groups_.front().get()) e = cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), s);
+    const bool all = &g == whole_.get(), first = all || &g == groups_.front().get(), last = all || &g == groups_.back().get();
+    if (first) e = cudaMemsetAsync(d_status_, 0, sizeof(unsigned) * size(), s);
     if (e == cudaSuccess)
         e = queue_steps(q, s, 1, true, layout_ == LBM_LAYOUT_AB ? flip ^ odd : flip,
                         layout_ == LBM_LAYOUT_AB ? aa : aa ^ odd);
-    if (e == cudaSuccess && (&g == whole_.get() || &g == groups_.back().get()))
+    if (e == cudaSuccess && last)
         e = launch_final_reduce(d_table_, d_stile_count_, size(), d_sums_, d_fscratch_, d_fcount_, s);
     return e;
 }
@@ -1008,9 +1009,13 @@ lbm_status Batch::step_group(StepGroup &g, long long n, int wx, bool begun)
         const long long m = left > 2 * kChunk ? kChunk : left;
         cudaGraphExec_t exec = nullptr;
         lbm_status st = graph_for(g, m, m == left, flip_, aa_phase_, g.shape, wx, &exec);
-        if (st == LBM_OK) CK(cudaGraphLaunch(exec, stream_));
-        else if (st != LBM_ERR_NO_MEMORY || !begun) return st;
-        else CK(queue_group(g, stream_, m, m == left, flip_, aa_phase_, g.shape, wx));
+        if (st != LBM_OK && (st != LBM_ERR_NO_MEMORY || !begun)) return st;
+        const cudaError_t e = st == LBM_OK ? cudaGraphLaunch(exec, stream_)
+                                           : queue_group(g, stream_, m, m == left, flip_, aa_phase_, g.shape, wx);
+        if (e != cudaSuccess) {
+            if (st != LBM_OK) split_ = dirty_ = true;  // some of the m steps may be queued
+            return cuda_fail(e, "launch of steps");
+        }
         advance(g, m);
         begun = true;
         left -= m;
@@ -1020,9 +1025,9 @@ lbm_status Batch::step_group(StepGroup &g, long long n, int wx, bool begun)
 
 // Each group (in a short call all instances as one: build_groups) takes all the steps before the
 // next; its graphs are recorded while the one before steps.  The instances share one phase (flip_,
-// aa_phase_), so a call is refused before its first launch or goes through (step_group); if a
-// launch itself fails behind another group's of an odd number of steps (split_), further calls are
-// refused.
+// aa_phase_), so a call is refused before its first launch or goes through (step_group).  If a
+// launch itself fails behind another group's of an odd number of steps, or amid steps queued one by
+// one, further calls are refused (split_).
 lbm_status Batch::step(long long n)
 {
     TraceRange trace("lbm.step");
