@@ -379,8 +379,9 @@ LBM_API double lbm_delta_rho_for_re_p(double re_p, double tau, double d_p, int32
                               double C_F, double rho0);
 
 /* ---------------------------------------------------------------------------------
- * Batched sweep: many independent periodic cells advanced together by one persistent
- * kernel launch per step (all instances must share collision, storage; layout A-B).
+ * Batched sweep: many independent periodic cells advanced together (all instances must
+ * share collision, storage and layout), in groups that each take all the steps of a call.  A
+ * call that fails before its first launch leaves every instance as it was.
  * ------------------------------------------------------------------------------- */
 LBM_API lbm_status lbm_batch_create(const lbm_desc *descs, int32_t n, void *cuda_stream,
                             lbm_batch **out);

@@ -921,9 +921,10 @@ __device__ __forceinline__ WarpItem locate_item(const InstanceDev &I, const Item
 }
 
 // Issue the 19 pulls of a located work item into raw[] (storage type, converted in
-// finish_item).  Unconditional: solid sources hold 0.  Warps whose cells are all away from
-// the y and z faces index through precomputed offsets (cell + pull_off[k], with a fix-up on
-// the first and last cell of a row); the others through their periodic neighbours.
+// finish_item).  Unconditional: the slot of a solid source holds the wall's part (see above).
+// Warps whose cells are all away from the y and z faces index through precomputed offsets (cell +
+// pull_off[k], with a fix-up on the first and last cell of a row); the others through their
+// periodic neighbours.
 template <int STORE, int KIND, typename R>
 __device__ __forceinline__ void pull_item(const InstanceDev &I, const Par<R> &P, const typename Store<STORE>::T *fs,
                                           const WarpItem &it, typename Store<STORE>::T (&raw)[Q])
